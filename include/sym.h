@@ -71,7 +71,9 @@ extern "C" {
                                   (no lookahead overlap; results are identical either way) */
 #define SYM_FLAG_NO_TENSOR_CORES 8u /* SYM_PREC_MIXED: external updates in FP32 on the SIMT
                                        pipes instead of tcgen05 TF32 splits (x = hi + lo, all four
-                                       partial products accumulated in FP32) */
+                                       partial products accumulated in FP32). SYM_PREC_FP64: updates
+                                       on the FP64 pipe instead of exact products of 8-bit digits
+                                       on the FP16 tensor cores (56-bit fixed point, 64-bit sums) */
 #define SYM_FLAG_NO_FUSED_LEVELS 16u /* run the launches of levels of narrow supernodes apart
                                         instead of as one fused launch per level and phase
                                         (SYM_EXPORT_BATCH_PANEL, _FWD_PANEL, _BWD_PANEL), for

@@ -32,6 +32,9 @@ struct sym_handle_s {
   long long *d_status = nullptr;
   long long *h_status = nullptr;  // pinned: [0] holds the reset value, [1] receives the status
   double *d_y = nullptr;          // solve work array
+  uint4 *d_dg = nullptr;          // digits of the FP64 panels (one matrix, tensor cores)
+  int32_t *d_exps = nullptr;      // their row scale exponents
+  bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
   double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix)
   int64_t y_cap = 0;
@@ -161,7 +164,7 @@ void release_device(sym_handle_s *h) {
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   {
     void *mp[] = {h->d_Linv, h->d_Lfinv, h->d_Lf, h->d_Axc, h->d_anorm, h->d_anorm_work, h->d_csr_p, h->d_csr_i,
-                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo};
+                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps};
     for (void *p : mp)
       if (p) cudaFree(p);
     if (h->h_eta) cudaFreeHost(h->h_eta);
@@ -352,6 +355,24 @@ int ensure_stage(sym_handle_s *h, int64_t count) {
   return SYM_OK;
 }
 
+// Digit storage of one FP64 matrix's factor on the tensor cores, at the first factorization of a
+// single matrix. Without the memory the SIMT kernels run.
+void ensure_digits(sym_handle_s *h) {
+  if (h->dg_tried || h->precision != SYM_PREC_FP64 || !h->dp.tensor_cores || h->plan.dg_size == 0) return;
+  h->dg_tried = true;
+  const size_t db = sizeof(uint4) * (size_t)h->plan.dg_size, eb = sizeof(int32_t) * (size_t)h->plan.n;
+  if (cudaMalloc(&h->d_dg, db) == cudaSuccess && cudaMalloc(&h->d_exps, eb) == cudaSuccess) {
+    h->device_bytes += (int64_t)(db + eb);
+  } else {
+    cudaGetLastError();
+    if (h->d_dg) cudaFree(h->d_dg);
+    h->d_dg = nullptr;
+    h->d_exps = nullptr;
+  }
+  h->dp.dg = h->d_dg;
+  h->dp.exps = h->d_exps;
+}
+
 int check_device(sym_handle_s *h) {
   if (!h) return fail(SYM_ERR_INVALID, "null handle");
   if (h->host_only) return fail(SYM_ERR_STATE, "handle was analyzed with SYM_FLAG_HOST_ONLY");
@@ -517,6 +538,11 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(diagonal inverses)");
       else bytes += sizeof(float) * P.dinv_storage;
     }
+    if (!rc) {
+      std::vector<int64_t> dpos(P.n);
+      for (int64_t k = 0; k < P.n; ++k) dpos[k] = Ap[P.perm[k]];  // the diagonal leads each column
+      rc = upload(dpos, &h->d_dpos, bytes);
+    }
     if (!rc && h->precision == SYM_PREC_MIXED) {
       e = cudaMalloc(&h->d_Lf, sizeof(float) * (P.storage() > 0 ? P.storage() : 1));
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(L)");
@@ -542,11 +568,6 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
         if (e != cudaSuccess) rc = cuda_fail(e, "cudaMallocHost(refinement)");
       }
       if (!rc) rc = ensure_rwork(h, sym::refine_work_doubles(P.n, 1));
-      if (!rc) {
-        std::vector<int64_t> dpos(P.n);
-        for (int64_t k = 0; k < P.n; ++k) dpos[k] = Ap[P.perm[k]];  // the diagonal leads each column
-        rc = upload(dpos, &h->d_dpos, bytes);
-      }
       if (!rc) {
         e = cudaMalloc(&h->d_piv, sizeof(double) * (P.n > 0 ? P.n : 1));
         if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(pivots)");
@@ -592,6 +613,7 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
     h->dp.storage = P.storage();
     h->dp.tensor_cores = (opt.flags & SYM_FLAG_NO_TENSOR_CORES) == 0;
     h->dp.piv = h->d_piv;
+    h->dp.oz = h->plan.oz.data();
     for (int c = 0; c < 2; ++c) h->dp.variant[c] = h->plan.variant[c].data();
     h->dp.batch_warp = h->plan.batch_warp.data();
     h->dp.batch_lanes = h->plan.batch_lanes.data();
@@ -630,6 +652,7 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
   if (rc) return rc;
   h->factored = false;
   h->nbatch = nbatch;
+  if (nbatch == 1) ensure_digits(h);
   for (int32_t b = 0; b < nbatch; ++b) h->h_status[b] = LLONG_MAX;
   CUDA_TRY(cudaMemcpyAsync(h->d_status, h->h_status, sizeof(long long) * nbatch, cudaMemcpyHostToDevice, h->stream),
            "status reset");

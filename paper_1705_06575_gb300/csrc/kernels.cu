@@ -2621,6 +2621,9 @@ cudaError_t prepare_factor() {
   if constexpr (std::is_same<T, float>::value) {
     e = prepare_update_tc();
     if (e != cudaSuccess) return e;
+  } else {
+    e = prepare_oz();
+    if (e != cudaSuccess) return e;
   }
   return cudaFuncSetAttribute(k_trtri<T, NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trtri_smem<NB>());
 }
@@ -2768,6 +2771,13 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
   k_zero<T><<<dim3(grid_for(d.storage, THREADS * 4), nb), THREADS, 0, st>>>(Lx, d.storage, bt);
   if (d.nnz_a > 0)
     k_scatter<T><<<dim3(grid_for(d.nnz_a, THREADS * 4), nb), THREADS, 0, st>>>(Ax, d.amap, Lx, d.nnz_a, bt);
+  // one FP64 matrix on the tensor cores
+  const bool oz = std::is_same<T, double>::value && nb == 1 && d.dg && d.tensor_cores;
+  if constexpr (std::is_same<T, double>::value)
+    if (oz) {
+      cudaError_t e = launch_oz_scale(st, d, Ax);
+      if (e != cudaSuccess) return e;
+    }
   trace_mark(trace, K_SCATTER, st);
   if (dual) {  // the auxiliary stream starts after the panels hold A
     cudaEventRecord(two->fork, st);
@@ -2789,6 +2799,11 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         panel = PANEL_NONE;
     }
     if (panel == PANEL_COVERED) {
+      if constexpr (std::is_same<T, double>::value)
+        if (oz && L.kind == K_TRSM && d.oz[li]) {
+          cudaError_t e = launch_oz_split(g, s, prio, d, Lx, L.off);
+          if (e != cudaSuccess) return e;
+        }
       if (dual) cudaEventRecord((*two->events)[li], s);
       trace_mark(trace, L.kind, st);
       continue;
@@ -2814,6 +2829,8 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
             e = launch_prio(k_update_f32, dim3(g, nb), F32_THREADS, 0, s, prio, d.sn, d.upd_tasks, d.upd_entries,
                             d.rel, Lx, L.off, bt);
         }
+        else if (oz && d.oz[li] && !alt)
+          e = launch_update_oz(g, d.oz[li], s, prio, d, Lx, L.off, status);
         // a batch, lanes = matrices: the default of small tiles and of full tiles with small entries
         // (alternatives: a warp per (tile, matrix) on the tile in shared or global memory), the
         // alternative of full tiles with large entries (default: one CTA per tile and matrix)
@@ -2868,10 +2885,13 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         else  // the tile in registers
           e = launch_prio(k_trsm_r<T>, dim3(g, nb), THREADS, trsm_smem<T, NB>(), s, prio, d.sn, d.tasks, Lx, L.off,
                           bt);
+        if constexpr (std::is_same<T, double>::value)
+          if (e == cudaSuccess && oz && d.oz[li]) e = launch_oz_split(g, s, prio, d, Lx, L.off);
         break;
       case K_GEMM:
         if constexpr (std::is_same<T, double>::value)
-          e = launch_prio(k_gemm<T>, dim3(g, nb), THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
+          e = oz && d.oz[li] ? launch_gemm_oz(g, s, prio, d, Lx, L.off, status) :
+              launch_prio(k_gemm<T>, dim3(g, nb), THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
         else
           e = launch_prio(k_gemm_f32, dim3(g, nb), F32_THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
         break;

@@ -47,8 +47,14 @@ struct DevPlan {
                                      // [0] for one matrix, [1] for batches: 1 runs the launch's
                                      // alternative kernel form (see factor_launch_has_alternative),
                                      // as the autotuner chose; null or 0: the default form
+  // FP64 factors of one matrix on the tensor cores (oz_update.cu): digits of the factored panels,
+  // row scale exponents (per permuted column) and the HOST array of launches (Plan::oz). dg is
+  // null where the SIMT kernels run (SYM_FLAG_NO_TENSOR_CORES, or no memory for the digits).
+  uint4 *dg = nullptr;
+  int32_t *exps = nullptr;
+  const int8_t *oz = nullptr;
   const double *axc = nullptr;       // FP32 factors: the FP64 copy of A's values (nnz_a per matrix)
-  const int64_t *dpos = nullptr;     // FP32 factors: index in A's values of C_kk, per column k
+  const int64_t *dpos = nullptr;     // index in A's values of C_kk, per column k
 };
 
 // Several matrices with one pattern (blockIdx.y = matrix): offsets, in elements, from one matrix to
@@ -94,6 +100,19 @@ cudaError_t prepare_solve();
 cudaError_t prepare_update_tc();
 cudaError_t launch_update_tc(dim3 grid, cudaStream_t st, int prio, const DevPlan &d, float *Lx, int64_t toff,
                              const Batch &bt, long long *status);
+
+// FP64 factors of one matrix on the tensor cores (oz_update.cu). Attributes (once per device,
+// outside capture); the row scales of one set of values; the digits of the row tiles of a TRSM
+// launch; one launch of external updates (cluster CTAs per tile share its entries); one launch of
+// trailing updates. A bounded wait that runs out records -1 in status.
+cudaError_t prepare_oz();
+cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax);
+cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
+                            int64_t toff);
+cudaError_t launch_update_oz(unsigned tasks, int cluster, cudaStream_t st, int prio, const DevPlan &d, double *Lx,
+                             int64_t toff, long long *status);
+cudaError_t launch_gemm_oz(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
+                           long long *status);
 
 // Whether a factor launch has a second kernel form (the autotuner times both). A batch
 // (nbatch > 1): FP64 updates with lanes mapped to matrices (default for small tiles and for full

@@ -1,0 +1,218 @@
+// oz.cuh — FP64 products on the FP16 tensor cores: device building blocks shared by the external
+// update and the in-supernode trailing update of FP64 factors (oz_update.cu).
+//
+// Fixed point. In a Cholesky factor every entry obeys |l_ik| <= sqrt(a_ii). Row i of the factor
+// gets the scale 2^e_i with sqrt(a_ii) < 0.986 * 2^e_i (e_i from the diagonal of A alone, known
+// before the factorization), and v = l_ik / 2^e_i is held as a 56-bit fixed-point number
+// v = sum_{s<7} d_s 2^(-7 - 8 s), the digits d_s integers in [-128, 127] (rounding error at most
+// 2^-56). A digit is exact in FP16, a product of digits is an integer of magnitude <= 2^14, and
+// an FP32 accumulator is exact while its sum stays below 2^24.
+//
+// Products. sum_k v_ik v_jk = sum_p 2^(-14 - 8 p) sum_{s+t=p} sum_k d_s(i,k) d_t(j,k). All pairs
+// s + t <= 7 are formed (34 products of digit matrices); the dropped ones are below 2^-62 of the
+// scale per term, as is the rounding of the digits, so the sum carries an error of the order of
+// 2^-62 sqrt(K) in units of sqrt(a_ii a_jj), less than FP64 multiply-adds leave (one rounding of
+// 2^-54 of the running value per step). The accumulators are combined in 64-bit integers (unit
+// 2^-62: the sum is below 2^62 by Cauchy-Schwarz, intermediate wrap-around cancels), whole tiles
+// are summed without any rounding, and the tile is updated with one FP64 rounding per entry.
+//
+// Layout. The digits of a factored panel are kept in FP16 as the tensor core reads them: octets of
+// eight columns, per octet the seven slices, per slice the rows, sixteen bytes each. A stage holds
+// 16 values of k of 64 rows per operand in the K-major core-matrix layout with the row groups 128
+// bytes apart and the octets LBO apart, so rows are copied as they are, two consecutive slices of
+// the A operand form one M = 128 operand, and consecutive slices of 32 rows of the B operand (a
+// half of the tile's columns) one operand of N = 32 per slice. The MMA of A slices (2a, 2a+1) with
+// B slices 0..T-1 adds to the half's accumulator column blocks 2a .. 2a+T-1 (32 columns each):
+// block c holds weight p = c in lanes 0-63 (even s) and p = c + 1 in lanes 64-127 (odd s). Four
+// MMAs per 16 values of k and half (N = 224, 192, 128, 64), 256 columns of tensor memory per half:
+// one half is read back while the other one accumulates. Each accumulator lane sums at most four
+// pairs per k, so 256 values of k (4 * 256 * 2^14 = 2^24) are exact; a segment of that length is
+// then read back.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "plan.h"
+#include "tc.cuh"
+
+namespace sym {
+namespace oz {
+
+constexpr int SL = 7;                       // digits per value
+constexpr uint32_t A_SLICE = 64 * 16;       // one octet of k of one slice: 64 rows of 16 bytes
+constexpr uint32_t B_SLICE = 32 * 16;       // the same of half the tile's columns
+constexpr uint32_t B_HALF = SL * B_SLICE;   // the other half of the columns
+constexpr uint32_t SBO = 128;               // next 8 rows
+constexpr uint32_t A_LBO = 8 * A_SLICE;     // next octet of k: seven slices and one of zeros (the
+constexpr uint32_t B_LBO = 2 * B_HALF;      // partner of slice 6) for A, two halves for B
+constexpr uint32_t A_BYTES = 2 * A_LBO;
+constexpr uint32_t B_BYTES = 2 * B_LBO;
+constexpr uint32_t STAGE = A_BYTES + B_BYTES;
+constexpr uint32_t TMEM_COLS = 512;
+constexpr int SEG_STEPS = 16;               // K = 16 steps per segment (256 values of k)
+constexpr uint64_t OFFSET = 0x0080808080808080ull;  // digit 0 is stored as byte 128
+constexpr uint64_t QMAX = 0x00FFFFFFFFFFFFFFull - OFFSET;
+
+// Scale exponent of a row from its diagonal entry a of A: sqrt(a) <= 0.986 * 2^e. Rows whose
+// diagonal is not a positive finite number fail as pivots whatever their scale.
+__device__ __forceinline__ int scale_exponent(double a) {
+  if (!(a > 0.0)) return 0;
+  if (!(a < 1.7e308)) return 513;
+  int x;
+  frexp(a, &x);  // a < 2^x; 1.03 a < 2^(x + 1)
+  double f = ldexp(a, -x);
+  if (f * 1.03 > 1.0) ++x;
+  return (x + 1) >> 1;
+}
+
+// v / 2^e as a 56-bit fixed-point number with unit 2^-55, rounded to nearest, saturated (a
+// saturated row fails as a pivot: its sum of squares exceeds its diagonal), plus OFFSET.
+__device__ __forceinline__ uint64_t to_fixed(double v, int e) {
+  const uint64_t bits = (uint64_t)__double_as_longlong(v);
+  const int E = (int)(bits >> 52) & 0x7ff;
+  const uint64_t m = (bits & 0xFFFFFFFFFFFFFull) | (E ? 0x10000000000000ull : 0ull);
+  const int sh = (E ? E : 1) - 1020 - e;  // q = m 2^sh
+  uint64_t q;
+  if (E == 0x7ff || sh > 2) q = QMAX;
+  else if (sh >= 0) q = m << sh;
+  else if (sh >= -54) q = (m + (1ull << (-sh - 1))) >> (-sh);
+  else q = 0;
+  q = q < QMAX ? q : QMAX;
+  return (bits >> 63) ? OFFSET - q : OFFSET + q;
+}
+
+__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+  return r;
+}
+// Byte transpose of four words: out[k] = byte k of w0, w1, w2, w3.
+__device__ __forceinline__ void transpose4(uint32_t w0, uint32_t w1, uint32_t w2, uint32_t w3, uint32_t (&out)[4]) {
+  const uint32_t t0 = prmt(w0, w1, 0x5140), t1 = prmt(w2, w3, 0x5140);
+  const uint32_t t2 = prmt(w0, w1, 0x7362), t3 = prmt(w2, w3, 0x7362);
+  out[0] = prmt(t0, t1, 0x5410);
+  out[1] = prmt(t0, t1, 0x7632);
+  out[2] = prmt(t2, t3, 0x5410);
+  out[3] = prmt(t2, t3, 0x7632);
+}
+// Two digits (bytes 128 + d) to FP16: the byte under the exponent byte 0x64 is 1024 + 128 + d,
+// exact; minus 1152.
+__device__ __forceinline__ uint32_t half2_of(uint32_t w, uint32_t sel) {
+  uint32_t h = prmt(w, 0x64646464u, sel), r;
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));
+  return r;
+}
+// The FP16 digits of eight values (fixed-point numbers with OFFSET), one slice per element of w.
+__device__ __forceinline__ void to_digits(const uint64_t (&q)[8], uint4 (&w)[SL]) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t lo[4], hi[4], b[SL];  // b[s]: digit s of the four values, one byte each
+    transpose4((uint32_t)q[4 * h], (uint32_t)q[4 * h + 1], (uint32_t)q[4 * h + 2], (uint32_t)q[4 * h + 3], lo);
+    transpose4((uint32_t)(q[4 * h] >> 32), (uint32_t)(q[4 * h + 1] >> 32), (uint32_t)(q[4 * h + 2] >> 32),
+               (uint32_t)(q[4 * h + 3] >> 32), hi);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b[6 - k] = lo[k];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) b[2 - k] = hi[k];
+#pragma unroll
+    for (int s = 0; s < SL; ++s) {
+      const uint32_t x = half2_of(b[s], 0x4140), y = half2_of(b[s], 0x4342);
+      if (h == 0) {
+        w[s].x = x;
+        w[s].y = y;
+      } else {
+        w[s].z = x;
+        w[s].w = y;
+      }
+    }
+  }
+}
+
+// Copy sixteen bytes of global memory to shared memory without registers (zeros where !in); groups
+// of copies of this thread, and a wait until at most N groups are in flight.
+__device__ __forceinline__ void copy16(uint32_t dst, const void *src, bool in) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16u : 0u) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// The MMAs of one K = 16 step of one half of the tile's columns, accumulating in the half's
+// column blocks at d. a, b: descriptors of the step's octets (slice 0; b: the half's rows). INIT:
+// first step of a segment, whose first two MMAs together cover all eight column blocks and
+// overwrite them.
+template <bool INIT>
+__device__ __forceinline__ void mma_step(uint32_t d, uint64_t a, uint64_t b) {
+  constexpr uint64_t AS = A_SLICE >> 4, BS = B_SLICE >> 4;
+  tc::mma_f16(d + 32 * 4, a + 4 * AS, b, tc::idesc_f16<128>(), INIT ? 0u : 1u);  // s 4,5: t 0-3
+  if (INIT) {
+    tc::mma_f16(d, a, b, tc::idesc_f16<128>(), 0u);                              // s 0,1: t 0-3
+    tc::mma_f16(d + 32 * 4, a, b + 4 * BS, tc::idesc_f16<96>(), 1u);             // s 0,1: t 4-6
+  } else {
+    tc::mma_f16(d, a, b, tc::idesc_f16<224>(), 1u);                              // s 0,1: t 0-6
+  }
+  tc::mma_f16(d + 32 * 2, a + 2 * AS, b, tc::idesc_f16<192>(), 1u);              // s 2,3: t 0-5
+  tc::mma_f16(d + 32 * 6, a + 6 * AS, b, tc::idesc_f16<64>(), 1u);               // s 6: t 0-1
+}
+
+// Read a finished segment of one half back and add it to the 64-bit sums, unit 2^-62: this warp's
+// 32 lanes, eight columns from addr (of block 0). Weight p sits in block p (lanes 0-63) or p - 1
+// (lanes 64-127, up). SHORT: a segment of at most 64 values of k, whose sums are at most 2^22 in
+// magnitude: adding 1.5 * 2^23 leaves the integer in the low bits (a conversion runs at 16 per
+// clock and SM, an addition at 128), and pairs of weights combine in 32 bits. diag: this lane's
+// row has its diagonal entry here, in column q0; dsum gets its approximate sum of squares.
+template <bool SHORT>
+__device__ __forceinline__ void drain(uint32_t addr, bool up, unsigned long long (&acc)[8], bool diag, int q0,
+                                      float &dsum) {
+  const uint32_t base = addr - (up ? 32u : 0u);
+#pragma unroll
+  for (int p = 0; p < 8; p += 2) {
+    uint32_t v[8], w[8];
+    tc::ld8x2(base + (p == 0 && up ? 32u : 32u * p), base + 32u * (p + 1), v, w);
+    if (p == 0 && up) {  // (weight 0 has no odd slice)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = 0u;
+    }
+    if (diag && p < 4) {
+      float x = 0.f, y = 0.f;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        x = q == q0 ? __uint_as_float(v[q]) : x;
+        y = q == q0 ? __uint_as_float(w[q]) : y;
+      }
+      const float u = 1.0f / (float)(1ll << (14 + 8 * p));
+      dsum += x * u + y * (u / 256.0f);
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      int x, y;
+      if constexpr (SHORT) {
+        x = __float_as_int(__uint_as_float(v[q]) + 12582912.0f) - 0x4B400000;
+        y = __float_as_int(__uint_as_float(w[q]) + 12582912.0f) - 0x4B400000;
+      } else {
+        x = __float2int_rn(__uint_as_float(v[q]));
+        y = __float2int_rn(__uint_as_float(w[q]));
+      }
+      if (p == 0) acc[q] += (unsigned long long)((unsigned)x * 65536u + (unsigned)y * 256u) << 32;
+      else if (p == 2) acc[q] += ((unsigned long long)(unsigned)x << 32) + (unsigned long long)((long long)y * (1 << 24));
+      else if (p == 4) acc[q] += SHORT ? (unsigned long long)((long long)(x * 256 + y) * 256)
+                                       : (unsigned long long)((long long)x * (1 << 16)) +
+                                             (unsigned long long)((long long)y * 256);
+      else acc[q] += (unsigned long long)(long long)(x + ((y + 128) >> 8));
+    }
+  }
+}
+
+// c - q 2^(-62) 2^ei 2^ej with one rounding of the product's conversion and one of the sum.
+__device__ __forceinline__ double apply(double c, long long q, int ei, int ej) {
+  const int x = ei + ej - 62;
+  if (x > -1000 && x < 1000) return fma(-(double)q, __hiloint2double((x + 1023) << 20, 0), c);
+  return c - ldexp((double)q, x);
+}
+
+}  // namespace oz
+}  // namespace sym

@@ -1,0 +1,639 @@
+// oz_update.cu — FP64 factors on the FP16 tensor cores: digits of the factored panels, the external
+// update of a tile by its descendants, and the trailing update inside a supernode. The arithmetic
+// (fixed-point digits, exact products, 64-bit sums) is described in oz.cuh.
+#include <cooperative_groups.h>
+#include <cuda_runtime.h>
+
+#include <cstdint>
+#include <type_traits>
+
+#include "kernels.h"
+#include "oz.cuh"
+#include "tc.cuh"
+
+namespace cg = cooperative_groups;
+
+namespace sym {
+namespace {
+
+__device__ __forceinline__ int64_t tile_base(int32_t i, int32_t ncols, int32_t ncb) {
+  return i < ncb ? (int64_t)i * NB : (int64_t)ncols + (int64_t)(i - ncb) * NB;
+}
+__device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows, int32_t ncb) {
+  const int64_t base = tile_base(i, ncols, ncb);
+  const int64_t r = (i < ncb ? ncols : nrows) - base;
+  return (int)(r < NB ? r : NB);
+}
+
+// Row scales of one factorization: exps[k] from C_kk (permuted column k).
+__global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restrict__ dpos, int32_t *__restrict__ exps,
+                           int64_t n) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) exps[k] = oz::scale_exponent(Ax[dpos[k]]);
+}
+
+// Digits of a factored row tile (task {J, i, s} of a TRSM launch): thread (row, o) takes the eight
+// columns of octet o (and o + 4) of one row. Storage: octet of columns, slice, row: sixteen bytes
+// each, at sn.dg + (octet * 7 + slice) * nrows + row; an even number of octets per panel.
+__global__ void __launch_bounds__(256) k_oz_split(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
+                                                  const int32_t *__restrict__ rows, const double *__restrict__ Lx,
+                                                  uint4 *__restrict__ dg, const int32_t *__restrict__ exps,
+                                                  int64_t toff) {
+  const Int4 t = tasks[toff + blockIdx.x];
+  const SNode sj = sn[t.a];
+  if (sj.dg < 0) return;
+  const int i = t.b, s = t.c;
+  const int ts = min(NB, sj.ncols - s * NB);
+  int64_t rb = tile_base(i, sj.ncols, sj.ncb);
+  int tm = tile_rows(i, sj.ncols, sj.nrows, sj.ncb);
+  const int half = t.d >> 16;
+  if (half) {
+    rb += (half - 1) * (NB / 2);
+    tm = max(0, min(NB / 2, tm - (half - 1) * (NB / 2)));
+  }
+  const int row = threadIdx.x & (NB - 1);
+  if (row >= tm) return;
+  const int64_t ld = sj.nrows, r = rb + row;
+  const int e = exps[rows[sj.rowp + r]];
+  for (int o = threadIdx.x >> 6; 16 * (o >> 1) < ts; o += 4) {
+    const double *src = Lx + sj.lx + (int64_t)(s * NB + 8 * o) * ld + r;
+    double v[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = 8 * o + c < ts ? src[c * ld] : 0.0;
+    uint64_t q[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) q[c] = oz::to_fixed(v[c], e);
+    uint4 w[oz::SL];
+    oz::to_digits(q, w);
+    uint4 *dst = dg + sj.dg + (int64_t)(s * (NB / 8) + o) * oz::SL * ld + r;
+#pragma unroll
+    for (int k = 0; k < oz::SL; ++k) dst[k * ld] = w[k];
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// The products. Two kernels share one pipeline: the external update of 64 x 64 tiles by all their
+// descendant entries (UPD; every entry's rows are placed in the tile's coordinates through inverse
+// row maps while they are staged, rows it does not touch are zero, so all entries of a tile add up
+// in the same accumulators), and the trailing update inside a supernode (one "entry": column tile
+// s of J, rows onto themselves).
+//
+// A tile's column groups of sixteen (over all its entries) form one sequence of chunks. A CTA
+// is persistent over tiles and its warps have fixed roles, linked by mbarriers with bounded waits
+// and without CTA-wide barriers:
+//   * warps 16-19 stage chunks into a six-stage ring (thread = operand, row: one asynchronous copy
+//     per octet and slice);
+//   * warps 20 and 21 issue the MMAs, one for each half of the tile's columns, whose segments end
+//     four chunks apart (an issuing thread is held until its MMA is nearly done, so one thread
+//     leaves the tensor core idle whenever it does anything else);
+//   * warps 0-15 read finished segments back (64-bit sums in registers), and with a half of a tile
+//     complete exchange the sums of the even-slice and odd-slice lanes and update C;
+//   * warps 22-23 prepare the entry descriptors and row maps of the following batches of entries
+//     (of this tile or the next), so their chains of dependent loads stay off the other warps.
+// One CTA per SM: the accumulators take all of tensor memory, the ring 180 KB. The MMAs read 140 KB
+// of shared memory per chunk and the staging writes 57 KB, 1.5k cycles at 128 bytes per clock
+// against 1.27k cycles of MMA time (measured without staging); shared memory is the bound.
+// Measured and not kept: digits kept as bytes and converted while they are staged (half the bytes
+// loaded, ~400 instructions per warp and chunk: 4.6k cycles per chunk); staging and read-back in
+// the same sixteen warps with whole-tile accumulators (4.1k cycles: the read-back, limited by the
+// conversions, stops both the staging and the MMAs).
+// A wait that runs out (wait_ns) records -1 in *status; every role then leaves its loop. withhold
+// != 0 (a failure-path test) issues no MMA and no commit.
+constexpr int NSTAGE = 6, LAG = 2;
+constexpr int EB = 16;      // entries per batch
+constexpr int NMETA = 2;    // batches in flight, one per descriptor warp
+constexpr int EPI_WARPS = 16, LOAD_WARPS = 4, MMA_WARP = EPI_WARPS + LOAD_WARPS;
+constexpr int META_WARP = MMA_WARP + 2;
+constexpr int OZ_THREADS = 32 * (META_WARP + NMETA);
+constexpr unsigned OZ_CTAS = OZ_SMS;
+struct OzBatch {
+  int64_t dg[EB];          // first octet of the entry's digits
+  int64_t c;               // offset of the tile in Lx (last batch of a tile)
+  int32_t ld[EB], ng[EB], rlo[EB], clo[EB];
+  int32_t ne, total;       // entries, groups; total = -1: no more tiles
+  int32_t last, diag;      // last batch of its tile; diag - 1: first row of a diagonal tile (0: none)
+  int32_t cld, tm, tn;
+  int16_t erow[NB], ecol[NB];  // scale exponents of the tile's rows and columns
+  int8_t inv[2][EB][NB];   // [0] rows, [1] columns: tile position -> entry row, or -1
+};
+struct OzShared {
+  OzBatch eb[NMETA];
+  unsigned long long red[NB * NB];  // exchanged sums
+  float dred[2][8][2][32];          // [half][warp pair][even, odd slices][lane]
+  uint64_t full[NSTAGE], empty[NSTAGE], done[2], drained[2], mfull[NMETA], mempty[NMETA], xch[8];
+  uint32_t tmem;
+  int bad;
+};
+constexpr size_t OZ_SMEM = NSTAGE * oz::STAGE + sizeof(OzShared) + 128;
+static_assert(OZ_SMEM <= 227 * 1024, "shared memory of one SM");
+
+// Segments of the two halves of a tile: at most SEG_STEPS steps each, half 1's first one half as
+// long, so that the two halves do not wait for their read-backs at the same time.
+struct Segments {
+  int n[2], lim[2];
+  __device__ __forceinline__ void tile() {
+    n[0] = n[1] = 0;
+    lim[0] = oz::SEG_STEPS;
+    lim[1] = oz::SEG_STEPS / 2;
+  }
+  // the next chunk; tile_end: the tile's last one. Returns 1 << h: first of a segment of half h,
+  // 4 << h: last of one.
+  __device__ __forceinline__ uint32_t chunk(bool tile_end) {
+    uint32_t info = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (n[h] == 0) info |= 1u << h;
+      if (++n[h] == lim[h] || tile_end) {
+        info |= 4u << h;
+        n[h] = 0;
+        lim[h] = oz::SEG_STEPS;
+      }
+    }
+    if (tile_end) tile();
+    return info;
+  }
+};
+
+template <bool UPD>
+__global__ void __launch_bounds__(OZ_THREADS, 1)
+    k_oz(const SNode *__restrict__ sn, const UpdTask *__restrict__ utasks, const UpdEntry *__restrict__ ents,
+         const int32_t *__restrict__ rel, const Int4 *__restrict__ tasks, const int32_t *__restrict__ rows,
+         double *__restrict__ Lx, const uint4 *__restrict__ dg, const int32_t *__restrict__ exps, int64_t toff,
+         int ntiles, long long *status, uint64_t wait_ns, int withhold) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *stage0 = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
+  OzShared &sh = *reinterpret_cast<OzShared *>(stage0 + NSTAGE * oz::STAGE);
+  cg::cluster_group cluster = cg::this_cluster();
+  const int cs = UPD ? (int)cluster.num_blocks() : 1, rank = UPD ? (int)cluster.block_rank() : 0;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tile0 = blockIdx.x / cs, tstep = gridDim.x / cs;  // a cluster shares a tile's entries
+
+  if (warp == MMA_WARP) tc::tmem_alloc(&sh.tmem, oz::TMEM_COLS);
+  if (tid == 0) {
+    for (int b = 0; b < NSTAGE; ++b) {
+      tc::mbar_init(&sh.full[b], LOAD_WARPS);
+      tc::mbar_init(&sh.empty[b], 2);
+    }
+    for (int b = 0; b < NMETA; ++b) {
+      tc::mbar_init(&sh.mfull[b], 1);
+      tc::mbar_init(&sh.mempty[b], LOAD_WARPS + EPI_WARPS + 2);
+    }
+    for (int h = 0; h < 2; ++h) {
+      tc::mbar_init(&sh.done[h], 1);
+      tc::mbar_init(&sh.drained[h], EPI_WARPS);
+    }
+    for (int b = 0; b < 8; ++b) tc::mbar_init(&sh.xch[b], 2);
+    tc::mbar_init_fence();
+    sh.bad = 0;
+  }
+  if (tid < 128) {  // the zero slice of every octet and stage
+    for (int b = 0; b < NSTAGE; ++b)
+      *reinterpret_cast<uint4 *>(stage0 + b * oz::STAGE + (tid >> 6) * oz::A_LBO + oz::SL * oz::A_SLICE +
+                                 (tid & 63) * 16) = make_uint4(0, 0, 0, 0);
+    tc::fence_smem_to_async();
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  tc::fence_after_sync();
+  const uint32_t tmem = sh.tmem;
+  volatile int *bad = &sh.bad;
+  // a bounded wait that also records its failure; false when this CTA gives up
+  auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if (!tc::mbar_wait(bar, parity, wait_ns)) *bad = 1;
+    return *bad == 0;
+  };
+
+  if (warp >= META_WARP) {
+    // ---- descriptors: batch number b of this CTA's sequence goes to warp b % NMETA
+    const int me = warp - META_WARP;
+    OzBatch &eb = sh.eb[me];
+    int b = 0, uses = 0;
+    bool ok = true;
+    for (int round = 0; ok; ++round) {
+      // (tiles are sorted by work: every other round runs backwards over the CTAs)
+      const int tile = round * tstep + ((round & 1) ? tstep - 1 - tile0 : tile0);
+      const bool end = tile >= ntiles;
+      int64_t ea = 0, ez = 1;
+      int J = 0, i = 0, j = 0, s = 0, hoff = 0, tmax = NB;
+      if (!end) {
+        if (UPD) {
+          const UpdTask t = utasks[toff + tile];
+          const int64_t etot = t.e1 - t.e0;
+          ea = t.e0 + etot * rank / cs;
+          ez = t.e0 + etot * (rank + 1) / cs;
+          i = t.bi;
+          j = t.bj;
+          J = t.J;
+        } else {
+          const Int4 t = tasks[toff + tile];
+          J = t.a;
+          i = t.b;
+          j = t.c;
+          s = t.d & 0xffff;
+          const int half = t.d >> 16;
+          if (half) {
+            hoff = (half - 1) * (NB / 2);
+            tmax = NB / 2;
+          }
+        }
+      }
+      for (int64_t e0 = ea; e0 < ez || e0 == ea; e0 += EB, ++b) {
+        if (b % NMETA != me) continue;
+        if (uses > 0) ok = wait(&sh.mempty[me], (uint32_t)(uses - 1) & 1u);
+        ++uses;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        int total = -1;
+        if (!end) {
+          const SNode sj = sn[J];
+          const int64_t rb = tile_base(i, sj.ncols, sj.ncb) + hoff;
+          const int left = tile_rows(i, sj.ncols, sj.nrows, sj.ncb) - hoff;
+          const int tm = max(0, min(tmax, left)), cb = j * NB, tn = min(NB, sj.ncols - cb);
+          const int ne = UPD ? (int)max((int64_t)0, min((int64_t)EB, ez - e0)) : 1;
+          int ng = 0;
+          if (UPD) {
+            for (int idx = lane; idx < ne * (NB / 4); idx += 32) {
+              reinterpret_cast<int32_t *>(&eb.inv[0][0][0])[idx] = -1;
+              reinterpret_cast<int32_t *>(&eb.inv[1][0][0])[idx] = -1;
+            }
+            if (lane < ne) {
+              const UpdEntry E = ents[e0 + lane];
+              const SNode *sk = &sn[E.K];
+              eb.dg[lane] = sk->dg;
+              eb.ld[lane] = sk->nrows;
+              eb.ng[lane] = ng = (sk->ncols + 15) >> 4;
+              eb.rlo[lane] = E.r_lo;
+              eb.clo[lane] = E.c_lo;
+            }
+            __syncwarp();
+            for (int k = 0; k < ne; ++k) {
+              const UpdEntry &E = ents[e0 + k];
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const int a = lane + 32 * h;
+                if (a < E.m) eb.inv[0][k][rel[E.relr + a] - (int)rb] = (int8_t)a;
+                if (a < E.n) eb.inv[1][k][rel[E.relc + a] - cb] = (int8_t)a;
+              }
+            }
+          } else {
+            ng = lane == 0 ? (min(NB, sj.ncols - s * NB) + 15) >> 4 : 0;
+            if (lane == 0) {
+              eb.dg[0] = sj.dg + (int64_t)s * (NB / 8) * oz::SL * sj.nrows;
+              eb.ld[0] = sj.nrows;
+              eb.ng[0] = ng;
+              eb.rlo[0] = (int32_t)rb;
+              eb.clo[0] = cb;
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int a = lane + 32 * h;
+              eb.inv[0][0][a] = (int8_t)(a < tm ? a : -1);
+              eb.inv[1][0][a] = (int8_t)(a < tn ? a : -1);
+            }
+          }
+          total = __reduce_add_sync(0xffffffffu, ng);
+          if (e0 + EB >= ez) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int a = lane + 32 * h;
+              if (a < tm) eb.erow[a] = (int16_t)exps[rows[sj.rowp + rb + a]];
+              if (a < tn) eb.ecol[a] = (int16_t)exps[sj.first + cb + a];
+            }
+          }
+          if (lane == 0) {
+            eb.ne = ne;
+            eb.last = e0 + EB >= ez;
+            eb.diag = i == j ? hoff + 1 : 0;
+            eb.c = sj.lx + (int64_t)cb * sj.nrows + rb;
+            eb.cld = sj.nrows;
+            eb.tm = tm;
+            eb.tn = tn;
+          }
+        }
+        if (lane == 0) eb.total = total;
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&sh.mfull[me]);
+      }
+      if (end) break;
+    }
+  } else if (warp >= MMA_WARP) {
+    // ---- MMA issue, one warp per half of the tile's columns. The whole warp runs the loop on values
+    // the compiler knows to be uniform (shuffles), lane 0 issues: with the loop inside one lane's
+    // branch every operand of every MMA is moved to a uniform register by itself.
+    const uint32_t h = __shfl_sync(0xffffffffu, (uint32_t)(warp - MMA_WARP), 0);
+    const uint32_t d = __shfl_sync(0xffffffffu, tmem, 0) + 256u * h;
+    const uint32_t smem0 = __shfl_sync(0xffffffffu, tc::smem_addr(stage0), 0);
+    const uint64_t adesc = tc::desc(smem0, oz::A_LBO, oz::SBO);
+    const uint64_t bdesc = tc::desc(smem0 + oz::A_BYTES + h * oz::B_HALF, oz::B_LBO, oz::SBO);
+    Segments seg;
+    seg.tile();
+    uint32_t st = 0, ph = 0, segs = 0;
+    bool ok = true;
+    for (int b = 0; ok; ++b) {
+      const int mb = b % NMETA;
+      if (!(ok = __all_sync(0xffffffffu, wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u)))) break;
+      const int total = __shfl_sync(0xffffffffu, *(volatile int *)&sh.eb[mb].total, 0);
+      const int last = __shfl_sync(0xffffffffu, *(volatile int *)&sh.eb[mb].last, 0);
+      if (total < 0) break;
+      if (lane == 0) tc::mbar_arrive(&sh.mempty[mb]);
+#pragma unroll 1
+      for (int c = 0; c < total; ++c) {
+        const uint32_t info = seg.chunk(last && c + 1 == total);
+        const uint32_t first = (info >> h) & 1u;
+        // the accumulators are free once the half's previous segment has been read
+        ok = (!first || segs == 0 || wait(&sh.drained[h], (segs - 1) & 1u)) && wait(&sh.full[st], ph);
+        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        segs += first;
+        const uint64_t a = adesc + st * (oz::STAGE >> 4), bd = bdesc + st * (oz::STAGE >> 4);
+        if (!withhold && lane == 0) {
+          tc::fence_after_sync();
+          if (first) oz::mma_step<true>(d, a, bd);
+          else oz::mma_step<false>(d, a, bd);
+          if (info & (4u << h)) tc::commit(&sh.done[h]);
+          tc::commit(&sh.empty[st]);
+        }
+        __syncwarp();
+        if (++st == NSTAGE) {
+          st = 0;
+          ph ^= 1;
+        }
+      }
+    }
+  } else if (warp >= EPI_WARPS) {
+    // ---- staging
+    const int lt = tid - 32 * EPI_WARPS, op = lt >> 6, p = lt & (NB - 1);  // operand, row
+    const uint32_t dst0 = tc::smem_addr(stage0) +
+                          (op ? oz::A_BYTES + (uint32_t)(p >> 5) * oz::B_HALF + 16u * (p & 31) : 16u * p);
+    const uint32_t lbo = op ? oz::B_LBO : oz::A_LBO, slice = op ? oz::B_SLICE : oz::A_SLICE;
+    // A chunk is announced (one arrival per warp: an asynchronous arrival of every thread costs ~8
+    // cycles each on the barrier, 1k cycles per chunk) LAG chunks after its copies were issued, or
+    // when the sequence pauses.
+    int it = 0, told = 0;  // chunks issued, chunks announced
+    auto tell = [&]() {
+      tc::fence_smem_to_async();
+      __syncwarp();
+      for (; told < it; ++told)
+        if (lane == 0) tc::mbar_arrive(&sh.full[told % NSTAGE]);
+    };
+    bool ok = true;
+    for (int b = 0; ok; ++b) {
+      const int mb = b % NMETA;
+      if (told < it && !__all_sync(0xffffffffu, tc::mbar_test(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) {
+        oz::copies_wait<0>();
+        tell();
+      }
+      if (!(ok = wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) break;
+      const OzBatch &eb = sh.eb[mb];
+      const int total = eb.total, ne = eb.ne;
+      if (total < 0) break;
+      int ci = 0, cgp = 0;  // position in the sequence of groups: entry, group
+      const uint4 *src = dg;
+      int64_t ld = 0;
+      int r = -1;
+      auto enter = [&]() {  // the row of entry ci at this thread's tile position
+        r = ci < ne ? eb.inv[op][ci][p] : -1;
+        ld = 0;
+        src = dg;
+        if (r >= 0) {
+          ld = eb.ld[ci];
+          src += eb.dg[ci] + (op ? eb.clo[ci] : eb.rlo[ci]) + r;
+        }
+      };
+      if (total > 0) enter();
+      for (int c = 0; c < total; ++c, ++it) {
+        const int st = it % NSTAGE;
+        if (it >= NSTAGE && !(ok = wait(&sh.empty[st], (uint32_t)(it / NSTAGE - 1) & 1u))) break;
+        const uint32_t dst = dst0 + (uint32_t)st * oz::STAGE;
+#pragma unroll
+        for (int o = 0; o < 2; ++o)
+#pragma unroll
+          for (int k = 0; k < oz::SL; ++k) {
+            oz::copy16(dst + o * lbo + k * slice, src, r >= 0);
+            src += ld;
+          }
+        oz::copies_commit();
+        if (it - told >= LAG) {
+          oz::copies_wait<LAG>();
+          tc::fence_smem_to_async();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&sh.full[told % NSTAGE]);
+          ++told;
+        }
+        if (++cgp == eb.ng[ci]) {
+          cgp = 0;
+          ++ci;
+          enter();
+        }
+      }
+      if (!ok) break;
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.mempty[mb]);
+    }
+    oz::copies_wait<0>();
+    tell();
+  } else {
+    // ---- read-back: lanes 32 (warp & 3) .. of tensor memory, columns 8 (warp >> 2) .. of each
+    // half of the tile
+    const int row = 32 * (warp & 1) + lane, g8 = 8 * (warp >> 2);
+    const bool up = (warp & 2) != 0;
+    const int pair = (warp & 1) | ((warp >> 2) << 1);  // this warp and the one with the other slices' sums
+    const uint32_t addr0 = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)g8;
+    unsigned long long acc0[8], acc1[8];  // (one set where a segment is a whole tile)
+    float ds0 = 0.f, ds1 = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) acc0[q] = acc1[q] = 0;
+    Segments seg;
+    seg.tile();
+    int segs[2] = {0, 0}, nx = 0;
+    // The finished segment of half h; fin: the tile's last one.
+    auto segment = [&](auto hc, unsigned long long(&acc)[8], float &dsum, const OzBatch &eb, bool fin) -> bool {
+      constexpr int h = decltype(hc)::value;
+      const int dtop = eb.diag - 1;          // (dtop >= 0: a diagonal tile)
+      const int c0 = 32 * h + g8, drow = row + dtop;
+      const bool here = dtop >= 0 && (drow & ~7) == c0;
+      const int k0 = c0 + (up ? 4 : 0);      // the four columns this thread finishes
+      double *C = Lx + eb.c + (int64_t)k0 * eb.cld + row;
+      double cv[4];
+      const int tm = eb.tm, tn = eb.tn;
+      if (!UPD) {  // C's entries, loaded while the MMAs run
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cv[q] = (row < tm && k0 + q < tn) ? C[(int64_t)q * eb.cld] : 0.0;
+      }
+      if (!wait(&sh.done[h], (uint32_t)segs[h] & 1u)) return false;
+      ++segs[h];
+      __syncwarp();
+      tc::fence_after_sync();
+      oz::drain<!UPD>(addr0 + 256u * h, up, acc, here, drow & 7, dsum);
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.drained[h]);
+      if (!fin || cs > 1) return true;
+      if (UPD) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) cv[q] = (row < tm && k0 + q < tn) ? C[(int64_t)q * eb.cld] : 0.0;
+      }
+      // hand four columns' sums to the other warp of the pair (its buffer of this half has been
+      // read: it has arrived for the other half since), keep four
+      unsigned long long *buf = sh.red + (pair * 2 + h) * 8 * 32 + lane;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        buf[(up ? q : q + 4) * 32] = up ? acc[q] : acc[q + 4];
+        acc[q] = up ? acc[q + 4] : acc[q];
+      }
+      if (here) sh.dred[h][pair][up][lane] = dsum;
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.xch[pair]);
+      if (!wait(&sh.xch[pair], (uint32_t)nx & 1u)) return false;
+      ++nx;
+      if (row < tm) {
+        const int ei = eb.erow[row];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int c = k0 + q;
+          if (c < tn && !(dtop >= 0 && c > drow)) {
+            const unsigned long long v = acc[q] + buf[(up ? q + 4 : q) * 32];
+            C[(int64_t)q * eb.cld] =
+                dtop >= 0 && c == drow && sh.dred[h][pair][0][lane] + sh.dred[h][pair][1][lane] > 1.5f
+                    ? -1.0
+                    : oz::apply(cv[q], (long long)v, ei, eb.ecol[c]);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[q] = 0;
+      dsum = 0.f;
+      return true;
+    };
+    bool ok = true;
+    for (int b = 0; ok; ++b) {
+      const int mb = b % NMETA;
+      if (!(ok = wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) break;
+      const OzBatch &eb = sh.eb[mb];
+      const int total = eb.total, last = eb.last;
+      if (total < 0) break;
+      for (int c = 0; c < total && ok; ++c) {
+        const bool fin = last && c + 1 == total;
+        const uint32_t info = seg.chunk(fin);
+        if (info & 4u) ok = segment(std::integral_constant<int, 0>(), acc0, ds0, eb, fin);
+        if (ok && (info & 8u)) {
+          if (UPD) ok = segment(std::integral_constant<int, 1>(), acc1, ds1, eb, fin);
+          else ok = segment(std::integral_constant<int, 1>(), acc0, ds0, eb, fin);
+        }
+      }
+      if (!ok) break;
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.mempty[mb]);
+    }
+    if (UPD && cs > 1 && ok) {  // the even-slice and odd-slice sums of this rank meet in shared memory
+      if (!up) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          sh.red[(g8 + q) * NB + row] = acc0[q];
+          sh.red[(32 + g8 + q) * NB + row] = acc1[q];
+        }
+      }
+      if ((row & 24) == g8) {  // the eight columns that hold the row's diagonal entry
+        sh.dred[0][pair][up][lane] = ds0;
+        sh.dred[1][pair][up][lane] = ds1;
+      }
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.xch[pair]);
+      if (up && wait(&sh.xch[pair], 0)) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          sh.red[(g8 + q) * NB + row] += acc0[q];
+          sh.red[(32 + g8 + q) * NB + row] += acc1[q];
+        }
+      }
+    }
+  }
+  tc::fence_before_sync();
+  __syncthreads();
+  if (warp == MMA_WARP) {
+    // (with a wait that ran out the last MMAs may still be in flight: let them finish, bounded, so
+    // that tensor memory is not given back under them)
+    if (sh.bad && !withhold) __nanosleep(100000);
+    tc::fence_after_sync();
+    tc::tmem_free(tmem, oz::TMEM_COLS);
+  }
+  if (tid == 0 && sh.bad) atomicMin(status, -1ll);
+  if (UPD && cs > 1) {
+    cluster.sync();  // every rank's sums of the whole tile are in its shared memory
+    const UpdTask t = utasks[toff + tile0];
+    const SNode sj = sn[t.J];
+    const int64_t rb = tile_base(t.bi, sj.ncols, sj.ncb);
+    const int tm = tile_rows(t.bi, sj.ncols, sj.nrows, sj.ncb), cb = t.bj * NB, tn = min(NB, sj.ncols - cb);
+    const bool diag = t.bi == t.bj;
+    double *C = Lx + sj.lx + (int64_t)cb * sj.nrows + rb;
+    // rank r finishes the columns c = r mod cs, adding the ranks in order (whole numbers)
+    for (int idx = tid; idx < NB * (NB / cs) && !sh.bad; idx += OZ_THREADS) {
+      const int r = idx & (NB - 1), c = (idx / NB) * cs + rank;
+      if (r >= tm || c >= tn || (diag && c > r)) continue;
+      double *x = C + (int64_t)c * sj.nrows + r;
+      const double old = *x;
+      unsigned long long v = 0;
+      float d = 0.f;
+      for (int o = 0; o < cs; ++o) {
+        v += cluster.map_shared_rank(sh.red, o)[c * NB + r];
+        if (diag && c == r) {
+          const float *dr = cluster.map_shared_rank(&sh.dred[c >> 5][(r >> 5) | ((c >> 3 & 3) << 1)][0][0], o);
+          d += dr[r & 31] + dr[32 + (r & 31)];
+        }
+      }
+      *x = d > 1.5f ? -1.0 : oz::apply(old, (long long)v, exps[rows[sj.rowp + rb + r]], exps[sj.first + cb + c]);
+    }
+    cluster.sync();  // keep the other ranks' shared memory alive until it has been read
+  }
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_oz(void (*kernel)(KArgs...), unsigned grid, int threads, size_t smem, int cs, cudaStream_t st,
+                      int prio, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  cfg.gridDim = dim3(grid * (unsigned)cs, 1, 1);
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  attr[0].id = cudaLaunchAttributePriority;
+  attr[0].val.priority = prio;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cs;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cs > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+}  // namespace
+
+cudaError_t prepare_oz() {
+  cudaError_t e = cudaFuncSetAttribute(k_oz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_oz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
+}
+cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax) {
+  k_oz_scale<<<(unsigned)((d.n + 255) / 256), 256, 0, st>>>(Ax, d.dpos, d.exps, d.n);
+  return cudaGetLastError();
+}
+cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
+                            int64_t toff) {
+  return launch_oz(k_oz_split, tasks, 256, 0, 1, st, prio, d.sn, d.tasks, d.rows, Lx, d.dg, (const int32_t *)d.exps,
+                   toff);
+}
+cudaError_t launch_update_oz(unsigned tasks, int cluster, cudaStream_t st, int prio, const DevPlan &d, double *Lx,
+                             int64_t toff, long long *status) {
+  const unsigned grid = cluster > 1 ? tasks : tasks < OZ_CTAS ? tasks : OZ_CTAS;
+  return launch_oz(k_oz<true>, grid, OZ_THREADS, OZ_SMEM, cluster, st, prio, d.sn, d.upd_tasks, d.upd_entries, d.rel,
+                   d.tasks, d.rows, Lx, (const uint4 *)d.dg, (const int32_t *)d.exps, toff, (int)tasks, status,
+                   d.tc_wait_ns, (int)d.tc_withhold);
+}
+cudaError_t launch_gemm_oz(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
+                           long long *status) {
+  return launch_oz(k_oz<false>, tasks < OZ_CTAS ? tasks : OZ_CTAS, OZ_THREADS, OZ_SMEM, 1, st, prio, d.sn,
+                   d.upd_tasks, d.upd_entries, d.rel, d.tasks, d.rows, Lx, (const uint4 *)d.dg,
+                   (const int32_t *)d.exps, toff, (int)tasks, status, d.tc_wait_ns, (int)d.tc_withhold);
+}
+
+}  // namespace sym

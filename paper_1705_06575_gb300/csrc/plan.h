@@ -80,6 +80,8 @@ inline int solve_lanes_for(const PanelForm &pf, unsigned nb, bool fp64) {
   if (nb > 1) return fp64 ? solve_panel_lanes(pf.pmax, pf.ncmax) : 0;
   return solve_panel_bytes(pf.pmax, pf.ncmax, 32, 8) <= PANEL_SMEM_HARD ? 32 : 0;
 }
+// SMs of the GPU: CTAs of the tensor-core kernels of FP64 factors (one per SM).
+constexpr int OZ_SMS = 152;
 // Trailing-update GEMM CTAs resident on the whole GPU at once (3 per SM on 152 SMs): the size of
 // one wave, used to split the last wave of a long launch into finer work.
 constexpr int GEMM_SLOTS = 3 * 152;
@@ -96,6 +98,7 @@ struct SNode {
   int64_t lx;     // offset into Lx
   int64_t dx;     // offset of the inverses of its diagonal tiles: tile s (order ts) is a
                   // column-major ts x ts block at dx + s * NB * NB
+  int64_t dg;     // offset of its digits (16-byte units; -1: none kept), see oz_update.cu
   int64_t tx;     // offset of its pushed products in the forward solve's buffer t: chunk ch of
                   // its columns gives t[tx + ch * (nrows - ncols) + (r - ncols)] for each row r
                   // below the diagonal block
@@ -228,6 +231,11 @@ struct Plan {
   std::vector<int8_t> panel_apart[2];  // per factor launch, on PANEL_FUSED ones: 1 if the
                                        // autotuner found the level faster as separate launches;
                                        // [0] one matrix, [1] batches
+  // Per factor launch of one FP64 matrix: nonzero if the launch runs on the tensor cores (K_UPDATE:
+  // CTAs per tile, K_GEMM) or its tiles' digits are taken once they are final (K_TRSM); dg_size:
+  // 16-byte units of digit storage.
+  std::vector<int8_t> oz;
+  int64_t dg_size = 0;
   std::vector<Launch> fwd_launches;
   std::vector<Launch> bwd_launches;
   // Per forward / backward solve launch, the fused narrow levels (single matrices, and batches in

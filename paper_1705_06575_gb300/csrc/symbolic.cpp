@@ -925,6 +925,61 @@ int analyze(int64_t n, const int64_t *Ap, const int32_t *Ai, const int32_t *perm
     }
     P.batch_warp[li] = cnt > 0.0 && elems <= BATCH_WARP_ELEMS * cnt;
   }
+  // One FP64 matrix: which launches run on the tensor cores, and which supernodes keep digits. An
+  // update launch does where the estimate of its time there is below the estimate of the SIMT
+  // kernel's. Both were fitted to the levels of the 64^3 7-point grid, microseconds per tile and SM:
+  // the tensor cores take 6.5 + 0.75 per sixteen columns of every entry (levels of 1 - 400 such
+  // groups per tile within 15%), whatever the entry's rows; the SIMT kernel 0.8 per entry plus the
+  // FP64 pipe's time for the entry's flops (8.2 GFLOP/s per SM). The two meet at level 7 (13 narrow
+  // entries per tile: 0.35 ms either way; level 1: 0.06 against 0.39 ms, level 19: 83.6 against
+  // 8.9 ms). A launch of fewer tiles than SMs is as long as its largest tile, shared by a cluster.
+  P.oz.assign(P.factor_launches.size(), 0);
+  std::vector<int8_t> keep(P.snodes.size(), 0);
+  for (size_t li = 0; li < P.factor_launches.size(); ++li) {
+    const Launch &L = P.factor_launches[li];
+    if (L.kind == K_UPDATE && L.tb != SMALL_TILE) {
+      double oz = 0.0, simt = 0.0, oz_max = 0.0, simt_max = 0.0;
+      for (int64_t t = L.off; t < L.off + L.count; ++t) {
+        const UpdTask &u = P.upd_tasks[t];
+        double a = 6.5, b = 0.0;
+        for (int64_t e = u.e0; e < u.e1; ++e) {
+          const UpdEntry &E = P.upd_entries[e];
+          const double nc = P.snodes[E.K].ncols;
+          a += 0.75 * ((P.snodes[E.K].ncols + 15) / 16);
+          b += 0.8 + (u.bi == u.bj ? 1.0 : 2.0) * E.m * E.n * nc / 8200.0;
+        }
+        oz += a;
+        simt += b;
+        oz_max = std::max(oz_max, a);
+        simt_max = std::max(simt_max, b);
+      }
+      const int64_t sms = OZ_SMS;
+      int cs = 1;
+      while (cs < 8 && 2 * cs * L.count <= sms) cs *= 2;
+      oz = std::max(oz / sms, 6.5 + (oz_max - 6.5) / cs);
+      simt = std::max(simt / sms, simt_max / std::max(1, L.cluster));
+      if (oz >= simt) continue;
+      P.oz[li] = (int8_t)cs;
+      for (int64_t t = L.off; t < L.off + L.count; ++t)
+        for (int64_t e = P.upd_tasks[t].e0; e < P.upd_tasks[t].e1; ++e) keep[P.upd_entries[e].K] = 1;
+    } else if (L.kind == K_GEMM) {
+      P.oz[li] = 1;
+      for (int64_t q = L.off; q < L.off + L.count; ++q) keep[P.tasks[q].a] = 1;
+    }
+  }
+  P.dg_size = 0;
+  for (size_t J = 0; J < P.snodes.size(); ++J) {
+    SNode &sj = P.snodes[J];
+    sj.dg = -1;
+    if (!keep[J]) continue;
+    sj.dg = P.dg_size;
+    P.dg_size += (int64_t)((sj.ncols + 15) / 16) * 14 * sj.nrows;
+  }
+  for (size_t li = 0; li < P.factor_launches.size(); ++li) {
+    const Launch &L = P.factor_launches[li];
+    if (L.kind != K_TRSM) continue;
+    for (int64_t q = L.off; q < L.off + L.count && !P.oz[li]; ++q) P.oz[li] = keep[P.tasks[q].a];
+  }
   // Levels of supernodes with at most SMALL_TILE columns run their POTRF, TRSM and TRTRI as one
   // launch (k_panel_b; a batch only where the panels fit, see panel_lanes). Such a level has one
   // launch of each (one column tile, all of it small-tile).

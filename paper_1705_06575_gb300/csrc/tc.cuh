@@ -83,6 +83,23 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t adesc, uint64
       "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// Instruction descriptor of kind::f16 with FP16 operands (A and B formats 0) and an FP32
+// accumulator, both operands K-major, M = 128.
+template <int N>
+__host__ __device__ constexpr uint32_t idesc_f16() {
+  static_assert(N % 16 == 0 && N >= 16 && N <= 256, "cta_group::1 shape with M = 128");
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+// D[tmem] (+)= A * B^T for one K = 16 step of FP16 operands, issued by one thread.
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+                                        uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
 // Arrive on the mbarrier once every MMA this thread issued before has completed.
 __device__ __forceinline__ void commit(uint64_t *mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -98,11 +115,12 @@ __device__ __forceinline__ void mbar_init_fence() {
 }
 
 // Wait until the phase of the given parity has completed; gives up after limit_ns nanoseconds
-// (globaltimer; default about a second) or 2^26 polls and returns false.
+// (globaltimer; default about a second) or 2^26 polls and returns false. The clock is read only
+// once 64 polls have failed: a read of globaltimer takes far longer than a wait that finds its
+// phase complete.
 __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, uint64_t limit_ns = 1000000000ull) {
   const uint32_t a = smem_addr(mbar);
-  uint64_t t0;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  uint64_t t0 = 0;
   for (int i = 0; i < (1 << 26); ++i) {
     uint32_t done;
     asm volatile(
@@ -113,10 +131,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, uint6
         : "r"(a), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((i & 255) == 255) {
+    if ((i & 63) == 63) {
       uint64_t t;
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-      if (t - t0 > limit_ns) return false;
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > limit_ns) return false;
     }
   }
   return false;
@@ -139,6 +158,34 @@ __device__ __forceinline__ void ld32(uint32_t taddr, float (&v)[32]) {
       : "memory");
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+// Eight columns at each of two addresses, as the FP32 bit patterns.
+__device__ __forceinline__ void ld8x2(uint32_t addr0, uint32_t addr1, uint32_t (&r)[8], uint32_t (&t)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(t[0]), "=r"(t[1]), "=r"(t[2]), "=r"(t[3]), "=r"(t[4]), "=r"(t[5]), "=r"(t[6]), "=r"(t[7])
+      : "r"(addr0), "r"(addr1)
+      : "memory");
+}
+// Whether the phase of the given parity has completed, without waiting.
+__device__ __forceinline__ bool mbar_test(uint64_t *mbar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(smem_addr(mbar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+// One arrival (release) on an mbarrier.
+__device__ __forceinline__ void mbar_arrive(uint64_t *mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(mbar)) : "memory");
 }
 
 }  // namespace tc
