@@ -34,6 +34,8 @@ struct sym_handle_s {
   double *d_y = nullptr;          // solve work array
   uint4 *d_dg = nullptr;          // digits of the FP64 panels (one matrix, tensor cores)
   int32_t *d_exps = nullptr;      // their row scale exponents
+  int2 *d_zu = nullptr;           // fixed-point data of their diagonal tiles
+  void *d_zc = nullptr;
   bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
   double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix)
@@ -164,7 +166,7 @@ void release_device(sym_handle_s *h) {
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   {
     void *mp[] = {h->d_Linv, h->d_Lfinv, h->d_Lf, h->d_Axc, h->d_anorm, h->d_anorm_work, h->d_csr_p, h->d_csr_i,
-                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps};
+                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps, h->d_zu, h->d_zc};
     for (void *p : mp)
       if (p) cudaFree(p);
     if (h->h_eta) cudaFreeHost(h->h_eta);
@@ -355,22 +357,32 @@ int ensure_stage(sym_handle_s *h, int64_t count) {
   return SYM_OK;
 }
 
-// Digit storage of one FP64 matrix's factor on the tensor cores, at the first factorization of a
-// single matrix. Without the memory the SIMT kernels run.
+// Digits and fixed-point data of one FP64 matrix's factor on the tensor cores, at the first
+// factorization of a single matrix that has tiles of more than SMALL_TILE columns. Without the
+// memory the SIMT kernels run.
 void ensure_digits(sym_handle_s *h) {
-  if (h->dg_tried || h->precision != SYM_PREC_FP64 || !h->dp.tensor_cores || h->plan.dg_size == 0) return;
+  if (h->dg_tried || h->precision != SYM_PREC_FP64 || !h->dp.tensor_cores || h->plan.max_ncols <= sym::SMALL_TILE)
+    return;
   h->dg_tried = true;
-  const size_t db = sizeof(uint4) * (size_t)h->plan.dg_size, eb = sizeof(int32_t) * (size_t)h->plan.n;
-  if (cudaMalloc(&h->d_dg, db) == cudaSuccess && cudaMalloc(&h->d_exps, eb) == cudaSuccess) {
-    h->device_bytes += (int64_t)(db + eb);
+  const size_t n = (size_t)h->plan.n;
+  const size_t bytes[4] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
+                           sizeof(int2) * (size_t)h->plan.dinv_storage, sym::oz_column_bytes() * n};
+  void **const ptr[4] = {(void **)&h->d_dg, (void **)&h->d_exps, (void **)&h->d_zu, &h->d_zc};
+  bool ok = true;
+  for (int i = 0; i < 4 && ok; ++i) ok = cudaMalloc(ptr[i], bytes[i] > 0 ? bytes[i] : 16) == cudaSuccess;
+  if (ok) {
+    for (size_t b : bytes) h->device_bytes += (int64_t)b;
   } else {
     cudaGetLastError();
-    if (h->d_dg) cudaFree(h->d_dg);
-    h->d_dg = nullptr;
-    h->d_exps = nullptr;
+    for (void **p : ptr) {
+      if (*p) cudaFree(*p);
+      *p = nullptr;
+    }
   }
   h->dp.dg = h->d_dg;
   h->dp.exps = h->d_exps;
+  h->dp.zu = h->d_zu;
+  h->dp.zc = h->d_zc;
 }
 
 int check_device(sym_handle_s *h) {

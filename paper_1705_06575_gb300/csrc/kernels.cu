@@ -2772,7 +2772,7 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
   if (d.nnz_a > 0)
     k_scatter<T><<<dim3(grid_for(d.nnz_a, THREADS * 4), nb), THREADS, 0, st>>>(Ax, d.amap, Lx, d.nnz_a, bt);
   // one FP64 matrix on the tensor cores
-  const bool oz = std::is_same<T, double>::value && nb == 1 && d.dg && d.tensor_cores;
+  const bool oz = std::is_same<T, double>::value && nb == 1 && d.exps && d.tensor_cores;
   if constexpr (std::is_same<T, double>::value)
     if (oz) {
       cudaError_t e = launch_oz_scale(st, d, Ax);
@@ -2868,6 +2868,8 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         else if constexpr (std::is_same<T, float>::value)  // the column chain in registers
           e = launch_prio(k_potrf_r, dim3(g, nb), PR_THREADS, 0, s, prio, d.sn, d.tasks, Lx, status, d.piv, d.axc,
                           d.dpos, L.off, bt);
+        else if (oz)  // in fixed point
+          e = launch_potrf_z(g, s, prio, d, Lx, L.off, status);
         else
           e = launch_prio(k_potrf<T, NB>, dim3(g, nb), THREADS, 0, s, prio, d.sn, d.tasks, Lx, status, d.piv, d.axc,
                           d.dpos, L.off, bt);
@@ -2882,11 +2884,19 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         else if (small)
           e = launch_prio(k_trsm<T, SMALL_TB>, dim3(g, nb), TS, trsm_smem<T, SMALL_TB>(), s, prio, d.sn, d.tasks, Lx,
                           L.off, bt);
-        else  // the tile in registers
-          e = launch_prio(k_trsm_r<T>, dim3(g, nb), THREADS, trsm_smem<T, NB>(), s, prio, d.sn, d.tasks, Lx, L.off,
-                          bt);
+        else {
+          bool done = false;
+          if constexpr (std::is_same<T, double>::value)
+            if (oz) {  // in fixed point, digits included
+              e = launch_trsm_z(g, s, prio, d, Lx, L.off);
+              done = true;
+            }
+          if (!done)  // the tile in registers
+            e = launch_prio(k_trsm_r<T>, dim3(g, nb), THREADS, trsm_smem<T, NB>(), s, prio, d.sn, d.tasks, Lx, L.off,
+                            bt);
+        }
         if constexpr (std::is_same<T, double>::value)
-          if (e == cudaSuccess && oz && d.oz[li]) e = launch_oz_split(g, s, prio, d, Lx, L.off);
+          if (e == cudaSuccess && oz && small && d.oz[li]) e = launch_oz_split(g, s, prio, d, Lx, L.off);
         break;
       case K_GEMM:
         if constexpr (std::is_same<T, double>::value)

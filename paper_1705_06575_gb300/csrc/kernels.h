@@ -48,10 +48,13 @@ struct DevPlan {
                                      // alternative kernel form (see factor_launch_has_alternative),
                                      // as the autotuner chose; null or 0: the default form
   // FP64 factors of one matrix on the tensor cores (oz_update.cu): digits of the factored panels,
-  // row scale exponents (per permuted column) and the HOST array of launches (Plan::oz). dg is
-  // null where the SIMT kernels run (SYM_FLAG_NO_TENSOR_CORES, or no memory for the digits).
+  // row scale exponents and fixed-point data of the diagonal tiles (exps, zc: per permuted column;
+  // zu: laid out as the diagonal-tile inverses) and the HOST array of launches (Plan::oz). exps is
+  // null where the SIMT kernels run (SYM_FLAG_NO_TENSOR_CORES, or no memory for these arrays).
   uint4 *dg = nullptr;
   int32_t *exps = nullptr;
+  int2 *zu = nullptr;
+  void *zc = nullptr;
   const int8_t *oz = nullptr;
   const double *axc = nullptr;       // FP32 factors: the FP64 copy of A's values (nnz_a per matrix)
   const int64_t *dpos = nullptr;     // index in A's values of C_kk, per column k
@@ -103,12 +106,17 @@ cudaError_t launch_update_tc(dim3 grid, cudaStream_t st, int prio, const DevPlan
 
 // FP64 factors of one matrix on the tensor cores (oz_update.cu). Attributes (once per device,
 // outside capture); the row scales of one set of values; the digits of the row tiles of a TRSM
-// launch; one launch of external updates (cluster CTAs per tile share its entries); one launch of
+// launch; full diagonal tiles and their panel solves in fixed point (the latter with the digits;
+// oz_column_bytes: size of DevPlan::zc per column); one launch of external updates (cluster CTAs per tile share its entries); one launch of
 // trailing updates. A bounded wait that runs out records -1 in status.
 cudaError_t prepare_oz();
 cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax);
 cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
                             int64_t toff);
+size_t oz_column_bytes();
+cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
+                           long long *status);
+cudaError_t launch_trsm_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff);
 cudaError_t launch_update_oz(unsigned tasks, int cluster, cudaStream_t st, int prio, const DevPlan &d, double *Lx,
                              int64_t toff, long long *status);
 cudaError_t launch_gemm_oz(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,

@@ -67,20 +67,62 @@ __device__ __forceinline__ int scale_exponent(double a) {
   return (x + 1) >> 1;
 }
 
-// v / 2^e as a 56-bit fixed-point number with unit 2^-55, rounded to nearest, saturated (a
-// saturated row fails as a pivot: its sum of squares exceeds its diagonal), plus OFFSET.
-__device__ __forceinline__ uint64_t to_fixed(double v, int e) {
+// |v| / 2^e as a fixed-point number with unit 2^-U, rounded to nearest, at most `most` (a saturated
+// row fails as a pivot: its sum of squares exceeds its diagonal; so does a NaN's row).
+template <int U>
+__device__ __forceinline__ uint64_t fixed_magnitude(double v, int e, uint64_t most) {
   const uint64_t bits = (uint64_t)__double_as_longlong(v);
   const int E = (int)(bits >> 52) & 0x7ff;
   const uint64_t m = (bits & 0xFFFFFFFFFFFFFull) | (E ? 0x10000000000000ull : 0ull);
-  const int sh = (E ? E : 1) - 1020 - e;  // q = m 2^sh
+  const int sh = (E ? E : 1) - (1075 - U) - e;  // q = m 2^sh
   uint64_t q;
-  if (E == 0x7ff || sh > 2) q = QMAX;
+  if (E == 0x7ff || sh > U - 53) q = most;
   else if (sh >= 0) q = m << sh;
   else if (sh >= -54) q = (m + (1ull << (-sh - 1))) >> (-sh);
   else q = 0;
-  q = q < QMAX ? q : QMAX;
-  return (bits >> 63) ? OFFSET - q : OFFSET + q;
+  return q < most ? q : most;
+}
+// v / 2^e with unit 2^-55 plus OFFSET: the digits' bytes.
+__device__ __forceinline__ uint64_t to_fixed(double v, int e) {
+  const uint64_t q = fixed_magnitude<55>(v, e, QMAX);
+  return v < 0.0 ? OFFSET - q : OFFSET + q;
+}
+// v / 2^e with unit 2^-60 (the panel solve's arithmetic).
+constexpr int64_t Q60MAX = (int64_t)(QMAX << 5);
+__device__ __forceinline__ int64_t to_fixed60(double v, int e) {
+  const int64_t q = (int64_t)fixed_magnitude<60>(v, e, (uint64_t)Q60MAX);
+  return v < 0.0 ? -q : q;
+}
+// x = h 2^30 + l with |l| <= 2^29.
+__device__ __forceinline__ int2 split30(int64_t x) {
+  const int64_t l = (int64_t)((uint64_t)x << 34) >> 34;
+  return make_int2((int)((x - l) >> 30), (int)l);
+}
+// The double x 2^(e - 60) (the exponent stays normal: |x| <= 2^60, -537 <= e <= 513).
+__device__ __forceinline__ double from_fixed60(int64_t x, int e) {
+  const double d = (double)x;
+  return x ? __hiloint2double(__double2hiint(d) + ((e - 60) << 20), __double2loint(d)) : 0.0;
+}
+
+// a b / 2^60 rounded, for halves a = (h, l) and b: the low halves' product is left out.
+__device__ __forceinline__ int64_t mul60(int2 a, int2 b) {
+  const int64_t m = (int64_t)a.x * (int64_t)b.y + (int64_t)a.y * (int64_t)b.x;
+  return (int64_t)a.x * (int64_t)b.x + ((m + (1ll << 29)) >> 30);
+}
+// 1 / (4 D / 2^60) with unit 2^-60 for 2^58 <= D < 2^60: an FP32 reciprocal r0 of D / 2^60 (24 bits),
+// held with unit 2^-22, e = 1 - (D / 2^60) r0 formed exactly modulo 2^64 (|e| < 2^-21.4, unit 2^-82),
+// and r0 (1 + e + e^2) / 4, Newton's series through second order: the error is below 2^-59.
+__device__ __forceinline__ int64_t reciprocal60(int64_t D) {
+  const float f = (float)(int)((D + (1ll << 35)) >> 36) * (1.0f / 16777216.0f);
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+  const int R = __float2int_rn(r * 4194304.0f);
+  const int64_t P = (D >> 30) * (int64_t)R, Q = (int64_t)((int)D & 0x3fffffff) * (int64_t)R;
+  const int64_t e = (int64_t)(0ull - (((uint64_t)P << 30) + (uint64_t)Q));
+  const float ef = (float)(int)(e >> 31) * (1.0f / 262144.0f);  // e 2^33 (unit 2^-51 to unit 2^-33)
+  const int64_t c = e + ((int64_t)__float2int_rn(ef * ef) << 16);
+  const int64_t h = (int64_t)(int)(c >> 30) * (int64_t)R, l = (int64_t)((int)c & 0x3fffffff) * (int64_t)R;
+  return ((int64_t)R << 36) + ((h + (l >> 30) + (1ll << 15)) >> 16);
 }
 
 __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {

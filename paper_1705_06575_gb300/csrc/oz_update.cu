@@ -72,6 +72,396 @@ __global__ void __launch_bounds__(256) k_oz_split(const SNode *__restrict__ sn, 
 }
 
 // ---------------------------------------------------------------------------------------------
+// Factorization of full diagonal tiles and their panel solves in fixed point. The FP64 pipe takes 64
+// cycles for a warp's multiply-add however many lanes work, which paces both the column chain of a
+// diagonal tile (44 us) and the panel solve (32 us of FP64 time for a 64 x 64 tile); 32 x 32 bit
+// integer multiply-adds into 64 bits run 13 times as fast. With the row scales every value here is
+// below 1: c_ij / 2^(e_i + e_j) is held with unit 2^-60, operands as two 30-bit halves, a product
+// takes three integer multiply-adds (the low halves' product is below 2^-62) and the sums are exact,
+// against an error of 2^-54 of the running value for every multiply-add in FP64.
+//
+// The chains hold no square root and no division by the pivot: with L = U diag(l_cc), U unit lower
+// triangular, y(r, c) = x(r, c) l_cc solves y_c = c_c - sum_{k<c} y_k u(c, k), and x follows at the
+// end, all columns at once. Column c's exponent sg = ceil(-log2(d_c) / 2) of its pivot d_c = l_cc^2
+// balances the two factors: yh = y 2^sg and uh = u 2^-sg = yh / delta, delta = d_c 2^(2 sg) in [1, 4),
+// are below 2 and 1 (|y| <= l_cc and |u| <= 1 / l_cc for a positive definite matrix), and x = yh /
+// sqrt(delta). An entry beyond its range (|x| > 0.9999: its row cannot have a positive pivot) is
+// clamped to it, which keeps the row's sum of squares above its diagonal.
+struct ZCol {
+  int32_t sg;       // exponent
+  int2 lam;         // 1 / sqrt(delta), halves
+  int32_t pad;
+  int64_t lim;      // 0.9999 l_cc: the range of y
+};
+constexpr int Z_THREADS = 256;
+
+// One sum's halves += (-y) u.
+__device__ __forceinline__ void z_mac(int64_t &hi, int64_t &mid, int2 ny, int2 u) {
+  hi += (int64_t)ny.x * (int64_t)u.x;
+  mid += (int64_t)ny.x * (int64_t)u.y;
+  mid += (int64_t)ny.y * (int64_t)u.x;
+}
+__device__ __forceinline__ int64_t z_value(int64_t hi, int64_t mid) { return hi + ((mid + (1ll << 29)) >> 30); }
+// (sums of more than 32 products of mixed halves could leave 64 bits: fold them, exactly)
+__device__ __forceinline__ void z_fold(int64_t &hi, int64_t &mid) {
+  hi += mid >> 30;
+  mid &= (1ll << 30) - 1;
+}
+__device__ __forceinline__ int64_t shfl64(int64_t v, int lane) {
+  return (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)v, lane);
+}
+// The reciprocal square root of 1 <= d < 4 (see rsqrt_newton in kernels.cu).
+__device__ __forceinline__ double rsqrt_delta(double d) {
+  double x0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(x0) : "d"(d));
+  const double e = fma(-d * x0, x0, 1.0);
+  return fma(x0 * e, fma(0.375, e, 0.5), x0);
+}
+
+// Diagonal tile s of J: 46 us for 64 columns, as the FP64 kernel (44 us); it is bound by the column
+// chain (800 cycles per column in the owner's registers, of which the reciprocal takes half) and
+// the integer multiply-adds of the trailing blocks (1.3k cycles per block). What it gives is the
+// panel solve's operands uh, sg and 1 / sqrt(delta), which the solve (20 us for 32 rows, 55 us with
+// FP64 and a launch for the digits) would otherwise derive in every CTA (38 us).
+// Columns go in blocks of four; warp w owns blocks w and w + 8, lane l rows l
+// and l + 32. Step b, one barrier: the owner of block b factors it (its own columns updated from
+// registers through shuffles), publishes yh and uh, and every warp adds the four columns to its
+// blocks right of them, the owner of block b + 1 that block first.
+constexpr size_t POTRF_SMEM = 2 * NB * NB * sizeof(int2);
+
+__global__ void __launch_bounds__(Z_THREADS) k_potrf_z(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
+                                                       double *__restrict__ Lx, const int32_t *__restrict__ exps,
+                                                       int2 *__restrict__ zu, ZCol *__restrict__ zc,
+                                                       long long *status, int64_t toff) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  int2(*ys)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw);                           // [c][row]: -yh
+  int2(*us)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw + NB * NB * sizeof(int2));  // [c][row]: uh
+  __shared__ int64_t dd[NB];  // delta / 4 of every column, unit 2^-60
+  __shared__ ZCol col[NB];
+  const Int4 t = tasks[toff + blockIdx.x];
+  const SNode sj = sn[t.a];
+  const int s = t.b;
+  const int ts = min(NB, sj.ncols - s * NB);
+  const int64_t ld = sj.nrows, g0 = sj.first + (int64_t)s * NB;
+  double *D = Lx + sj.lx + (int64_t)(s * NB) * ld + s * NB;
+  const int32_t *ec = exps + g0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int64_t hi[2][4][2], mid[2][4][2];  // [slot][column][row half]
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 4 * (warp + 8 * q) + k, r = lane + 32 * h;
+        int64_t v = 0;
+        if (r >= c && r < ts) {
+          const double x = D[(int64_t)c * ld + r];
+          v = r == c && !(x > 0.0) ? -(1ll << 58) : oz::to_fixed60(x, ec[r] + ec[c]);
+        }
+        hi[q][k][h] = v;
+        mid[q][k][h] = 0;
+      }
+  const int nblk = (ts + 3) >> 2;
+  int bn = warp;  // the block in slot 0
+  // block bn + 8 q += the columns of block b. A diagonal entry below -1 stays there: its row fails as a
+  // pivot, and further squares (at most 4 per block) must not wrap around 8 to a positive value.
+  auto mac = [&](int q, int b, const int2 (&y)[4][2]) {
+    const int c0 = 4 * (bn + 8 * q);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int4 p0 = *reinterpret_cast<const int4 *>(&us[4 * b + j][c0]);
+      const int4 p1 = *reinterpret_cast<const int4 *>(&us[4 * b + j][c0 + 2]);
+      const int2 u[4] = {make_int2(p0.x, p0.y), make_int2(p0.z, p0.w), make_int2(p1.x, p1.y), make_int2(p1.z, p1.w)};
+      if (c0 < 32) {  // (rows 0-31 of later columns are above the diagonal)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z_mac(hi[q][k][0], mid[q][k][0], y[j][0], u[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) z_mac(hi[q][k][1], mid[q][k][1], y[j][1], u[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      int64_t &v = c0 < 32 ? hi[q][k][0] : hi[q][k][1];
+      if (lane == ((c0 + k) & 31) && v < -(1ll << 60)) v = -(1ll << 60);
+    }
+  };
+  auto factor = [&](int b) {  // the owner of block b (slot 0)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * b + k;
+      if (c >= ts) {  // (uniform) columns past the tile contribute nothing
+        ys[c][lane] = ys[c][lane + 32] = us[c][lane] = us[c][lane + 32] = make_int2(0, 0);
+        continue;
+      }
+      const int64_t v0 = z_value(hi[0][k][0], mid[0][k][0]), v1 = z_value(hi[0][k][1], mid[0][k][1]);
+      int64_t d = shfl64(c < 32 ? v0 : v1, c & 31);
+      if (d <= 0) {
+        if (lane == 0) atomicMin(status, (long long)(g0 + c));
+        d = 1ll << 59;
+      }
+      const int sg = (61 - (63 - __clzll(d))) >> 1;
+      const int64_t dq = (int64_t)((uint64_t)d << (2 * sg - 2));  // delta / 4
+      const int2 rho = oz::split30(oz::reciprocal60(dq));
+      float root;  // sqrt(delta) = l_cc 2^sg, to a few parts in 10^6
+      asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"((float)(int)(dq >> 36) * (4.0f / 16777216.0f)));
+      const int64_t lim = (int64_t)__float2int_rn(root * (0.9999f * 536870912.0f)) << (31 - sg);
+      if (lane == 0) {
+        dd[c] = dq;
+        col[c].sg = sg;
+        col[c].lim = lim;
+      }
+      int2 ny[2], u[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = lane + 32 * h;
+        int64_t v = h ? v1 : v0;
+        v = v > lim ? lim : v < -lim ? -lim : v;
+        v = r == c ? d : r > c ? v : 0;
+        const int64_t yh = (int64_t)((uint64_t)v << sg);
+        ny[h] = oz::split30(-yh);
+        u[h] = oz::split30(oz::mul60(oz::split30(yh), rho));
+        ys[c][r] = ny[h];
+        us[c][r] = u[h];
+      }
+#pragma unroll
+      for (int k2 = k + 1; k2 < 4; ++k2) {
+        const int c2 = 4 * b + k2;
+        const int2 w = c2 < 32 ? u[0] : u[1];
+        const int2 uc = make_int2(__shfl_sync(0xffffffffu, w.x, c2 & 31), __shfl_sync(0xffffffffu, w.y, c2 & 31));
+#pragma unroll
+        for (int h = 0; h < 2; ++h) z_mac(hi[0][k2][h], mid[0][k2][h], ny[h], uc);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        hi[0][k][h] = hi[1][k][h];
+        mid[0][k][h] = mid[1][k][h];
+      }
+    bn += 8;
+  };
+  if (warp == 0 && nblk > 0) factor(0);
+  __syncthreads();
+  for (int b = 0; b + 1 < nblk; ++b) {
+    if (bn < nblk) {
+      int2 y[4][2];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        y[j][0] = ys[4 * b + j][lane];
+        y[j][1] = ys[4 * b + j][lane + 32];
+      }
+      const bool two = bn + 8 < nblk && bn < 8;  // slot 1 holds a block as well
+      mac(0, b, y);
+      if (b == 7) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) z_fold(hi[0][k][h], mid[0][k][h]);
+      }
+      if (bn == b + 1) {  // (warp-uniform)
+        factor(b + 1);    // moves slot 1 to slot 0
+        if (two) mac(0, b, y);
+        if (two && b == 7) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) z_fold(hi[0][k][h], mid[0][k][h]);
+        }
+      } else if (two) {
+        mac(1, b, y);
+        if (b == 7) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) z_fold(hi[1][k][h], mid[1][k][h]);
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (tid < ts) {
+    const double lam = rsqrt_delta((double)dd[tid] * (4.0 / 1152921504606846976.0));
+    col[tid].lam = oz::split30(__double2ll_rn(lam * 1152921504606846976.0));
+    zc[g0 + tid] = col[tid];
+  }
+  __syncthreads();
+  // the tile in FP64 and uh for its panel solves
+  int2 *zt = zu + sj.dx + (int64_t)s * NB * NB;
+  for (int idx = tid; idx < ts * NB; idx += Z_THREADS) {
+    const int r = idx & (NB - 1), c = idx / NB;
+    if (r >= ts) continue;
+    double x = 0.0;
+    if (r >= c) {
+      const int2 ny = ys[c][r];
+      x = oz::from_fixed60(oz::mul60(make_int2(-ny.x, -ny.y), col[c].lam), ec[r]);
+    }
+    D[(int64_t)c * ld + r] = x;
+    zt[c * ts + r] = r > c ? us[c][r] : make_int2(0, 0);
+  }
+}
+
+// Tile (i, s) <- tile * L_ss^-T, and its digits. Thread (r, g) owns row r and the column blocks g,
+// g + G, ...; a tile of at most 32 rows (the halves of a short launch) spreads its rows over G = 8
+// groups of one warp each, else G = 4 groups of two warps. Step b, one barrier: every thread adds the four solved columns of block b to its
+// columns right of them, the owners of block b + 1 first taking that block and solving it in
+// registers so that the next step can begin.
+constexpr size_t TRSM_SMEM = 2 * NB * NB * sizeof(int2) + NB * sizeof(ZCol);
+
+template <int N, int G, int C>
+__device__ __forceinline__ void trsm_mac(int64_t (&hi)[C], int64_t (&mid)[C], const int2 (&x)[4], const int2 *l) {
+#pragma unroll
+  for (int u = 0; u < N; ++u)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int4 p = *reinterpret_cast<const int4 *>(l + j * NB + 4 * G * u);
+      const int4 q = *reinterpret_cast<const int4 *>(l + j * NB + 4 * G * u + 2);
+      z_mac(hi[4 * u], mid[4 * u], x[j], make_int2(p.x, p.y));
+      z_mac(hi[4 * u + 1], mid[4 * u + 1], x[j], make_int2(p.z, p.w));
+      z_mac(hi[4 * u + 2], mid[4 * u + 2], x[j], make_int2(q.x, q.y));
+      z_mac(hi[4 * u + 3], mid[4 * u + 3], x[j], make_int2(q.z, q.w));
+    }
+}
+
+template <int G>
+__device__ __forceinline__ void trsm_z(unsigned char *smem_raw, const SNode &sj, int s, int64_t rb, int tm,
+                                       const int32_t *__restrict__ rows, double *__restrict__ Lx,
+                                       uint4 *__restrict__ dg, const int32_t *__restrict__ exps,
+                                       const int2 *__restrict__ zu, const ZCol *__restrict__ zc) {
+  constexpr int ROWS = Z_THREADS / G, C = NB / G;  // rows, columns per thread
+  int2(*us)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw);                           // [c][row]: uh(row, c)
+  int2(*xs)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw + NB * NB * sizeof(int2));  // [c][row]: -yh(row, c)
+  ZCol *col = reinterpret_cast<ZCol *>(smem_raw + 2 * NB * NB * sizeof(int2));
+  const int ts = min(NB, sj.ncols - s * NB);
+  const int64_t ld = sj.nrows, g0 = sj.first + (int64_t)s * NB;
+  double *B = Lx + sj.lx + (int64_t)(s * NB) * ld + rb;
+  const int tid = threadIdx.x, r = tid & (ROWS - 1), g = tid / ROWS;
+  const bool live = (r & ~31) < tm;  // warp-uniform: some row of this warp is in the tile
+  const int er = r < tm ? exps[rows[sj.rowp + rb + r]] : 0;
+  double bv[C];
+#pragma unroll
+  for (int u = 0; u < C; ++u) {
+    const int c = 4 * G * (u >> 2) + 4 * g + (u & 3);
+    bv[u] = (r < tm && c < ts) ? B[(int64_t)c * ld + r] : 0.0;
+  }
+  const int2 *zt = zu + sj.dx + (int64_t)s * NB * NB;
+#pragma unroll 4
+  for (int idx = tid; idx < NB * NB; idx += Z_THREADS) {
+    const int rr = idx & (NB - 1), c = idx / NB;
+    us[c][rr] = rr > c && rr < ts ? zt[c * ts + rr] : make_int2(0, 0);
+  }
+  if (tid < NB) {
+    ZCol z = {0, make_int2(0, 0), 0, 0};
+    col[tid] = tid < ts ? zc[g0 + tid] : z;
+  }
+  int64_t hi[C], mid[C];
+#pragma unroll
+  for (int u = 0; u < C; ++u) {
+    const int c = 4 * G * (u >> 2) + 4 * g + (u & 3);
+    hi[u] = r < tm && c < ts ? oz::to_fixed60(bv[u], er + exps[g0 + c]) : 0;
+    mid[u] = 0;
+  }
+  __syncthreads();
+  int bn = g;  // the block in sums 0-3
+  auto solve = [&](int b) {  // the owners of block b: sums 0-3 move out
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * b + k;
+      const int64_t lim = col[c].lim;
+      int64_t v = z_value(hi[k], mid[k]);
+      v = v > lim ? lim : v < -lim ? -lim : v;
+      const int2 ny = oz::split30(-(int64_t)((uint64_t)v << col[c].sg));
+      xs[c][r] = ny;
+#pragma unroll
+      for (int k2 = k + 1; k2 < 4; ++k2) z_mac(hi[k2], mid[k2], ny, us[c][4 * b + k2]);
+    }
+#pragma unroll
+    for (int u = 0; u < C - 4; ++u) {
+      hi[u] = hi[u + 4];
+      mid[u] = mid[u + 4];
+    }
+    bn += G;
+  };
+  const int nblk = (ts + 3) >> 2;
+  if (live && g == 0) solve(0);
+  __syncthreads();
+  for (int b = 0; b + 1 < nblk; ++b) {
+    if (live && bn < nblk) {
+      int2 x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = xs[4 * b + j][r];
+      if (b == 8) {
+#pragma unroll
+        for (int u = 0; u < C; ++u) z_fold(hi[u], mid[u]);
+      }
+      if (bn == b + 1) {  // (warp-uniform)
+        trsm_mac<1, G>(hi, mid, x, &us[4 * b][4 * bn]);
+        solve(b + 1);
+      }
+      const int2 *l = &us[4 * b][4 * bn];
+      switch ((nblk - bn + G - 1) / G) {  // blocks bn, bn + G, ... below nblk
+        case 1: trsm_mac<1, G>(hi, mid, x, l); break;
+        case 2: trsm_mac<2, G>(hi, mid, x, l); break;
+        case 3:
+          if constexpr (G == 4) trsm_mac<3, G>(hi, mid, x, l);
+          break;
+        case 4:
+          if constexpr (G == 4) trsm_mac<4, G>(hi, mid, x, l);
+          break;
+        default: break;
+      }
+    }
+    __syncthreads();
+  }
+  // the tile in FP64 and its digits: thread (row, o) takes octets o, o + G, ... of one row
+  if (r < tm) {
+    for (int o = g; 16 * (o >> 1) < ts; o += G) {
+      uint64_t q[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int c = 8 * o + k;
+        int64_t x = 0;
+        if (c < ts) {
+          const int2 ny = xs[c][r];
+          x = oz::mul60(make_int2(-ny.x, -ny.y), col[c].lam);
+          B[(int64_t)c * ld + r] = oz::from_fixed60(x, er);
+        }
+        x = (x + 16) >> 5;
+        x = max(min(x, (int64_t)oz::QMAX), -(int64_t)oz::QMAX);
+        q[k] = (uint64_t)(x + (int64_t)oz::OFFSET);
+      }
+      if (sj.dg >= 0) {
+        uint4 w[oz::SL];
+        oz::to_digits(q, w);
+        uint4 *dst = dg + sj.dg + (int64_t)(s * (NB / 8) + o) * oz::SL * ld + rb + r;
+#pragma unroll
+        for (int k = 0; k < oz::SL; ++k) dst[k * ld] = w[k];
+      }
+    }
+  }
+}
+
+__global__ void __launch_bounds__(Z_THREADS) k_trsm_z(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
+                                                      const int32_t *__restrict__ rows, double *__restrict__ Lx,
+                                                      uint4 *__restrict__ dg, const int32_t *__restrict__ exps,
+                                                      const int2 *__restrict__ zu, const ZCol *__restrict__ zc,
+                                                      int64_t toff) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const Int4 t = tasks[toff + blockIdx.x];
+  const SNode sj = sn[t.a];
+  int64_t rb = tile_base(t.b, sj.ncols, sj.ncb);
+  int tm = tile_rows(t.b, sj.ncols, sj.nrows, sj.ncb);
+  const int half = t.d >> 16;  // 0: whole tile; 1, 2: its first or second 32 rows
+  if (half) {
+    rb += (half - 1) * (NB / 2);
+    tm = max(0, min(NB / 2, tm - (half - 1) * (NB / 2)));
+  }
+  if (tm > NB / 2) trsm_z<4>(smem_raw, sj, t.c, rb, tm, rows, Lx, dg, exps, zu, zc);
+  else trsm_z<8>(smem_raw, sj, t.c, rb, tm, rows, Lx, dg, exps, zu, zc);
+}
+
+// ---------------------------------------------------------------------------------------------
 // The products. Two kernels share one pipeline: the external update of 64 x 64 tiles by all their
 // descendant entries (UPD; every entry's rows are placed in the tile's coordinates through inverse
 // row maps while they are staged, rows it does not touch are zero, so all entries of a tile add up
@@ -609,6 +999,10 @@ cudaError_t launch_oz(void (*kernel)(KArgs...), unsigned grid, int threads, size
 }  // namespace
 
 cudaError_t prepare_oz() {
+  cudaError_t e0 = cudaFuncSetAttribute(k_trsm_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRSM_SMEM);
+  if (e0 != cudaSuccess) return e0;
+  e0 = cudaFuncSetAttribute(k_potrf_z, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)POTRF_SMEM);
+  if (e0 != cudaSuccess) return e0;
   cudaError_t e = cudaFuncSetAttribute(k_oz<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(k_oz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
@@ -621,6 +1015,16 @@ cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const Dev
                             int64_t toff) {
   return launch_oz(k_oz_split, tasks, 256, 0, 1, st, prio, d.sn, d.tasks, d.rows, Lx, d.dg, (const int32_t *)d.exps,
                    toff);
+}
+size_t oz_column_bytes() { return sizeof(ZCol); }
+cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
+                           long long *status) {
+  return launch_oz(k_potrf_z, tasks, Z_THREADS, POTRF_SMEM, 1, st, prio, d.sn, d.tasks, Lx, (const int32_t *)d.exps,
+                   d.zu, (ZCol *)d.zc, status, toff);
+}
+cudaError_t launch_trsm_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff) {
+  return launch_oz(k_trsm_z, tasks, Z_THREADS, TRSM_SMEM, 1, st, prio, d.sn, d.tasks, d.rows, Lx, d.dg,
+                   (const int32_t *)d.exps, (const int2 *)d.zu, (const ZCol *)d.zc, toff);
 }
 cudaError_t launch_update_oz(unsigned tasks, int cluster, cudaStream_t st, int prio, const DevPlan &d, double *Lx,
                              int64_t toff, long long *status) {
