@@ -61,7 +61,10 @@ struct sym_handle_s {
   bool solve_prepared = false;
   cudaStream_t capture_stream = nullptr;
   sym::PrecondGraph pgraph;       // the FP32 preconditioner of the refined solve, as a graph
+  // (with the captured graphs kept, so that moved inputs and outputs are patched in)
   cudaGraphExec_t fgraph = nullptr;
+  cudaGraph_t fgraph_src = nullptr, sgraph_src = nullptr;
+  sym::CapturedNodes fnodes, snodes;
   const double *fgraph_ax = nullptr;
   cudaGraphExec_t sgraph = nullptr;
   const void *sgraph_key[3] = {nullptr, nullptr, nullptr};
@@ -159,6 +162,21 @@ int collect_trace(sym_handle_s *h, const sym::LaunchTrace &tr, double flop_scale
   return SYM_OK;
 }
 
+void drop_factor_graph(sym_handle_s *h) {
+  if (h->fgraph) cudaGraphExecDestroy(h->fgraph);
+  if (h->fgraph_src) cudaGraphDestroy(h->fgraph_src);
+  h->fgraph = nullptr;
+  h->fgraph_src = nullptr;
+  h->fnodes = sym::CapturedNodes();
+}
+void drop_solve_graph(sym_handle_s *h) {
+  if (h->sgraph) cudaGraphExecDestroy(h->sgraph);
+  if (h->sgraph_src) cudaGraphDestroy(h->sgraph_src);
+  h->sgraph = nullptr;
+  h->sgraph_src = nullptr;
+  h->snodes = sym::CapturedNodes();
+}
+
 void release_device(sym_handle_s *h) {
   for (cudaEvent_t e : h->la_events) cudaEventDestroy(e);
   if (h->la_fork) cudaEventDestroy(h->la_fork);
@@ -173,8 +191,8 @@ void release_device(sym_handle_s *h) {
     if (h->h_pivinfo) cudaFreeHost(h->h_pivinfo);
   }
   for (cudaEvent_t e : h->events) cudaEventDestroy(e);
-  if (h->fgraph) cudaGraphExecDestroy(h->fgraph);
-  if (h->sgraph) cudaGraphExecDestroy(h->sgraph);
+  drop_factor_graph(h);
+  drop_solve_graph(h);
   sym::precond_graph_reset(h->pgraph);
   if (h->capture_stream) cudaStreamDestroy(h->capture_stream);
   void *ptrs[] = {h->d_sn, h->d_rows, h->d_rel, h->d_amap, h->d_updt, h->d_upde, h->d_tasks,
@@ -224,17 +242,13 @@ sym::Batch factor_batch(const sym_handle_s *h, int32_t nbatch, int64_t stride) {
   return bt;
 }
 
+// (The mixed precision factors its own copy of A's values, see copy_values.)
 cudaError_t enqueue_factor(sym_handle_s *h, const double *Ax, int32_t nbatch, int64_t stride, cudaStream_t st,
-                           sym::LaunchTrace *tr) {
-  const sym::Batch bt = factor_batch(h, nbatch, stride);
+                           sym::LaunchTrace *tr, sym::CapturedNodes *nodes = nullptr) {
+  sym::Batch bt = factor_batch(h, nbatch, stride);
   if (h->precision == SYM_PREC_MIXED) {
-    const int64_t nnz = h->plan.nnz_a;
-    if (nnz > 0) {
-      cudaError_t e = cudaMemcpy2DAsync(h->d_Axc, sizeof(double) * nnz, Ax, sizeof(double) * (nbatch > 1 ? stride : nnz),
-                                        sizeof(double) * nnz, nbatch, cudaMemcpyDeviceToDevice, st);
-      if (e != cudaSuccess) return e;
-    }
-    cudaError_t e = sym::run_factor<float>(h->dp, h->plan.factor_launches, Ax, h->d_Lf, h->d_Lfinv, h->d_status,
+    bt.ax = h->plan.nnz_a;
+    cudaError_t e = sym::run_factor<float>(h->dp, h->plan.factor_launches, h->d_Axc, h->d_Lf, h->d_Lfinv, h->d_status,
                                            st, tr, bt, h->aux_stream ? &h->two : nullptr);
     if (e != cudaSuccess) return e;
     for (int32_t b = 0; b < nbatch; ++b) {
@@ -245,14 +259,20 @@ cudaError_t enqueue_factor(sym_handle_s *h, const double *Ax, int32_t nbatch, in
                             h->d_pivinfo, st);
   }
   return sym::run_factor<double>(h->dp, h->plan.factor_launches, Ax, h->d_Lx, h->d_Linv, h->d_status, st, tr, bt,
-                                 h->aux_stream ? &h->two : nullptr);
+                                 h->aux_stream ? &h->two : nullptr, nodes);
+}
+
+// The mixed precision keeps a copy of A's values (before the factorization, outside its graph).
+cudaError_t copy_values(sym_handle_s *h, const double *Ax, int32_t nbatch, int64_t stride) {
+  const int64_t nnz = h->plan.nnz_a;
+  if (h->precision != SYM_PREC_MIXED || nnz == 0) return cudaSuccess;
+  return cudaMemcpy2DAsync(h->d_Axc, sizeof(double) * nnz, Ax, sizeof(double) * (nbatch > 1 ? stride : nnz),
+                           sizeof(double) * nnz, nbatch, cudaMemcpyDeviceToDevice, h->stream);
 }
 
 void drop_graphs(sym_handle_s *h) {
-  if (h->fgraph) cudaGraphExecDestroy(h->fgraph);
-  if (h->sgraph) cudaGraphExecDestroy(h->sgraph);
-  h->fgraph = nullptr;
-  h->sgraph = nullptr;
+  drop_factor_graph(h);
+  drop_solve_graph(h);
   sym::precond_graph_reset(h->pgraph);
 }
 
@@ -677,6 +697,7 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
     }
     h->prepared = true;
   }
+  CUDA_TRY(copy_values(h, Ax, nbatch, stride), "copy A's values");
   sym::LaunchTrace tr, *trp = nullptr;
   if (h->profiling) {
     rc = ensure_events(h, h->plan.factor_launches.size() + 3);
@@ -685,27 +706,36 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
     trp = &tr;
   }
   if (!trp && h->use_graphs) {
-    // Replay the captured launch sequence; capture it again when Ax or the batch moved.
-    if (!h->fgraph || h->fgraph_ax != Ax || h->fgraph_nb != nbatch || h->fgraph_stride != stride) {
+    // Replay the captured launch sequence; capture it again when the batch changes. A moved Ax is
+    // patched into the nodes that read it (a capture of the 64^2 grid's 87 launches takes 0.3 ms).
+    if (!h->fgraph || h->fgraph_nb != nbatch || h->fgraph_stride != stride) {
       rc = ensure_capture_stream(h);
       if (rc) return rc;
-      if (h->fgraph) cudaGraphExecDestroy(h->fgraph);
-      h->fgraph = nullptr;
-      cudaGraph_t g = nullptr;
+      drop_factor_graph(h);
       CUDA_TRY(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal), "capture factor");
-      cudaError_t e = enqueue_factor(h, Ax, nbatch, stride, h->capture_stream, nullptr);
-      cudaError_t e2 = cudaStreamEndCapture(h->capture_stream, &g);
-      if (e != cudaSuccess || e2 != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
+      cudaError_t e = enqueue_factor(h, Ax, nbatch, stride, h->capture_stream, nullptr, &h->fnodes);
+      cudaError_t e2 = cudaStreamEndCapture(h->capture_stream, &h->fgraph_src);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess)
+        e = cudaGraphInstantiate(&h->fgraph, h->fgraph_src, cudaGraphInstantiateFlagUseNodePriority);
+      if (e != cudaSuccess) {
+        drop_factor_graph(h);
         cudaGetLastError();
-        return cuda_fail(e != cudaSuccess ? e : e2, "capture factor");
+        return cuda_fail(e, "capture factor");
       }
-      e = cudaGraphInstantiate(&h->fgraph, g, cudaGraphInstantiateFlagUseNodePriority);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_fail(e, "instantiate factor graph");
       h->fgraph_ax = Ax;
       h->fgraph_nb = nbatch;
       h->fgraph_stride = stride;
+    } else if (h->fgraph_ax != Ax) {
+      cudaError_t e = cudaSuccess;
+      if (h->fnodes.first) e = sym::patch_address(h->fgraph, h->fnodes.first, sym::SCATTER_ARGS, 0, Ax);
+      if (e == cudaSuccess && h->fnodes.second)
+        e = sym::patch_address(h->fgraph, h->fnodes.second, sym::SCALE_ARGS, 0, Ax);
+      if (e != cudaSuccess) {
+        drop_factor_graph(h);
+        return cuda_fail(e, "factor graph");
+      }
+      h->fgraph_ax = Ax;
     }
     CUDA_TRY(cudaGraphLaunch(h->fgraph, h->stream), "factor graph");
   } else {
@@ -794,28 +824,24 @@ int solve_impl(sym_handle h, int32_t nbatch, int32_t nrhs, const double *B, int6
     trp = &tr;
   }
   if (!trp && h->use_graphs && n > 0 && nrhs > 0) {
-    const bool same = h->sgraph && h->sgraph_key[0] == B && h->sgraph_key[1] == X &&
-                      h->sgraph_key[2] == h->d_y && h->sgraph_ikey[0] == nrhs && h->sgraph_ikey[1] == ldb &&
+    const bool same = h->sgraph && h->sgraph_key[2] == h->d_y && h->sgraph_ikey[0] == nrhs && h->sgraph_ikey[1] == ldb &&
                       h->sgraph_ikey[2] == ldx && h->sgraph_nb == nbatch && h->sgraph_bx[0] == bstride &&
                       h->sgraph_bx[1] == xstride;
     if (!same) {
       rc = ensure_capture_stream(h);
       if (rc) return rc;
-      if (h->sgraph) cudaGraphExecDestroy(h->sgraph);
-      h->sgraph = nullptr;
-      cudaGraph_t g = nullptr;
+      drop_solve_graph(h);
       CUDA_TRY(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal), "capture solve");
       cudaError_t e = sym::run_solve<double>(h->dp, h->plan.fwd_launches, h->plan.bwd_launches, h->d_Lx, h->d_Linv,
-                                             nrhs, B, ldb, X, ldx, h->d_y, h->capture_stream, nullptr, bt);
-      cudaError_t e2 = cudaStreamEndCapture(h->capture_stream, &g);
-      if (e != cudaSuccess || e2 != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
+                                             nrhs, B, ldb, X, ldx, h->d_y, h->capture_stream, nullptr, bt, &h->snodes);
+      cudaError_t e2 = cudaStreamEndCapture(h->capture_stream, &h->sgraph_src);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&h->sgraph, h->sgraph_src, 0);
+      if (e != cudaSuccess) {
+        drop_solve_graph(h);
         cudaGetLastError();
-        return cuda_fail(e != cudaSuccess ? e : e2, "capture solve");
+        return cuda_fail(e, "capture solve");
       }
-      e = cudaGraphInstantiate(&h->sgraph, g, 0);
-      cudaGraphDestroy(g);
-      if (e != cudaSuccess) return cuda_fail(e, "instantiate solve graph");
       h->sgraph_key[0] = B;
       h->sgraph_key[1] = X;
       h->sgraph_key[2] = h->d_y;
@@ -825,6 +851,17 @@ int solve_impl(sym_handle h, int32_t nbatch, int32_t nrhs, const double *B, int6
       h->sgraph_nb = nbatch;
       h->sgraph_bx[0] = bstride;
       h->sgraph_bx[1] = xstride;
+    } else {  // moved right-hand sides or solutions: patched into the permutations
+      cudaError_t e = cudaSuccess;
+      if (h->sgraph_key[0] != B) e = sym::patch_address(h->sgraph, h->snodes.first, sym::PERM_ARGS, 1, B);
+      if (e == cudaSuccess && h->sgraph_key[1] != X)
+        e = sym::patch_address(h->sgraph, h->snodes.second, sym::PERM_ARGS, 2, X);
+      if (e != cudaSuccess) {
+        drop_solve_graph(h);
+        return cuda_fail(e, "solve graph");
+      }
+      h->sgraph_key[0] = B;
+      h->sgraph_key[1] = X;
     }
     CUDA_TRY(cudaGraphLaunch(h->sgraph, h->stream), "solve graph");
     return SYM_OK;

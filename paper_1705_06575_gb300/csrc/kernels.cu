@@ -2759,10 +2759,33 @@ cudaError_t launch_panel_b(const DevPlan &d, const PanelForm &pf, unsigned g, un
 #undef SYM_PANEL
 }
 
+cudaError_t captured_node(cudaStream_t st, cudaGraphNode_t *node) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaGraphNode_t *deps = nullptr;
+  size_t ndeps = 0;
+  // (after a launch the capturing stream depends on exactly that launch's node)
+  cudaError_t e = cudaStreamGetCaptureInfo(st, &cap, nullptr, nullptr, &deps, nullptr, &ndeps);
+  if (e != cudaSuccess) return e;
+  if (cap != cudaStreamCaptureStatusActive || ndeps != 1) return cudaErrorInvalidValue;
+  *node = deps[0];
+  return cudaSuccess;
+}
+
+cudaError_t patch_address(cudaGraphExec_t exec, cudaGraphNode_t node, int nargs, int arg, const void *address) {
+  cudaKernelNodeParams p = {};
+  cudaError_t e = cudaGraphKernelNodeGetParams(node, &p);
+  if (e != cudaSuccess) return e;
+  void *args[8];
+  for (int i = 0; i < nargs; ++i) args[i] = p.kernelParams[i];
+  args[arg] = &address;
+  p.kernelParams = args;
+  return cudaGraphExecKernelNodeSetParams(exec, node, &p);
+}
+
 template <typename T>
 cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, const double *Ax,
                        T *Lx, T *Linv, long long *status, cudaStream_t st, LaunchTrace *trace, const Batch &bt,
-                       const TwoStreams *two) {
+                       const TwoStreams *two, CapturedNodes *nodes) {
   const unsigned nb = (unsigned)bt.count;
   // With two streams the schedule's stream/wait fields are honoured (lookahead); otherwise (and
   // when tracing) every launch goes to st in list order, which satisfies every wait.
@@ -2771,11 +2794,16 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
   k_zero<T><<<dim3(grid_for(d.storage, THREADS * 4), nb), THREADS, 0, st>>>(Lx, d.storage, bt);
   if (d.nnz_a > 0)
     k_scatter<T><<<dim3(grid_for(d.nnz_a, THREADS * 4), nb), THREADS, 0, st>>>(Ax, d.amap, Lx, d.nnz_a, bt);
+  if (nodes && d.nnz_a > 0) {
+    cudaError_t e = captured_node(st, &nodes->first);
+    if (e != cudaSuccess) return e;
+  }
   // one FP64 matrix on the tensor cores
   const bool oz = std::is_same<T, double>::value && nb == 1 && d.exps && d.tensor_cores;
   if constexpr (std::is_same<T, double>::value)
     if (oz) {
       cudaError_t e = launch_oz_scale(st, d, Ax);
+      if (e == cudaSuccess && nodes) e = captured_node(st, &nodes->second);
       if (e != cudaSuccess) return e;
     }
   trace_mark(trace, K_SCATTER, st);
@@ -3107,17 +3135,26 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
 template <typename T>
 cudaError_t run_solve(const DevPlan &d, const std::vector<Launch> &fwd, const std::vector<Launch> &bwd,
                       const T *Lx, const T *Linv, int nrhs, const double *B, int64_t ldb, double *X,
-                      int64_t ldx, double *y, cudaStream_t st, LaunchTrace *trace, const Batch &bt) {
+                      int64_t ldx, double *y, cudaStream_t st, LaunchTrace *trace, const Batch &bt,
+                      CapturedNodes *nodes) {
   const int64_t n = d.n;
   const unsigned nb = (unsigned)bt.count;
   if (n == 0 || nrhs == 0) return cudaSuccess;
   trace_mark(trace, -1, st);
   k_perm_in<double><<<dim3(grid_for(n * nrhs, THREADS), nb), THREADS, 0, st>>>(d.perm, B, ldb, y, n, nrhs, bt);
   trace_mark(trace, S_PERM, st);
+  if (nodes) {
+    cudaError_t e = captured_node(st, &nodes->first);
+    if (e != cudaSuccess) return e;
+  }
   cudaError_t e = run_sweeps<T, double>(d, fwd, bwd, Lx, Linv, nrhs, y, st, trace, bt);
   if (e != cudaSuccess) return e;
   k_perm_out<double><<<dim3(grid_for(n * nrhs, THREADS), nb), THREADS, 0, st>>>(d.perm, y, X, ldx, n, nrhs, bt);
   trace_mark(trace, S_PERM, st);
+  if (nodes) {
+    e = captured_node(st, &nodes->second);
+    if (e != cudaSuccess) return e;
+  }
   return cudaGetLastError();
 }
 
@@ -3161,14 +3198,14 @@ template cudaError_t prepare_factor<double>();
 template cudaError_t prepare_factor<float>();
 template cudaError_t run_factor<double>(const DevPlan &, const std::vector<Launch> &, const double *,
                                         double *, double *, long long *, cudaStream_t, LaunchTrace *,
-                                        const Batch &, const TwoStreams *);
+                                        const Batch &, const TwoStreams *, CapturedNodes *);
 template cudaError_t run_factor<float>(const DevPlan &, const std::vector<Launch> &, const double *,
                                        float *, float *, long long *, cudaStream_t, LaunchTrace *,
-                                       const Batch &, const TwoStreams *);
+                                       const Batch &, const TwoStreams *, CapturedNodes *);
 template cudaError_t run_solve<double>(const DevPlan &, const std::vector<Launch> &,
                                        const std::vector<Launch> &, const double *, const double *, int,
                                        const double *, int64_t, double *, int64_t, double *,
-                                       cudaStream_t, LaunchTrace *, const Batch &);
+                                       cudaStream_t, LaunchTrace *, const Batch &, CapturedNodes *);
 template cudaError_t run_sweeps<float, float>(const DevPlan &, const std::vector<Launch> &,
                                               const std::vector<Launch> &, const float *, const float *, int,
                                               float *, cudaStream_t, LaunchTrace *, const Batch &);

@@ -88,6 +88,18 @@ struct LaunchTrace {
   int used = 0;
 };
 
+// The graph nodes of a captured launch sequence that hold the caller's addresses, so that new
+// addresses are patched into the instantiated graph instead of capturing it again: a factorization
+// reads A's values in two kernels (their first argument; the second one only on the tensor cores), a
+// solve the right-hand sides in the first permutation (second argument) and writes the solutions in
+// the last one (third argument). patch_address replaces argument `arg` of the node, a pointer.
+struct CapturedNodes {
+  cudaGraphNode_t first = nullptr, second = nullptr;
+};
+cudaError_t captured_node(cudaStream_t st, cudaGraphNode_t *node);
+cudaError_t patch_address(cudaGraphExec_t exec, cudaGraphNode_t node, int nargs, int arg, const void *address);
+constexpr int SCATTER_ARGS = 5, SCALE_ARGS = 4, PERM_ARGS = 7;
+
 // Per-device function attributes the factor kernels need (call with the device current, before
 // the first run_factor and outside stream capture).
 template <typename T>
@@ -138,7 +150,7 @@ bool factor_launch_has_alternative(const Launch &L, int32_t nbatch, bool fp64);
 template <typename T>
 cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, const double *Ax,
                        T *Lx, T *Linv, long long *status, cudaStream_t st, LaunchTrace *trace = nullptr,
-                       const Batch &bt = Batch(), const TwoStreams *two = nullptr);
+                       const Batch &bt = Batch(), const TwoStreams *two = nullptr, CapturedNodes *nodes = nullptr);
 
 // Solve with nrhs right-hand sides: y = P b, forward sweep, backward sweep, x = P^T y.
 // y: device work array of n * nrhs (ld n); Linv: the diagonal-tile inverses run_factor wrote.
@@ -146,7 +158,7 @@ template <typename T>
 cudaError_t run_solve(const DevPlan &d, const std::vector<Launch> &fwd, const std::vector<Launch> &bwd,
                       const T *Lx, const T *Linv, int nrhs, const double *B, int64_t ldb, double *X,
                       int64_t ldx, double *y, cudaStream_t st, LaunchTrace *trace = nullptr,
-                      const Batch &bt = Batch());
+                      const Batch &bt = Batch(), CapturedNodes *nodes = nullptr);
 
 // The forward and backward sweeps alone on a permuted block y (n x nrhs, ld n) of type V.
 template <typename T, typename V>
