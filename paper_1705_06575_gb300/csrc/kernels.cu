@@ -2823,8 +2823,11 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
     if (panel != PANEL_NONE) {  // unless the autotuner keeps the level apart or a batch's panels do not fit
       const int32_t head = d.batch_panel[li].head;
       const int8_t *apart = d.panel_apart[nb > 1 ? 1 : 0];
-      if ((apart && apart[head]) || panel_lanes_for(d.batch_panel[head], nb, std::is_same<T, float>::value) == 0)
-        panel = PANEL_NONE;
+      constexpr bool f32 = std::is_same<T, float>::value;
+      const bool sep = !apart             ? false
+                       : apart[head] >= 0 ? apart[head] != 0
+                                          : batch_level_apart(d.batch_panel[head], launches[head].count, nb, f32);
+      if (sep || panel_lanes_for(d.batch_panel[head], nb, f32) == 0) panel = PANEL_NONE;
     }
     if (panel == PANEL_COVERED) {
       if constexpr (std::is_same<T, double>::value)
@@ -2859,18 +2862,25 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         }
         else if (oz && d.oz[li] && !alt)
           e = launch_update_oz(g, d.oz[li], s, prio, d, Lx, L.off, status);
-        // a batch, lanes = matrices: the default of small tiles and of full tiles with small entries
-        // (alternatives: a warp per (tile, matrix) on the tile in shared or global memory), the
-        // alternative of full tiles with large entries (default: one CTA per tile and matrix)
-        else if (nb > 1 && d.batch_lanes && d.batch_lanes[li] > 0 &&
-                 (small || (d.batch_warp && d.batch_warp[li])) != alt)
+        // a batch's small tiles: lanes = matrices, or a warp per (tile, matrix) where there are few
+        // (the alternative the other way round)
+        else if (small && nb > 1 && d.batch_lanes && d.batch_lanes[li] > 0 &&
+                 ((int64_t)g * nb > BATCH_WARP_UPDATE) != alt)
           e = launch_update_mb<T>(d.batch_lanes[li], g, nb, s, prio, d, Lx, L.off, bt);
-        else if (small && nb > 1)  // a batch: one warp per (tile, matrix)
+        else if (small && nb > 1)
           e = launch_prio(k_update_wb<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, 0, s, prio,
                           d.sn, d.upd_tasks, d.upd_entries, d.rel, Lx, L.off, (int32_t)nb, bt);
-        else if (!small && nb > 1 && d.batch_warp && d.batch_warp[li])  // small entries of a batch
+        // a batch's full tiles with small entries: a warp per (tile, matrix) in global memory, or one
+        // CTA per pair where there are few (the alternative the other way round: 64 x 100^2 and 128 x
+        // 64^2 grids at 256 - 7000 pairs; against lanes = matrices the warps are 1.1 - 5 times faster
+        // on every such level of these and of 512 x 128^2)
+        else if (!small && nb > 1 && d.batch_warp && d.batch_warp[li] &&
+                 ((int64_t)g * nb > BATCH_CTA_UPDATE) != alt)
           e = launch_prio(k_update_wg<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, 0, s, prio,
                           d.sn, d.upd_tasks, d.upd_entries, d.rel, Lx, L.off, (int32_t)nb, bt);
+        // (full tiles with large entries: one CTA per pair, alternative lanes = matrices)
+        else if (!small && nb > 1 && d.batch_warp && !d.batch_warp[li] && d.batch_lanes && d.batch_lanes[li] > 0 && alt)
+          e = launch_update_mb<T>(d.batch_lanes[li], g, nb, s, prio, d, Lx, L.off, bt);
         else if (small)
           e = launch_prio(k_update_flat<T, SMALL_TB, false>, dim3(g, nb), TS, 0, s, prio, d.sn, d.upd_tasks,
                           d.upd_entries, d.rel, Lx, L.off, bt);
@@ -2882,12 +2892,12 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
                           d.upd_entries, d.rel, Lx, L.off, bt);
         break;
       case K_POTRF:
-        // small tiles of a batch: a warp per tile (throughput); of one matrix: a CTA per tile, whose
+        // small tiles of a large batch: a warp per tile (throughput); otherwise a CTA per tile, whose
         // four warps shorten each column step of the tile (latency; 64^2 factor 0.96 -> 0.83 ms);
         // the autotuner's choice (alt) swaps the two
         if (panel == PANEL_FUSED)
           e = launch_panel_b<T>(d, d.batch_panel[li], g, nb, s, prio, Lx, Linv, status, L.off, bt);
-        else if (small && (nb > 1) != alt)
+        else if (small && (nb > 1 && (int64_t)g * nb > BATCH_CTA_POTRF) != alt)
           e = launch_prio(k_potrf_w<T>, dim3((g + WT_WARPS - 1) / WT_WARPS, nb), 32 * WT_WARPS, 0, s, prio, d.sn,
                           d.tasks, (int64_t)g, Lx, status, d.piv, d.axc, d.dpos, L.off, bt);
         else if (small)
@@ -2903,10 +2913,8 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
                           d.dpos, L.off, bt);
         break;
       case K_TRSM:
-        // (a warp-per-tile form with the column pairs mapped flat onto the lanes made the
-        // 512 x 128^2 batch's TRSM slower, 11.0 -> 16.3 ms: its tiles have enough rows; the
-        // warp-per-(tile, matrix) form is the autotuner's alternative)
-        if (small && nb > 1 && alt)
+        // small tiles of a large batch: a warp per (tile, matrix) (the alternative the other way round)
+        if (small && nb > 1 && ((int64_t)g * nb > BATCH_CTA_TRSM) != alt)
           e = launch_prio(k_trsm_w<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, trsm_w_smem<T>(), s,
                           prio, d.sn, d.tasks, Lx, L.off, (int32_t)nb, bt);
         else if (small)
@@ -2934,7 +2942,7 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
           e = launch_prio(k_gemm_f32, dim3(g, nb), F32_THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
         break;
       case K_TRTRI:
-        if (small && (nb > 1) != alt)  // (as for POTRF)
+        if (small && (nb > 1 && (int64_t)g * nb > BATCH_CTA_TRTRI) != alt)  // (as for POTRF)
           e = launch_prio(k_trtri_w<T>, dim3((g + WT_WARPS - 1) / WT_WARPS, nb), 32 * WT_WARPS, 0, s, prio, d.sn,
                           d.tasks, (int64_t)g, (const T *)Lx, Linv, L.off, bt);
         else

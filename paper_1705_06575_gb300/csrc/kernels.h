@@ -135,13 +135,13 @@ cudaError_t launch_gemm_oz(unsigned tasks, cudaStream_t st, int prio, const DevP
                            long long *status);
 
 // Whether a factor launch has a second kernel form (the autotuner times both). A batch
-// (nbatch > 1): FP64 updates with lanes mapped to matrices (default for small tiles and for full
-// tiles with small entries, DevPlan::batch_warp) against one warp per (tile, matrix) (small tiles;
-// full tiles with small entries, in global memory) or one CTA per tile and matrix (the default of
-// full tiles with large entries); small-tile POTRF, TRSM and TRTRI, one warp per (tile, matrix)
-// or one CTA per tile and matrix. One matrix: clustered FP64 updates or one CTA per tile; FP32
-// full-tile updates on the tensor cores or the SIMT pipes; small-tile POTRF and TRTRI, one CTA or
-// one warp per tile. fp64: the factor's precision.
+// (nbatch > 1): FP64 small-tile updates with lanes mapped to matrices or one warp per (tile, matrix);
+// FP64 full-tile updates with one warp per (tile, matrix) in global memory (small entries,
+// DevPlan::batch_warp) or lanes mapped to matrices (large ones), against one CTA per tile and matrix;
+// small-tile POTRF, TRSM and TRTRI, one warp per (tile, matrix) or one CTA (which of two forms is the
+// default depends on the number of pairs, BATCH_* in plan.h). One matrix: FP64 updates on the tensor
+// cores or clustered, against one CTA per tile; FP32 full-tile updates on the tensor cores or the
+// SIMT pipes; small-tile POTRF and TRTRI, one CTA or one warp per tile. fp64: the factor's precision.
 bool factor_launch_has_alternative(const Launch &L, int32_t nbatch, bool fp64);
 
 // Numeric factorization: scatter A into the zeroed panels, then run the launch schedule.

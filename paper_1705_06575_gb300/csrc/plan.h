@@ -76,6 +76,26 @@ inline int panel_lanes_for(const PanelForm &pf, unsigned nb, bool f32) {
   if (nb > 1) return panel_lanes(pf.pmax, pf.ncmax, f32);
   return panel_smem_bytes(pf.pmax, pf.ncmax, f32, 32) <= PANEL_SMEM_HARD ? 32 : 0;
 }
+// Whether a batch runs a narrow level as separate launches before the autotuner has timed it: the
+// panels need more than the soft limit (512 x 128^2 9-point batch, its two such levels: 1.46 and
+// 0.63 ms apart against 1.72 and 0.72 ms fused), or there are too few warps to hide each one's
+// column chain (128 x 64^2, 5 supernodes: 0.05 against 0.12 ms; 64 x 100^2, 16 supernodes: 0.05
+// against 0.08 ms; 34 supernodes, 544 warps: fused is faster).
+constexpr int64_t BATCH_PANEL_WARPS = 2 * 152;
+inline bool batch_level_apart(const PanelForm &pf, int64_t count, unsigned nb, bool f32) {
+  const int g = panel_lanes(pf.pmax, pf.ncmax, f32);
+  if (g == 0 || panel_smem_bytes(pf.pmax, pf.ncmax, f32, g) > PANEL_SMEM_SOFT) return true;
+  return count * (int64_t)((nb + 32 / g - 1) / (32 / g)) < BATCH_PANEL_WARPS;
+}
+// Batches: up to this many (tile, matrix) pairs of a launch latency counts and a pair gets more
+// threads. Full-tile updates with small entries: a CTA per pair instead of a warp (128 x 64^2 grids,
+// 256 pairs of 31 entries: 0.12 against 0.43 ms; 64 x 100^2, 1536 pairs: 0.23 against 0.31 ms, 2816
+// pairs: equal). Small-tile updates: a warp per pair instead of lanes = matrices (20 x 24^2, 160 pairs:
+// 0.03 against 0.10 ms; 8192 pairs: equal). Small-tile POTRF: a CTA instead of a warp (512 x 128^2, 4608
+// pairs: 0.15 against 0.19 ms); TRTRI the same (128 pairs: 0.027 against 0.045 ms, 2048 pairs: 0.072
+// against 0.035 ms) and TRSM (2176 pairs: 0.062 against 0.049 ms, 2048: equal).
+constexpr int64_t BATCH_CTA_UPDATE = 2048, BATCH_WARP_UPDATE = 4096, BATCH_CTA_POTRF = 6000, BATCH_CTA_TRTRI = 1024,
+                  BATCH_CTA_TRSM = 2048;
 inline int solve_lanes_for(const PanelForm &pf, unsigned nb, bool fp64) {
   if (nb > 1) return fp64 ? solve_panel_lanes(pf.pmax, pf.ncmax) : 0;
   return solve_panel_bytes(pf.pmax, pf.ncmax, 32, 8) <= PANEL_SMEM_HARD ? 32 : 0;
@@ -228,7 +248,8 @@ struct Plan {
                                       // or 8), else 0
   std::vector<PanelForm> batch_panel;  // per factor launch: fused narrow levels (batches and,
                                        // where panel_apart[0] allows, single matrices)
-  std::vector<int8_t> panel_apart[2];  // per factor launch, on PANEL_FUSED ones: 1 if the
+  std::vector<int8_t> panel_apart[2];  // per factor launch, on PANEL_FUSED ones (-1 for batches:
+                                       // not timed, batch_level_apart decides): 1 if the
                                        // autotuner found the level faster as separate launches;
                                        // [0] one matrix, [1] batches
   // Per factor launch of one FP64 matrix: nonzero if the launch runs on the tensor cores (K_UPDATE:

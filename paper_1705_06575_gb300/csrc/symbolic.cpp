@@ -984,7 +984,7 @@ int analyze(int64_t n, const int64_t *Ap, const int32_t *Ai, const int32_t *perm
   // launch (k_panel_b; a batch only where the panels fit, see panel_lanes). Such a level has one
   // launch of each (one column tile, all of it small-tile).
   P.batch_panel.assign(P.factor_launches.size(), PanelForm{PANEL_NONE, 0, 0, -1});
-  for (auto &v : P.panel_apart) v.assign(P.factor_launches.size(), 0);
+  for (int c = 0; c < 2; ++c) P.panel_apart[c].assign(P.factor_launches.size(), (int8_t)-c);
   for (int32_t l = 0; l < nlev; ++l) {
     int64_t pmax = 0, ncmax = 0;
     bool narrow = P.levelptr[l + 1] > P.levelptr[l];
