@@ -118,25 +118,32 @@ __device__ __forceinline__ double rsqrt_delta(double d) {
   return fma(x0 * e, fma(0.375, e, 0.5), x0);
 }
 
-// Diagonal tile s of J: 46 us for 64 columns, as the FP64 kernel (44 us); it is bound by the column
-// chain (800 cycles per column in the owner's registers, of which the reciprocal takes half) and
-// the integer multiply-adds of the trailing blocks (1.3k cycles per block). What it gives is the
-// panel solve's operands uh, sg and 1 / sqrt(delta), which the solve (20 us for 32 rows, 55 us with
-// FP64 and a launch for the digits) would otherwise derive in every CTA (38 us).
-// Columns go in blocks of four; warp w owns blocks w and w + 8, lane l rows l
-// and l + 32. Step b, one barrier: the owner of block b factors it (its own columns updated from
-// registers through shuffles), publishes yh and uh, and every warp adds the four columns to its
-// blocks right of them, the owner of block b + 1 that block first.
+// Diagonal tile s of J (33 to 64 columns), 16 warps. Columns go in blocks of four. Warp w of the first
+// eight owns block w at the rows 0-31, warp w of the other eight blocks w and w + 8 at the rows 32-63
+// (one row per lane). A block's owner at the rows that hold its diagonal factors it in registers (its
+// own columns updated through shuffles) and publishes yh, uh and 1 / delta; the other warps then add
+// its columns to their blocks. While the upper rows walk the first eight blocks, the lower rows follow
+// one block behind, so the pivots' chain carries the work of one row per lane only; named barriers
+// link each group's steps and hand the upper blocks to the lower group. (With both rows in one lane and
+// one barrier for all, 46 us for 64 columns: 800 cycles per column; the FP64 kernel 44 us.)
 constexpr size_t POTRF_SMEM = 2 * NB * NB * sizeof(int2);
+constexpr int POTRF_Z_THREADS = 512;
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void bar_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
-__global__ void __launch_bounds__(Z_THREADS) k_potrf_z(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
-                                                       double *__restrict__ Lx, const int32_t *__restrict__ exps,
-                                                       int2 *__restrict__ zu, ZCol *__restrict__ zc,
-                                                       long long *status, int64_t toff) {
+__global__ void __launch_bounds__(POTRF_Z_THREADS) k_potrf_z(const SNode *__restrict__ sn,
+                                                             const Int4 *__restrict__ tasks, double *__restrict__ Lx,
+                                                             const int32_t *__restrict__ exps, int2 *__restrict__ zu,
+                                                             ZCol *__restrict__ zc, long long *status, int64_t toff) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int2(*ys)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw);                           // [c][row]: -yh
   int2(*us)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw + NB * NB * sizeof(int2));  // [c][row]: uh
   __shared__ int64_t dd[NB];  // delta / 4 of every column, unit 2^-60
+  __shared__ int2 rhos[NB];   // 1 / delta, halves
   __shared__ ZCol col[NB];
   const Int4 t = tasks[toff + blockIdx.x];
   const SNode sj = sn[t.a];
@@ -145,142 +152,130 @@ __global__ void __launch_bounds__(Z_THREADS) k_potrf_z(const SNode *__restrict__
   const int64_t ld = sj.nrows, g0 = sj.first + (int64_t)s * NB;
   double *D = Lx + sj.lx + (int64_t)(s * NB) * ld + s * NB;
   const int32_t *ec = exps + g0;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int64_t hi[2][4][2], mid[2][4][2];  // [slot][column][row half]
+  const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 7, low = tid >> 8;  // low: rows 32-63
+  const int row = lane + 32 * low;
+  int64_t hi[2][4], mid[2][4];  // [block w, block w + 8][column]
 #pragma unroll
   for (int q = 0; q < 2; ++q)
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int c = 4 * (warp + 8 * q) + k, r = lane + 32 * h;
-        int64_t v = 0;
-        if (r >= c && r < ts) {
-          const double x = D[(int64_t)c * ld + r];
-          v = r == c && !(x > 0.0) ? -(1ll << 58) : oz::to_fixed60(x, ec[r] + ec[c]);
-        }
-        hi[q][k][h] = v;
-        mid[q][k][h] = 0;
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * (w + 8 * q) + k;
+      int64_t v = 0;
+      if (row >= c && row < ts) {
+        const double x = D[(int64_t)c * ld + row];
+        v = row == c && !(x > 0.0) ? -(1ll << 58) : oz::to_fixed60(x, ec[row] + ec[c]);
       }
+      hi[q][k] = v;
+      mid[q][k] = 0;
+    }
   const int nblk = (ts + 3) >> 2;
-  int bn = warp;  // the block in slot 0
-  // block bn + 8 q += the columns of block b. A diagonal entry below -1 stays there: its row fails as a
-  // pivot, and further squares (at most 4 per block) must not wrap around 8 to a positive value.
-  auto mac = [&](int q, int b, const int2 (&y)[4][2]) {
-    const int c0 = 4 * (bn + 8 * q);
+  // this warp's block at q += the columns of block b. A diagonal entry below -1 stays there: its row
+  // fails as a pivot, and further squares (at most 4 per block) must not wrap around 8 to a positive
+  // value.
+  auto mac = [&](auto qc, int b) {
+    constexpr int q = decltype(qc)::value;
+    const int c0 = 4 * (w + 8 * q);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
+      const int2 y = ys[4 * b + j][row];
       const int4 p0 = *reinterpret_cast<const int4 *>(&us[4 * b + j][c0]);
       const int4 p1 = *reinterpret_cast<const int4 *>(&us[4 * b + j][c0 + 2]);
-      const int2 u[4] = {make_int2(p0.x, p0.y), make_int2(p0.z, p0.w), make_int2(p1.x, p1.y), make_int2(p1.z, p1.w)};
-      if (c0 < 32) {  // (rows 0-31 of later columns are above the diagonal)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) z_mac(hi[q][k][0], mid[q][k][0], y[j][0], u[k]);
-      }
-#pragma unroll
-      for (int k = 0; k < 4; ++k) z_mac(hi[q][k][1], mid[q][k][1], y[j][1], u[k]);
+      z_mac(hi[q][0], mid[q][0], y, make_int2(p0.x, p0.y));
+      z_mac(hi[q][1], mid[q][1], y, make_int2(p0.z, p0.w));
+      z_mac(hi[q][2], mid[q][2], y, make_int2(p1.x, p1.y));
+      z_mac(hi[q][3], mid[q][3], y, make_int2(p1.z, p1.w));
     }
+    if (q == low) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      int64_t &v = c0 < 32 ? hi[q][k][0] : hi[q][k][1];
-      if (lane == ((c0 + k) & 31) && v < -(1ll << 60)) v = -(1ll << 60);
+      for (int k = 0; k < 4; ++k)
+        if (row == c0 + k && hi[q][k] < -(1ll << 60)) hi[q][k] = -(1ll << 60);
     }
   };
-  auto factor = [&](int b) {  // the owner of block b (slot 0)
+  // One column of this warp's rows, given its pivot data: yh and uh, and the block's later columns.
+  auto column = [&](auto qc, int b, int k, int64_t v, int2 rho, int sg, auto &&ucol) {
+    constexpr int q = decltype(qc)::value;
+    const int c = 4 * b + k;
+    const int64_t yh = (int64_t)((uint64_t)v << sg);
+    const int2 y = oz::split30(yh), ny = make_int2(-y.x, -y.y), u = oz::split30(oz::mul60(y, rho));
+#pragma unroll
+    for (int k2 = 1; k2 < 4; ++k2)
+      if (k2 > k) z_mac(hi[q][k2], mid[q][k2], ny, ucol(u, 4 * b + k2));
+    ys[c][row] = ny;
+    us[c][row] = u;
+  };
+  // Block b at the rows that hold its diagonal (its owner warp).
+  auto factor = [&](auto qc, int b) {
+    constexpr int q = decltype(qc)::value;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const int c = 4 * b + k;
-      if (c >= ts) {  // (uniform) columns past the tile contribute nothing
-        ys[c][lane] = ys[c][lane + 32] = us[c][lane] = us[c][lane + 32] = make_int2(0, 0);
+      if (q == 1 && c >= ts) {  // (uniform) columns past the tile contribute nothing
+        ys[c][row] = us[c][row] = make_int2(0, 0);
         continue;
       }
-      const int64_t v0 = z_value(hi[0][k][0], mid[0][k][0]), v1 = z_value(hi[0][k][1], mid[0][k][1]);
-      int64_t d = shfl64(c < 32 ? v0 : v1, c & 31);
+      int64_t v = z_value(hi[q][k], mid[q][k]);
+      int64_t d = shfl64(v, c & 31);
       if (d <= 0) {
         if (lane == 0) atomicMin(status, (long long)(g0 + c));
         d = 1ll << 59;
       }
       const int sg = (61 - (63 - __clzll(d))) >> 1;
       const int64_t dq = (int64_t)((uint64_t)d << (2 * sg - 2));  // delta / 4
-      const int2 rho = oz::split30(oz::reciprocal60(dq));
       float root;  // sqrt(delta) = l_cc 2^sg, to a few parts in 10^6
       asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"((float)(int)(dq >> 36) * (4.0f / 16777216.0f)));
       const int64_t lim = (int64_t)__float2int_rn(root * (0.9999f * 536870912.0f)) << (31 - sg);
+      const int2 rho = oz::split30(oz::reciprocal60(dq));
+      v = v > lim ? lim : v < -lim ? -lim : v;
+      v = row == c ? d : row > c ? v : 0;
+      column(qc, b, k, v, rho, sg, [&](int2 u, int c2) {
+        return make_int2(__shfl_sync(0xffffffffu, u.x, c2 & 31), __shfl_sync(0xffffffffu, u.y, c2 & 31));
+      });
       if (lane == 0) {
         dd[c] = dq;
+        rhos[c] = rho;
         col[c].sg = sg;
         col[c].lim = lim;
       }
-      int2 ny[2], u[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = lane + 32 * h;
-        int64_t v = h ? v1 : v0;
-        v = v > lim ? lim : v < -lim ? -lim : v;
-        v = r == c ? d : r > c ? v : 0;
-        const int64_t yh = (int64_t)((uint64_t)v << sg);
-        ny[h] = oz::split30(-yh);
-        u[h] = oz::split30(oz::mul60(oz::split30(yh), rho));
-        ys[c][r] = ny[h];
-        us[c][r] = u[h];
-      }
-#pragma unroll
-      for (int k2 = k + 1; k2 < 4; ++k2) {
-        const int c2 = 4 * b + k2;
-        const int2 w = c2 < 32 ? u[0] : u[1];
-        const int2 uc = make_int2(__shfl_sync(0xffffffffu, w.x, c2 & 31), __shfl_sync(0xffffffffu, w.y, c2 & 31));
-#pragma unroll
-        for (int h = 0; h < 2; ++h) z_mac(hi[0][k2][h], mid[0][k2][h], ny[h], uc);
-      }
     }
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        hi[0][k][h] = hi[1][k][h];
-        mid[0][k][h] = mid[1][k][h];
-      }
-    bn += 8;
   };
-  if (warp == 0 && nblk > 0) factor(0);
-  __syncthreads();
-  for (int b = 0; b + 1 < nblk; ++b) {
-    if (bn < nblk) {
-      int2 y[4][2];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        y[j][0] = ys[4 * b + j][lane];
-        y[j][1] = ys[4 * b + j][lane + 32];
+  using Q0 = std::integral_constant<int, 0>;
+  using Q1 = std::integral_constant<int, 1>;
+  // barriers: 1 the upper rows' steps, 2 the lower rows', 3 + b hands block b to the lower rows
+  if (!low) {
+    for (int b = 0; b < 8; ++b) {
+      if (w == b) {
+        factor(Q0(), b);
+        bar_arrive(3 + b, 32 + 256);
       }
-      const bool two = bn + 8 < nblk && bn < 8;  // slot 1 holds a block as well
-      mac(0, b, y);
-      if (b == 7) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int h = 0; h < 2; ++h) z_fold(hi[0][k][h], mid[0][k][h]);
-      }
-      if (bn == b + 1) {  // (warp-uniform)
-        factor(b + 1);    // moves slot 1 to slot 0
-        if (two) mac(0, b, y);
-        if (two && b == 7) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) z_fold(hi[0][k][h], mid[0][k][h]);
-        }
-      } else if (two) {
-        mac(1, b, y);
-        if (b == 7) {
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int h = 0; h < 2; ++h) z_fold(hi[1][k][h], mid[1][k][h]);
-        }
-      }
+      bar_sync(1, 256);
+      if (w > b) mac(Q0(), b);
     }
-    __syncthreads();
+  } else {
+    for (int b = 0; b < 8; ++b) {
+      bar_sync(3 + b, 32 + 256);
+      if (w == b) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const int c = 4 * b + k;
+          const int64_t lim = col[c].lim;
+          int64_t v = z_value(hi[0][k], mid[0][k]);
+          v = v > lim ? lim : v < -lim ? -lim : v;
+          column(Q0(), b, k, v, rhos[c], col[c].sg, [&](int2, int c2) { return us[c][c2]; });
+        }
+      }
+      bar_sync(2, 256);
+      if (w > b) mac(Q0(), b);
+      mac(Q1(), b);
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) z_fold(hi[1][k], mid[1][k]);
+    for (int b = 8; b < nblk; ++b) {
+      if (w == b - 8) factor(Q1(), b);
+      bar_sync(2, 256);
+      if (w > b - 8) mac(Q1(), b);
+    }
   }
+  __syncthreads();
   if (tid < ts) {
     const double lam = rsqrt_delta((double)dd[tid] * (4.0 / 1152921504606846976.0));
     col[tid].lam = oz::split30(__double2ll_rn(lam * 1152921504606846976.0));
@@ -289,7 +284,7 @@ __global__ void __launch_bounds__(Z_THREADS) k_potrf_z(const SNode *__restrict__
   __syncthreads();
   // the tile in FP64 and uh for its panel solves
   int2 *zt = zu + sj.dx + (int64_t)s * NB * NB;
-  for (int idx = tid; idx < ts * NB; idx += Z_THREADS) {
+  for (int idx = tid; idx < ts * NB; idx += POTRF_Z_THREADS) {
     const int r = idx & (NB - 1), c = idx / NB;
     if (r >= ts) continue;
     double x = 0.0;
@@ -1019,7 +1014,7 @@ cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const Dev
 size_t oz_column_bytes() { return sizeof(ZCol); }
 cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
                            long long *status) {
-  return launch_oz(k_potrf_z, tasks, Z_THREADS, POTRF_SMEM, 1, st, prio, d.sn, d.tasks, Lx, (const int32_t *)d.exps,
+  return launch_oz(k_potrf_z, tasks, POTRF_Z_THREADS, POTRF_SMEM, 1, st, prio, d.sn, d.tasks, Lx, (const int32_t *)d.exps,
                    d.zu, (ZCol *)d.zc, status, toff);
 }
 cudaError_t launch_trsm_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff) {
