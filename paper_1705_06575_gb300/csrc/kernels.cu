@@ -1419,8 +1419,8 @@ __global__ void __launch_bounds__(TileCfg<TB>::threads) k_bstep(const SNode *__r
 }
 
 // Cluster forms of the solve steps (tiles of up to NB columns). A task {J, i, s} runs on a
-// thread-block cluster of four CTAs; CTA q of the cluster owns the 16 rows (forward) or columns
-// (backward) 16 q .. 16 q + 15 of tile i. Forward, launch s (s = -1 .. ncb - 2):
+// thread-block cluster of four or eight CTAs (StepCfg); CTA q of the cluster owns the rows (forward)
+// or columns (backward) QR q .. QR q + QR - 1 of tile i. Forward, launch s (s = -1 .. ncb - 2):
 //   every task applies the solved tile s (if s >= 0) to its rows: y_i -= L_is y_s;
 //   the task i = s + 1 then solves its tile in place, y_i <- L_ii^{-1} y_i, each CTA taking its
 //   16 rows of the inverse and the whole updated tile, gathered from the four CTAs through
@@ -1429,15 +1429,32 @@ __global__ void __launch_bounds__(TileCfg<TB>::threads) k_bstep(const SNode *__r
 // z_i <- L_ii^{-T} z_i. So the tile a step solves is written once, already solved, and read by
 // the next launch only: no CTA applies the inverse of another tile, and the critical path of a
 // step is one quarter tile's update plus one quarter of its solve.
-constexpr int QR = 16;  // rows (or columns) per CTA of a cluster task
+//
+// A warp-wide FP64 instruction takes its sub-partition's pipe for 64 cycles. With two or more right-
+// hand sides the FP64 kernel therefore gives every thread one output (row, right-hand side) and a
+// share of k, so that only the few shares are added up (through shared memory), and spreads a task
+// over eight CTAs of eight rows; with one, and in FP32, sixteen lanes share an output and add up by
+// shuffles, four CTAs per task. (With shuffles for 8 right-hand sides 32 of 64 FP64 instructions per
+// warp and product were additions of partial sums. 48^3 7-point solve: 8 right-hand sides 7.6 -> 5.0 ms,
+// 4 right-hand sides 4.15 -> 3.0 ms.)
+template <typename V, int NR>
+struct StepCfg {
+  static constexpr bool split = sizeof(V) == 8 && NR >= 2;
+  static constexpr int CS = split ? 8 : 4;       // CTAs per cluster task
+  static constexpr int QR = NB / CS;             // rows (or columns) per CTA
+  static constexpr int NP = NR <= 4 ? 4 : 8;     // right-hand sides, padded (split)
+  static constexpr int KS = THREADS / (QR * NP); // shares of k (split)
+};
 
 template <typename V, int NR>
 struct StepCSmem {
+  static constexpr int QR = StepCfg<V, NR>::QR;
   V L[NB][QR + 1];     // [k][row]: this CTA's rows of L_is (forward) or L_si^T (backward)
   V I[NB][QR + 1];     // [k][row]: this CTA's rows of L_ii^{-1} (forward) or of L_ii^{-T}
   V ys[NR][NB];        // the solved tile s
   V yq[NR][QR];        // this CTA's rows of tile i after the update (read by the cluster)
   V yf[NR][NB];        // the whole updated tile i (solving tasks)
+  V part[StepCfg<V, NR>::split ? THREADS : 1];  // the shares' sums
 };
 
 // 16-lane sum (lanes l and l ^ 8, ^4, ^2, ^1 are partners; lane g of each 16 holds part g).
@@ -1456,11 +1473,13 @@ __global__ void __launch_bounds__(THREADS) k_step_c(const SNode *__restrict__ sn
   Lx += blockIdx.y * bt.lx;
   Linv += blockIdx.y * bt.dinv;
   y += blockIdx.y * bt.y;
+  using Cfg = StepCfg<V, NR>;
+  constexpr int QR = Cfg::QR;
   __shared__ StepCSmem<V, NR> S;
   cg::cluster_group cluster = cg::this_cluster();
   pdl_trigger_early<V>();
   const int q = (int)cluster.block_rank();
-  const Int4 t = tasks[toff + blockIdx.x / 4];
+  const Int4 t = tasks[toff + blockIdx.x / Cfg::CS];
   const SNode sj = sn[t.a];
   const int i = t.b, s = t.c;
   const int ti = min(NB, sj.ncols - i * NB);
@@ -1506,51 +1525,85 @@ __global__ void __launch_bounds__(THREADS) k_step_c(const SNode *__restrict__ sn
     if (has_s && k < ts) S.ys[c][k] = y[(int64_t)(r0 + c) * n + gs + k];
   }
   __syncthreads();
-  // y_i(o) -= sum_k L(o, k) ys(k) for this CTA's outputs o: 16 lanes per output split k.
-  V acc[NR];
+  if constexpr (Cfg::split) {
+    // thread (row po, right-hand side pc, share pk of k); threads below QR * NP finish the outputs
+    const int po = tid % QR, pc = (tid / QR) % Cfg::NP, pk = tid / (QR * Cfg::NP);
+    auto product = [&](const V(&M)[NB][QR + 1], const V(&x)[NR][NB], int lo, int hi) -> V {
+      V a = V(0);
+      if (pc < NR)
+        for (int k = lo + ((pk - lo) & (Cfg::KS - 1)); k < hi; k += Cfg::KS) a = fma(M[k][po], x[pc][k], a);
+      S.part[tid] = a;
+      __syncthreads();
+      if (pk == 0 && pc < NR)
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = V(0);
-  if (o < QR) {
-    for (int k = g; k < ts; k += 16) {
-      const V l = S.L[k][o];
-#pragma unroll
-      for (int c = 0; c < NR; ++c) acc[c] = fma(l, S.ys[c][k], acc[c]);
+        for (int j = 1; j < Cfg::KS; ++j) a += S.part[tid + j * QR * Cfg::NP];
+      return a;
+    };
+    const bool out = pk == 0 && pc < NR && po < rq;
+    const int64_t at = (int64_t)(r0 + pc) * n + gi + o0 + po;
+    const V old = out ? y[at] : V(0);
+    const V v = old - product(S.L, S.ys, 0, ts);
+    if (!solves) {
+      if (out) y[at] = v;
+      return;  // (uniform across the cluster: its CTAs share the task)
     }
-  }
-#pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = sum16(acc[c]);
-  if (g == 0 && o < rq) {
-#pragma unroll
-    for (int c = 0; c < NR; ++c) {
-      const int64_t at = (int64_t)(r0 + c) * n + gi + o0 + o;
-      const V v = y[at] - acc[c];
-      if (solves) S.yq[c][o] = v;
-      else y[at] = v;
+    if (out) S.yq[pc][po] = v;
+    cluster.sync();  // every part of the updated tile is in its CTA's shared memory
+    for (int idx = tid; idx < NR * ti; idx += THREADS) {
+      const int k = idx % ti, c = idx / ti;
+      const V *rem = cluster.map_shared_rank(&S.yq[0][0], k / QR);
+      S.yf[c][k] = rem[c * QR + k % QR];
     }
-  }
-  if (!solves) return;  // (uniform across the cluster: its four CTAs share the task)
-  cluster.sync();       // every quarter of the updated tile is in its CTA's shared memory
-  for (int idx = tid; idx < NR * ti; idx += THREADS) {
-    const int k = idx % ti, c = idx / ti;
-    const V *rem = cluster.map_shared_rank(&S.yq[0][0], k / QR);
-    S.yf[c][k] = rem[c * QR + k % QR];
-  }
-  __syncthreads();
+    __syncthreads();
+    const V x = product(S.I, S.yf, FWD ? 0 : o0 + po, FWD ? min(ti, o0 + po + 1) : ti);  // the inverse's nonzeros
+    if (out) y[at] = x;
+  } else {
+    // y_i(o) -= sum_k L(o, k) ys(k) for this CTA's outputs o: 16 lanes per output split k.
+    V acc[NR];
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = V(0);
-  if (o < QR) {
-    const int lo = FWD ? 0 : o0 + o, hi = FWD ? o0 + o + 1 : ti;  // the inverse's nonzeros
-    for (int k = lo + ((g - lo) & 15); k < hi; k += 16) {
-      const V l = S.I[k][o];
+    for (int c = 0; c < NR; ++c) acc[c] = V(0);
+    if (o < QR) {
+      for (int k = g; k < ts; k += 16) {
+        const V l = S.L[k][o];
 #pragma unroll
-      for (int c = 0; c < NR; ++c) acc[c] = fma(l, S.yf[c][k], acc[c]);
+        for (int c = 0; c < NR; ++c) acc[c] = fma(l, S.ys[c][k], acc[c]);
+      }
     }
-  }
 #pragma unroll
-  for (int c = 0; c < NR; ++c) acc[c] = sum16(acc[c]);
-  if (g == 0 && o < rq) {
+    for (int c = 0; c < NR; ++c) acc[c] = sum16(acc[c]);
+    if (g == 0 && o < rq) {
 #pragma unroll
-    for (int c = 0; c < NR; ++c) y[(int64_t)(r0 + c) * n + gi + o0 + o] = acc[c];
+      for (int c = 0; c < NR; ++c) {
+        const int64_t at = (int64_t)(r0 + c) * n + gi + o0 + o;
+        const V v = y[at] - acc[c];
+        if (solves) S.yq[c][o] = v;
+        else y[at] = v;
+      }
+    }
+    if (!solves) return;  // (uniform across the cluster: its four CTAs share the task)
+    cluster.sync();       // every quarter of the updated tile is in its CTA's shared memory
+    for (int idx = tid; idx < NR * ti; idx += THREADS) {
+      const int k = idx % ti, c = idx / ti;
+      const V *rem = cluster.map_shared_rank(&S.yq[0][0], k / QR);
+      S.yf[c][k] = rem[c * QR + k % QR];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NR; ++c) acc[c] = V(0);
+    if (o < QR) {
+      const int lo = FWD ? 0 : o0 + o, hi = FWD ? o0 + o + 1 : ti;  // the inverse's nonzeros
+      for (int k = lo + ((g - lo) & 15); k < hi; k += 16) {
+        const V l = S.I[k][o];
+#pragma unroll
+        for (int c = 0; c < NR; ++c) acc[c] = fma(l, S.yf[c][k], acc[c]);
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NR; ++c) acc[c] = sum16(acc[c]);
+    if (g == 0 && o < rq) {
+#pragma unroll
+      for (int c = 0; c < NR; ++c) y[(int64_t)(r0 + c) * n + gi + o0 + o] = acc[c];
+    }
   }
   cluster.sync();  // keep this CTA's quarter alive until the others have read it
 }
@@ -2548,10 +2601,10 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int threads, size_t 
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
-// Launch of a cluster-form solve step: clusters of four CTAs along x, programmatic dependent
-// launch (see pdl_wait).
+// Launch of a cluster-form solve step: clusters of cs CTAs along x, programmatic dependent launch
+// (see pdl_wait).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_step_c(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, Args... args) {
+cudaError_t launch_step_c(void (*kernel)(KArgs...), int cs, dim3 grid, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[2];
   cfg.gridDim = grid;
@@ -2559,7 +2612,7 @@ cudaError_t launch_step_c(void (*kernel)(KArgs...), dim3 grid, cudaStream_t st, 
   cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = 4;
+  attr[0].val.clusterDim.x = (unsigned)cs;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -3056,7 +3109,8 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
             break;
           }
           if (L.cluster == 4) {
-            SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, true>, dim3(4 * g, nb), st, d.sn, d.tasks, Lx,
+            SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, true>, StepCfg<V, NR>::CS,
+                                                   dim3(StepCfg<V, NR>::CS * g, nb), st, d.sn, d.tasks, Lx,
                                                    Linv, y, n, r0, L.off, bt)));
             break;
           }
@@ -3122,7 +3176,8 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
             break;
           }
           if (L.cluster == 4) {
-            SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, false>, dim3(4 * g, nb), st, d.sn, d.tasks, Lx,
+            SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, false>, StepCfg<V, NR>::CS,
+                                                   dim3(StepCfg<V, NR>::CS * g, nb), st, d.sn, d.tasks, Lx,
                                                    Linv, y, n, r0, L.off, bt)));
             break;
           }
