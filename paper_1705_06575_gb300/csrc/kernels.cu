@@ -8,8 +8,8 @@
 //       tc_update.cu);
 //   (b) dense Cholesky of the diagonal block — k_potrf (per diagonal tile; k_potrf_r for FP32
 //       tiles of order NB) and
-//   (c) dense triangular solves on the rows below it — k_trsm (k_trsm_r for FP32 tiles of
-//       NB columns), with k_gemm applying the
+//   (c) dense triangular solves on the rows below it — k_trsm (k_trsm_f, k_trsm_r for full
+//       tiles), with k_gemm applying the
 //       trailing updates inside J when J is wider than one tile.
 // Supernodes of one level of the supernodal tree are independent and run in the same launches.
 // The solve follows Sec. 3.1: diagonal block first, then the off-diagonal part; the forward
@@ -653,16 +653,166 @@ __global__ void __launch_bounds__(TileCfg<TB>::threads) k_trsm(const SNode *__re
   }
 }
 
-// (b') FP32 diagonal tiles of order up to NB with the column chain in registers. Warp w of the
-// first eight owns the columns w, w + 8, ... (lane l: rows l and l + 32 of each), the oldest
-// unfinished one in v[0]; a column is published in shared memory once final. Step c, one barrier:
-// the owner of column c applies column c - 1 to it, takes the FP64 pivot, scales the column and
-// publishes it; every owner applies column c - 1 to its other columns right of it; warp 8
-// subtracts l(k, c - 1)^2 from the FP64 diagonal of the rows k > c. Every element and every pivot
-// sees the operations of k_potrf in the same order, so the factors are bit-identical; what
-// changes is that the trailing columns stay in registers (k_potrf looks up a packed index and
-// goes through shared memory for every update, and its barrier waits for those chains).
-constexpr int PR_OWNERS = 8, PR_THREADS = 32 * (PR_OWNERS + 1);
+// (b') FP32 diagonal tiles of order up to NB, columns in blocks of four. Warp w owns the blocks w and
+// w + 8 (lane l: rows l and l + 32 of each column), the older one in slot 0. Step b, one barrier: the
+// owner of block b factors it in registers (its own columns through shuffles) and publishes it, and
+// every warp applies it to its blocks right of it, the owner of block b + 1 to that block first. Lanes
+// 0-7 of a warp carry the FP64 diagonal of its eight columns (lane 4 q + k: column k of slot q): each
+// applied column subtracts l^2 there. Every element sees the operations of k_potrf in the same order.
+// The chain of the 64 columns bounds it, and the FP64 pipe was its longest part: a warp's operation on
+// it takes 64 cycles, conversions too, whatever the number of active lanes (30 us per 64-column tile,
+// 34 us with one barrier per column, 25 us with integers). So the diagonals are held as 64-bit integers (FIX): unit 2^(E-60)
+// for a diagonal in [2^E, 2^(E+1)), where the square of an FP32 number is exact before one shift and
+// the error per column, 2^-60 of the diagonal, is below that of an FP64 subtraction. A tile with a
+// diagonal that is not positive and finite, or whose E is outside [-60, 100], takes FP64 throughout.
+constexpr int PR_THREADS = 256, PR_LD = NB + 4;
+
+// d - l^2 in units of 2^(E-60); a square beyond 2^61 units (or of Inf, NaN) leaves a negative number, and
+// negative numbers stay negative.
+__device__ __forceinline__ long long sub_square(long long d, float l, int E) {
+  const unsigned u = __float_as_uint(l);
+  const unsigned m = (u & 0x7fffffu) | 0x800000u;
+  const int n = 254 + E - 2 * (int)((u >> 23) & 0xff);  // l^2 = m^2 2^14 units >> n; l = 0: n > 63
+  const unsigned long long p = ((unsigned long long)m * m) << 14;
+  const long long sq = n < 0 ? 1ll << 62 : (long long)(p >> min(n, 63));
+  return max(d, -1ll) - sq;
+}
+__device__ __forceinline__ double sub_square(double d, float l, int) { return fma(-(double)l, (double)l, d); }
+
+constexpr int FIX_EMIN = -60, FIX_EMAX = 100;
+__device__ __forceinline__ bool fixed_range(double d) {
+  const long long b = __double_as_longlong(d);
+  return b >= (long long)(1023 + FIX_EMIN) << 52 && b < (long long)(1024 + FIX_EMAX) << 52;
+}
+
+template <bool FIX>
+__device__ __forceinline__ void potrf_f(float (*col)[PR_LD], long long *ps, int *es, float *D, int64_t ld, int ts,
+                                        int64_t g0, double d0, long long *status, double *__restrict__ piv) {
+  using DG = std::conditional_t<FIX, long long, double>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float v[2][4][2];  // [slot][column][row half]
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = 4 * (warp + 8 * q) + k, r = lane + 32 * h;
+        v[q][k][h] = (c < ts && r < ts && r >= c) ? D[(int64_t)c * ld + r] : 0.f;
+      }
+  int rd = 4 * (warp + 8 * ((lane >> 2) & 1)) + (lane & 3);  // the column whose diagonal lanes 0-7 carry
+  DG dg;
+  int eg = 0;  // E of this diagonal
+  if constexpr (FIX) {
+    const long long b = __double_as_longlong(d0);
+    eg = (int)(b >> 52) - 1023;
+    dg = ((b & 0xfffffffffffffll) | 0x10000000000000ll) << 8;
+  } else {
+    dg = d0;
+  }
+  const int nblk = (ts + 3) >> 2;
+  int bn = warp;  // the block in slot 0
+  auto apply = [&](auto qc, int b) {  // slot q -= block b
+    constexpr int q = decltype(qc)::value;
+    const int c0 = 4 * (bn + 8 * q);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const float *p = col[4 * b + j];
+      const float p0 = p[lane], p1 = p[lane + 32];
+      const float4 l4 = *reinterpret_cast<const float4 *>(p + c0);
+      const float l[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[q][k][0] = fma(-p0, l[k], v[q][k][0]);
+        v[q][k][1] = fma(-p1, l[k], v[q][k][1]);
+      }
+    }
+  };
+  auto apply_diagonal = [&](int b) {
+    float l[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) l[j] = col[4 * b + j][rd & (NB - 1)];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) dg = sub_square(dg, l[j], eg);
+  };
+  auto factor = [&](int b) {  // the owner of block b (slot 0); slot 1 moves to slot 0
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * b + k;
+      if (c >= ts) {  // (uniform) columns past the tile
+        col[c][lane] = col[c][lane + 32] = 0.f;
+        continue;
+      }
+      DG d = __shfl_sync(0xffffffffu, dg, k);
+      bool positive;
+      if constexpr (FIX) {
+        positive = d > 0;
+        if (lane == k) ps[c] = d, es[c] = eg;
+      } else {
+        const long long bits = __double_as_longlong(d);
+        positive = bits > 0 && bits <= 0x7ff0000000000000ll;  // d > 0, without the FP64 pipe
+        if (lane == k && piv) piv[g0 + c] = positive ? d : 1.0;
+      }
+      if (!positive && lane == 0) atomicMin(status, (long long)(g0 + c));
+      float df = 1.f;
+      if (positive) {
+        if constexpr (FIX) {
+          const int E = __shfl_sync(0xffffffffu, eg, k);
+          df = __ll2float_rn(d) * __int_as_float((E - 60 + 127) << 23);
+        } else {
+          df = (float)d;
+        }
+      }
+      const float xf = rsqrt_newton(df);  // d x = sqrt(d)
+      float x[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int r = lane + 32 * h;
+        x[h] = r == c ? df * xf : r > c ? v[0][k][h] * xf : 0.f;
+        col[c][r] = x[h];
+      }
+      if (k < 3) {  // (slot 1 gets this block from shared memory in the next step)
+        const float l = __shfl_sync(0xffffffffu, c < 32 ? x[0] : x[1], (c & 28) + (lane & 3));
+        dg = sub_square(dg, lane < 4 ? l : 0.f, eg);
+      }
+#pragma unroll
+      for (int k2 = k + 1; k2 < 4; ++k2) {
+        const float l = __shfl_sync(0xffffffffu, c < 32 ? x[0] : x[1], (c & 28) + k2);
+        v[0][k2][0] = fma(-x[0], l, v[0][k2][0]);
+        v[0][k2][1] = fma(-x[1], l, v[0][k2][1]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      v[0][k][0] = v[1][k][0];
+      v[0][k][1] = v[1][k][1];
+    }
+    dg = __shfl_down_sync(0xffffffffu, dg, 4);
+    eg = __shfl_down_sync(0xffffffffu, eg, 4);
+    rd += 32;
+    bn += 8;
+  };
+  using Q0 = std::integral_constant<int, 0>;
+  using Q1 = std::integral_constant<int, 1>;
+  if (warp == 0 && nblk > 0) factor(0);
+  __syncthreads();
+  for (int b = 0; b + 1 < nblk; ++b) {
+    if (bn < nblk) {
+      const bool two = bn < 8 && bn + 8 < nblk;  // slot 1 holds a block as well
+      apply_diagonal(b);
+      apply(Q0(), b);
+      if (two) apply(Q1(), b);
+      if (bn == b + 1) factor(b + 1);  // (warp-uniform)
+    }
+    __syncthreads();
+  }
+  if (FIX && piv && tid < ts)
+    piv[g0 + tid] = ps[tid] > 0 ? (double)ps[tid] * __longlong_as_double((long long)(es[tid] - 60 + 1023) << 52) : 1.0;
+  for (int idx = tid; idx < ts * ts; idx += PR_THREADS) {
+    const int r = idx % ts, c = idx / ts;
+    D[(int64_t)c * ld + r] = col[c][r];
+  }
+}
 
 __global__ void __launch_bounds__(PR_THREADS) k_potrf_r(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
                                                        float *__restrict__ Lx, long long *status,
@@ -672,8 +822,8 @@ __global__ void __launch_bounds__(PR_THREADS) k_potrf_r(const SNode *__restrict_
   Lx += blockIdx.y * bt.lx;
   status += blockIdx.y;
   if (axc) axc += blockIdx.y * bt.nnz;
-  __shared__ float col[NB][NB + 1];  // [c][row]: column c once final, zero above the diagonal
-  __shared__ double dd[NB];          // FP64 diagonal (see k_potrf)
+  if (piv) piv += blockIdx.y * bt.piv;
+  __shared__ __align__(16) float col[NB][PR_LD];  // [c][row]: column c once final, zero above the diagonal
   const Int4 t = tasks[toff + blockIdx.x];
   const SNode sj = sn[t.a];
   const int s = t.b;
@@ -681,90 +831,116 @@ __global__ void __launch_bounds__(PR_THREADS) k_potrf_r(const SNode *__restrict_
   const int64_t ld = sj.nrows;
   float *D = Lx + sj.lx + (int64_t)(s * NB) * ld + s * NB;
   const int64_t g0 = sj.first + (int64_t)s * NB;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  float v[8][2];  // owners: column cn + 8 u at rows lane, lane + 32
-  int cn = warp;
-  if (warp < PR_OWNERS) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rd = 4 * (warp + 8 * ((lane >> 2) & 1)) + (lane & 3);  // the column whose diagonal lanes 0-7 carry
+  double d0 = 1.0;
+  if (lane < 8 && rd < ts) d0 = diag64(D[(int64_t)rd * ld + rd], axc, dpos, g0 + rd);
+  __shared__ long long ps[NB];  // pivots and
+  __shared__ int es[NB];        // their units
+  if (__syncthreads_and(fixed_range(d0))) potrf_f<true>(col, ps, es, D, ld, ts, g0, d0, status, piv);
+  else potrf_f<false>(col, ps, es, D, ld, ts, g0, d0, status, piv);
+}
+
+// (c') FP32 panel TRSM of full tiles, columns in blocks of four: thread (r, g) owns row r and the
+// blocks g, g + G, ...; a tile of at most 32 rows spreads its rows over G = 8 groups, else G = 4. Step b,
+// one barrier: every thread applies the four solved columns of block b to its columns right of them, the
+// owners of block b + 1 that block first, which they then solve in registers. The same operations in
+// the same order as k_trsm and k_trsm_r (bit-identical), a quarter of the barriers: 17 us per
+// launch where k_trsm_r takes 26 us (the launches of a conductance matrix on 64^3: 3.7 ms, 5.6 ms).
+template <int G>
+__device__ __forceinline__ void trsm_f(float (*Ls)[PR_LD], float (*xs)[PR_LD], float *dinv, float *B, const float *D,
+                                       int64_t ld, int ts, int tm) {
+  constexpr int ROWS = THREADS / G, C = NB / G;  // rows, columns per thread
+  const int tid = threadIdx.x, r = tid & (ROWS - 1), g = tid / ROWS;
+  const bool live = (r & ~31) < tm;  // warp-uniform: some row of this warp is in the tile
+  for (int idx = tid; idx < NB * NB; idx += THREADS) {
+    const int rr = idx & (NB - 1), c = idx / NB;
+    Ls[c][rr] = rr >= c && rr < ts ? D[(int64_t)c * ld + rr] : 0.f;
+  }
+  float x[C];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int cc = warp + 8 * u, r = lane + 32 * h;
-        v[u][h] = (cc < ts && r < ts && r >= cc) ? D[(int64_t)cc * ld + r] : 0.f;
-      }
-  } else {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = lane + 32 * h;
-      if (r < ts) dd[r] = diag64(D[(int64_t)r * ld + r], axc, dpos, g0 + r);
-    }
+  for (int u = 0; u < C; ++u) {
+    const int c = 4 * G * (u >> 2) + 4 * g + (u & 3);
+    x[u] = (r < tm && c < ts) ? B[(int64_t)c * ld + r] : 0.f;
   }
   __syncthreads();
-  for (int c = 0; c < ts; ++c) {
-    if (warp < PR_OWNERS) {
-      float p0 = 0.f, p1 = 0.f;  // column c - 1 at this lane's rows
-      if (c > 0) {
-        p0 = col[c - 1][lane];
-        p1 = col[c - 1][lane + 32];
-      }
-      const bool own = cn == c;  // warp-uniform
-      if (own) {
-        double d = dd[c];
-        if (c > 0) {
-          const float l = col[c - 1][c];
-          v[0][0] = fma(-p0, l, v[0][0]);
-          v[0][1] = fma(-p1, l, v[0][1]);
-          d = fma(-(double)l, (double)l, d);
-        }
-        if (!(d > 0.0)) {
-          if (lane == 0) atomicMin(status, (long long)(g0 + c));
-          d = 1.0;
-        }
-        if (lane == 0 && piv) piv[blockIdx.y * bt.piv + g0 + c] = d;
-        const float df = (float)d;
-        const float xf = rsqrt_newton(df);  // d x = sqrt(d)
+  if (tid < NB) dinv[tid] = tid < ts ? 1.f / Ls[tid][tid] : 0.f;
+  __syncthreads();
+  const int nblk = (ts + 3) >> 2;
+  int bn = g;  // the block in x[0..3]
+  auto solve = [&](int b) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int r = lane + 32 * h;
-          col[c][r] = r == c ? df * xf : r > c ? v[0][h] * xf : 0.f;
-        }
-      }
-      if (c > 0) {
+    for (int k = 0; k < 4; ++k) {
+      const int c = 4 * b + k;
+      const float xc = x[k] * dinv[c];
+      xs[c][r] = xc;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int cc = cn + 8 * u;
-          if ((u > 0 || !own) && cc < ts) {
-            const float l = col[c - 1][cc];
-            v[u][0] = fma(-p0, l, v[u][0]);
-            v[u][1] = fma(-p1, l, v[u][1]);
-          }
-        }
-      }
-      if (own) {
+      for (int k2 = k + 1; k2 < 4; ++k2) x[k2] = fma(-xc, Ls[c][4 * b + k2], x[k2]);
+    }
 #pragma unroll
-        for (int u = 0; u < 7; ++u) {
-          v[u][0] = v[u + 1][0];
-          v[u][1] = v[u + 1][1];
-        }
-        v[7][0] = v[7][1] = 0.f;
-        cn += 8;
-      }
-    } else if (c > 0) {
+    for (int u = 0; u < C - 4; ++u) x[u] = x[u + 4];
+    bn += G;
+  };
+  if (live && g == 0) solve(0);
+  __syncthreads();
+  for (int b = 0; b + 1 < nblk; ++b) {
+    if (live && bn < nblk) {
+      float xp[4];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int k = lane + 32 * h;
-        if (k > c && k < ts) {
-          const float l = col[c - 1][k];
-          dd[k] = fma(-(double)l, (double)l, dd[k]);
+      for (int j = 0; j < 4; ++j) xp[j] = xs[4 * b + j][r];
+      auto apply = [&](auto uc) {
+        constexpr int u = decltype(uc)::value;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 l = *reinterpret_cast<const float4 *>(&Ls[4 * b + j][4 * bn + 4 * G * u]);
+          x[4 * u] = fma(-xp[j], l.x, x[4 * u]);
+          x[4 * u + 1] = fma(-xp[j], l.y, x[4 * u + 1]);
+          x[4 * u + 2] = fma(-xp[j], l.z, x[4 * u + 2]);
+          x[4 * u + 3] = fma(-xp[j], l.w, x[4 * u + 3]);
         }
+      };
+      const bool mine = bn == b + 1;  // (warp-uniform)
+      if (mine) {
+        apply(std::integral_constant<int, 0>());
+        solve(b + 1);
+      }
+      if (bn < nblk) apply(std::integral_constant<int, 0>());
+      if (bn + G < nblk) apply(std::integral_constant<int, 1>());
+      if constexpr (G == 4) {
+        if (bn + 2 * G < nblk) apply(std::integral_constant<int, 2>());
+        if (bn + 3 * G < nblk) apply(std::integral_constant<int, 3>());
       }
     }
     __syncthreads();
   }
-  for (int idx = tid; idx < ts * ts; idx += PR_THREADS) {
-    const int r = idx % ts, c = idx / ts;
-    D[(int64_t)c * ld + r] = col[c][r];
+  for (int idx = tid; idx < tm * ts; idx += THREADS) {
+    const int rr = idx % tm, c = idx / tm;
+    B[(int64_t)c * ld + rr] = xs[c][rr];
   }
+}
+
+__global__ void __launch_bounds__(THREADS) k_trsm_f(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
+                                                    float *__restrict__ Lx, int64_t toff, const Batch bt) {
+  Lx += blockIdx.y * bt.lx;
+  __shared__ __align__(16) float Ls[NB][PR_LD];  // [col][row], lower triangle of L_ss
+  __shared__ float xs[NB][PR_LD];                // [col][row]: solved columns
+  __shared__ float dinv[NB];
+  const Int4 t = tasks[toff + blockIdx.x];
+  const SNode sj = sn[t.a];
+  const int i = t.b, s = t.c;
+  const int ts = min(NB, sj.ncols - s * NB);
+  int64_t rb = d_row_tile_base(i, sj.ncols, sj.ncb);
+  int tm = d_row_tile_rows(i, sj.ncols, sj.nrows, sj.ncb);
+  const int half = t.d >> 16;  // 0: whole tile; 1, 2: its first or second 32 rows
+  if (half) {
+    rb += (half - 1) * (NB / 2);
+    tm = max(0, min(NB / 2, tm - (half - 1) * (NB / 2)));
+  }
+  const int64_t ld = sj.nrows;
+  const float *D = Lx + sj.lx + (int64_t)(s * NB) * ld + s * NB;
+  float *B = Lx + sj.lx + (int64_t)(s * NB) * ld + rb;
+  if (tm > NB / 2) trsm_f<4>(Ls, xs, dinv, B, D, ld, ts, tm);
+  else trsm_f<8>(Ls, xs, dinv, B, D, ld, ts, tm);
 }
 
 // (c'') Panel TRSM of full tiles with the tile in registers: thread (r, g) owns row r of the tile
@@ -2651,9 +2827,11 @@ inline void trace_mark(LaunchTrace *tr, int32_t kind, cudaStream_t st) {
 
 template <typename T>
 cudaError_t prepare_factor() {
-  cudaError_t e = cudaFuncSetAttribute(k_trsm_r<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)trsm_smem<T, NB>());
-  if (e != cudaSuccess) return e;
+  cudaError_t e = cudaSuccess;
+  if constexpr (std::is_same<T, double>::value) {
+    e = cudaFuncSetAttribute(k_trsm_r<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsm_smem<T, NB>());
+    if (e != cudaSuccess) return e;
+  }
   e = cudaFuncSetAttribute(k_trsm<T, SMALL_TB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)trsm_smem<T, SMALL_TB>());
   if (e != cudaSuccess) return e;
@@ -2980,7 +3158,9 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
               e = launch_trsm_z(g, s, prio, d, Lx, L.off);
               done = true;
             }
-          if (!done)  // the tile in registers
+          if constexpr (std::is_same<T, float>::value)
+            e = launch_prio(k_trsm_f, dim3(g, nb), THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
+          else if (!done)  // the tile in registers
             e = launch_prio(k_trsm_r<T>, dim3(g, nb), THREADS, trsm_smem<T, NB>(), s, prio, d.sn, d.tasks, Lx, L.off,
                             bt);
         }
