@@ -38,7 +38,7 @@ struct sym_handle_s {
   void *d_zc = nullptr;
   bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
-  double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix)
+  double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix or group of right-hand sides)
   int64_t y_cap = 0;
   double *d_stage = nullptr;      // staging for the host-pointer variants
   int64_t stage_cap = 0;
@@ -312,7 +312,8 @@ int ensure_batch(sym_handle_s *h, int32_t nbatch) {
     h->dp.piv = h->d_piv;
   }
   if (!rc) rc = regrow((void **)&h->d_status, sizeof(long long) * nb, "cudaMalloc(status batch)");
-  if (!rc) rc = regrow((void **)&h->d_t, sizeof(double) * sym::SOLVE_MAXRHS * P.tsize * nb, "cudaMalloc(solve buffer batch)");
+  const int64_t tmats = std::max<int64_t>(nb, h->dp.tgroups);
+  if (!rc) rc = regrow((void **)&h->d_t, sizeof(double) * sym::SOLVE_MAXRHS * P.tsize * tmats, "cudaMalloc(solve buffer batch)");
   h->dp.t = h->d_t;
   if (!rc) {
     if (h->h_status) cudaFreeHost(h->h_status);
@@ -550,8 +551,16 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
     if (!rc) rc = upload(P.contrib_ptr, &h->d_cptr, bytes);
     if (!rc) rc = upload(P.contrib, &h->d_contrib, bytes);
     if (!rc) {
-      const int64_t tb = (int64_t)sizeof(double) * sym::SOLVE_MAXRHS * (P.tsize > 0 ? P.tsize : 1);
-      e = cudaMalloc(&h->d_t, tb);
+      int64_t tb = (int64_t)sizeof(double) * sym::SOLVE_MAXRHS * (P.tsize > 0 ? P.tsize : 1);
+      h->dp.tgroups = sym::SOLVE_GROUPS;
+      e = cudaMalloc(&h->d_t, tb * sym::SOLVE_GROUPS);
+      if (e == cudaSuccess) {
+        tb *= sym::SOLVE_GROUPS;
+      } else {  // one group of right-hand sides at a time
+        cudaGetLastError();
+        h->dp.tgroups = 1;
+        e = cudaMalloc(&h->d_t, tb);
+      }
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(solve buffer)");
       else bytes += tb;
     }

@@ -3213,7 +3213,7 @@ inline const PanelForm *solve_panel(const PanelForm *forms, int64_t nform, size_
 
 template <typename T, typename V>
 cudaError_t launch_solve_b(bool forward, const DevPlan &d, const PanelForm &pf, unsigned g, unsigned nb,
-                           cudaStream_t st, const T *Lx, const T *Linv, V *y, V *tbuf, int r0, int nr, int64_t off,
+                           unsigned ny, cudaStream_t st, const T *Lx, const T *Linv, V *y, V *tbuf, int r0, int nr, int64_t off,
                            const Batch &bt) {
   if constexpr (std::is_same<T, V>::value) {
     const int lanes = solve_lanes_for(pf, nb, std::is_same<T, double>::value);
@@ -3222,11 +3222,11 @@ cudaError_t launch_solve_b(bool forward, const DevPlan &d, const PanelForm &pf, 
     const size_t smem = (size_t)solve_panel_bytes(pf.pmax, pf.ncmax, lanes, nrb);
 #define SYM_SOLVE_B(G, NRB)                                                                                      \
   if (lanes == G && nrb == NRB)                                                                                  \
-    return forward ? launch_pdl(k_fwd_b<T, V, G, NRB>, dim3(g, (nb + 32 / G - 1) / (32 / G)), 32, smem, st,     \
+    return forward ? launch_pdl(k_fwd_b<T, V, G, NRB>, dim3(g, (ny + 32 / G - 1) / (32 / G)), 32, smem, st,     \
                                 d.sn, d.tasks, d.cptr, d.contrib, Lx, Linv, y, tbuf, d.tsize, d.n, r0, nr, off,  \
-                                (int32_t)nb, pf.pmax, pf.ncmax, bt)                                              \
-                   : launch_pdl(k_bwd_b<T, V, G, NRB>, dim3(g, (nb + 32 / G - 1) / (32 / G)), 32, smem, st,     \
-                                d.sn, d.rows, d.tasks, Lx, Linv, y, d.n, r0, nr, off, (int32_t)nb, pf.pmax,       \
+                                (int32_t)ny, pf.pmax, pf.ncmax, bt)                                              \
+                   : launch_pdl(k_bwd_b<T, V, G, NRB>, dim3(g, (ny + 32 / G - 1) / (32 / G)), 32, smem, st,     \
+                                d.sn, d.rows, d.tasks, Lx, Linv, y, d.n, r0, nr, off, (int32_t)ny, pf.pmax,       \
                                 pf.ncmax, bt);
     SYM_SOLVE_B(1, 1)
     SYM_SOLVE_B(2, 1)
@@ -3240,15 +3240,47 @@ cudaError_t launch_solve_b(bool forward, const DevPlan &d, const PanelForm &pf, 
   return cudaErrorInvalidValue;
 }
 
+// One matrix and several right-hand sides: groups of nr go through the sweeps together, as a batch that
+// shares its panels (grid dimension y, at most tgroups * MAXRHS columns per pass). The chain of step
+// launches bounds a pass, and each step is a few CTAs whose time grows with nr (FP64 pipe, barriers),
+// so groups of one are the fastest as long as reading the panels once per group is cheap; beyond
+// SHARE entries times columns, groups of four or so. Milliseconds with groups of 1 / 4 / 8 (FP64,
+// 7-point conductance unless stated): 64^2 grid, 8 columns 0.16 / 0.32 / 0.53; 31^3, 16 columns 1.65 /
+// 1.89 / 2.42; 48^3, 8 columns (500 M) 3.95 / 4.27 / 5.02 and 32 (2 G) 11.0 / 9.95 / 10.9; 64^3, 4
+// columns (790 M) 6.42 / 6.32, 16 columns 17.9 / 15.4 / 16.9; FP32 with refinement: 31^3, 16 columns
+// (150 M) 2.9 / 3.1 / 3.8 and 32 4.5 / 4.0 / 4.6. (One group of 8 after another: 48^3, 16 columns
+// 10.1 ms against 6.3 now.) A width that does not divide the columns leaves the rest to another pass.
+template <typename T>
+int group_width(int64_t storage, int columns) {
+  constexpr int64_t SHARE = std::is_same<T, double>::value ? 600000000 : 250000000;
+  if (storage * columns <= SHARE) return 1;
+  for (const int nr : {4, 5, 3, 6, 7, 8, 2})
+    if (columns % nr == 0) return nr;
+  return columns <= 16 ? 1 : 4;
+}
+
 template <typename T, typename V>
 cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const std::vector<Launch> &bwd,
                        const T *Lx, const T *Linv, int nrhs, V *y, cudaStream_t st, LaunchTrace *trace,
-                       const Batch &bt) {
+                       const Batch &batch) {
   const int64_t n = d.n;
-  const unsigned nb = (unsigned)bt.count;
+  const unsigned nb = (unsigned)batch.count;
   V *tbuf = reinterpret_cast<V *>(d.t);
-  for (int r0 = 0; r0 < nrhs; r0 += MAXRHS) {
-    const int nr = nrhs - r0 < MAXRHS ? nrhs - r0 : MAXRHS;
+  for (int r0 = 0, next; r0 < nrhs; r0 = next) {
+    int nr = std::min(nrhs - r0, MAXRHS), groups = 1;
+    if (nb == 1) {
+      const int columns = std::min(nrhs - r0, d.tgroups * MAXRHS);
+      nr = group_width<T>(d.storage, columns);
+      groups = columns / nr;
+    }
+    next = r0 + groups * nr;
+    const unsigned ny = nb > 1 ? nb : (unsigned)groups;
+    Batch bt = batch;
+    if (nb == 1) {
+      bt.lx = bt.dinv = 0;  // (the groups share the matrix's panels)
+      bt.y = (int64_t)nr * n;
+      bt.t = (int64_t)nr * d.tsize;
+    }
     constexpr bool fp64 = std::is_same<T, double>::value && std::is_same<V, double>::value;
     for (size_t li = 0; li < fwd.size(); ++li) {
       const Launch &L = fwd[li];
@@ -3257,7 +3289,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
       // a fused narrow level: its step launch runs the sums, steps and pushes
       if (const PanelForm *pf = solve_panel(d.fwd_panel, d.nfwd_panel, fwd.size(), li, nb, fp64, nr)) {
         if (pf->role == PANEL_FUSED)
-          e = launch_solve_b<T, V>(true, d, *pf, g, nb, st, Lx, Linv, y, tbuf, r0, nr, L.off, bt);
+          e = launch_solve_b<T, V>(true, d, *pf, g, nb, ny, st, Lx, Linv, y, tbuf, r0, nr, L.off, bt);
         if (e != cudaSuccess) return e;
         trace_mark(trace, L.kind, st);
         continue;
@@ -3266,7 +3298,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
         case S_FGATHER: {
           cudaLaunchConfig_t cfg = {};
           cudaLaunchAttribute attr[1];
-          cfg.gridDim = dim3(g * (unsigned)L.cluster, nb, 1);
+          cfg.gridDim = dim3(g * (unsigned)L.cluster, ny, 1);
           cfg.blockDim = dim3(THREADS, 1, 1);
           cfg.dynamicSmemBytes = 0;
           cfg.stream = st;
@@ -3290,14 +3322,14 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
           }
           if (L.cluster == 4) {
             SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, true>, StepCfg<V, NR>::CS,
-                                                   dim3(StepCfg<V, NR>::CS * g, nb), st, d.sn, d.tasks, Lx,
+                                                   dim3(StepCfg<V, NR>::CS * g, ny), st, d.sn, d.tasks, Lx,
                                                    Linv, y, n, r0, L.off, bt)));
             break;
           }
           e = L.tb == SMALL_TB
-                  ? launch_pdl(k_fstep<T, V, SMALL_TB>, dim3(g, nb), TileCfg<SMALL_TB>::threads,
+                  ? launch_pdl(k_fstep<T, V, SMALL_TB>, dim3(g, ny), TileCfg<SMALL_TB>::threads,
                                step_smem<V, SMALL_TB>(), st, d.sn, d.tasks, Lx, Linv, y, n, r0, nr, L.off, bt)
-                  : launch_pdl(k_fstep<T, V, NB>, dim3(g, nb), THREADS, step_smem<V, NB>(), st, d.sn, d.tasks, Lx,
+                  : launch_pdl(k_fstep<T, V, NB>, dim3(g, ny), THREADS, step_smem<V, NB>(), st, d.sn, d.tasks, Lx,
                                Linv, y, n, r0, nr, L.off, bt);
           break;
         case S_FPUSH:
@@ -3306,7 +3338,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
                                                 32 * WT_WARPS, 0, st, d.sn, d.tasks, Lx, (const V *)y, tbuf, d.tsize,
                                                 n, r0, L.off, (int32_t)nb, bt)));
           } else {
-            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_fpush<T, V, NR>, dim3(g, nb), THREADS, 0, st, d.sn, d.tasks, Lx,
+            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_fpush<T, V, NR>, dim3(g, ny), THREADS, 0, st, d.sn, d.tasks, Lx,
                                                 (const V *)y, tbuf, d.tsize, n, r0, L.off, bt)));
           }
           break;
@@ -3316,7 +3348,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
                                                 32 * WT_WARPS, 0, st, d.sn, d.tasks, d.cptr, d.contrib,
                                                 (const V *)tbuf, d.tsize, y, n, r0, L.off, (int32_t)nb, bt)));
           } else {
-            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_fsum<V, NR>, dim3(g, nb), THREADS, 0, st, d.sn, d.tasks, d.cptr,
+            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_fsum<V, NR>, dim3(g, ny), THREADS, 0, st, d.sn, d.tasks, d.cptr,
                                                 d.contrib, (const V *)tbuf, d.tsize, y, n, r0, L.off, bt)));
           }
           break;
@@ -3332,7 +3364,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
       cudaError_t e = cudaSuccess;
       if (const PanelForm *pf = solve_panel(d.bwd_panel, d.nbwd_panel, bwd.size(), li, nb, fp64, nr)) {
         if (pf->role == PANEL_FUSED)
-          e = launch_solve_b<T, V>(false, d, *pf, g, nb, st, Lx, Linv, y, tbuf, r0, nr, L.off, bt);
+          e = launch_solve_b<T, V>(false, d, *pf, g, nb, ny, st, Lx, Linv, y, tbuf, r0, nr, L.off, bt);
         if (e != cudaSuccess) return e;
         trace_mark(trace, L.kind, st);
         continue;
@@ -3344,7 +3376,7 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
                                                 32 * WT_WARPS, 0, st, d.sn, d.rows, d.tasks, Lx, y, n, r0, L.off,
                                                 (int32_t)nb, bt)));
           } else {
-            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_bgather<T, V, NR>, dim3(g, nb), THREADS, 0, st, d.sn, d.rows,
+            SYM_NR_DISPATCH(nr, (e = launch_pdl(k_bgather<T, V, NR>, dim3(g, ny), THREADS, 0, st, d.sn, d.rows,
                                                 d.tasks, Lx, y, n, r0, L.off, bt)));
           }
           break;
@@ -3357,12 +3389,12 @@ cudaError_t run_sweeps(const DevPlan &d, const std::vector<Launch> &fwd, const s
           }
           if (L.cluster == 4) {
             SYM_NR_DISPATCH(nr, (e = launch_step_c(k_step_c<T, V, NR, false>, StepCfg<V, NR>::CS,
-                                                   dim3(StepCfg<V, NR>::CS * g, nb), st, d.sn, d.tasks, Lx,
+                                                   dim3(StepCfg<V, NR>::CS * g, ny), st, d.sn, d.tasks, Lx,
                                                    Linv, y, n, r0, L.off, bt)));
             break;
           }
           if (L.tb != SMALL_TB) return cudaErrorInvalidValue;  // (wider supernodes: the cluster form)
-          e = launch_pdl(k_bstep<T, V, SMALL_TB>, dim3(g, nb), TileCfg<SMALL_TB>::threads, step_smem<V, SMALL_TB>(),
+          e = launch_pdl(k_bstep<T, V, SMALL_TB>, dim3(g, ny), TileCfg<SMALL_TB>::threads, step_smem<V, SMALL_TB>(),
                          st, d.sn, d.tasks, Lx, Linv, y, n, r0, nr, L.off, bt);
           break;
         default:

@@ -19,7 +19,8 @@ struct DevPlan {
   const int32_t *perm = nullptr;
   const int64_t *cptr = nullptr;     // contribution lists of the forward solve (n + 1)
   const int32_t *contrib = nullptr;
-  void *t = nullptr;                 // forward-solve buffer: SOLVE_MAXRHS x tsize of the solve type
+  void *t = nullptr;                 // forward-solve buffer: SOLVE_MAXRHS x tsize of the solve type for each
+  int32_t tgroups = 1;               // of tgroups groups of right-hand sides (or the matrices of a batch)
   int64_t tsize = 0;
   int64_t n = 0;
   int64_t nnz_a = 0;

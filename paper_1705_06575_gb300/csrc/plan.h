@@ -20,6 +20,7 @@ constexpr int SOLVE_BG = 16;
 constexpr int SOLVE_CW = 512;
 // Right-hand sides per pass of the solve kernels (the buffer t holds this many).
 constexpr int SOLVE_MAXRHS = 8;
+constexpr int SOLVE_GROUPS = 4;  // groups of SOLVE_MAXRHS right-hand sides that one pass takes along
 // Order bound of the tiles that the small-tile kernel variants take.
 constexpr int SMALL_TILE = 32;
 // Batches: full-tile update launches whose entries have at most this many output elements on
