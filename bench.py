@@ -10,7 +10,8 @@ numeric phase on a fixed pattern).
 
 value  = factor flops (sum of squared column counts of L) per step / step time, summed over ranks
 e2e    = the same metric through the host-pointer C ABI (H2D of A's values and B, D2H of X)
-roofline: the kernel kind with the largest share of the step, against the measured FP64 FMA peak
+roofline: the kernel kind with the largest share of the step, against the tensor cores' rate of exact FP64
+  products (the update and the GEMM) or the measured FP64 FMA peak
 cpu_baseline / --impl reference: the CPU FP64 oracle (up-looking factor), single thread, timed on
 the leading block of the same matrix (a bounded sample; see --cpu-flops).
 """
@@ -41,29 +42,13 @@ WORKLOADS = {
 WORKLOAD_DESC = WORKLOADS[WORKLOAD]
 NRHS = 4
 METRIC = "refactor GFLOP/s and ms/(factor+solve) vs plain FP64 GPU path at bwd err<=1e-12"
-# DRAM traffic of the dominant kernel (the FP64 update, k_update_flat) per launch of the 64^3
-# step, from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum averaged over the 19
-# update launches of one step). It holds only for the kernel source it was taken on: the
-# sha256 (first 16 hex digits) of the kernel's definition text in csrc/kernels.cu. When that
-# text changes, the line reports null until the traffic is captured again.
-UPDATE_TRAFFIC = {"bytes_per_launch": 5.4518e8, "kernel_sha16": "6f9b0de4cc0dd30c"}
+# Dense FP16/BF16 rate of a library GEMM on GB300 (burst, TFLOP/s) and the MMA flops that one FP64 flop
+# takes as exact products of 8-bit digits (34 digit pairs): the roofline of the FP64 factor's k_oz.
+FP16_PEAK_TF, DIGIT_PRODUCTS = 1878.6, 34
 
 CLOCK_QUERY = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
                "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
                "clocks_event_reasons.sw_thermal_slowdown,clocks_event_reasons.sw_power_cap")
-
-
-def kernel_source_sha16(name="k_update_flat"):
-    """sha256 (16 hex digits) of the definition of a kernel template in csrc/kernels.cu: from the
-    template line before the kernel's name to the first closing brace at column 0."""
-    import hashlib
-    import re
-    src = open(os.path.join(ROOT, "paper_1705_06575_gb300", "csrc", "kernels.cu")).read()
-    m = re.search(r"\ntemplate <[^\n]*>\n[^\n]*\n\s*" + re.escape(name) + r"\(", src)
-    if not m:
-        return None
-    end = src.index("\n}\n", m.start())
-    return hashlib.sha256(src[m.start():end + 3].encode()).hexdigest()[:16]
 
 
 def dist_env():
@@ -599,16 +584,16 @@ def run_ours(args):
     # (sym_stats.update_flops); other kernels have no such split and report executed flops.
     useful = info.update_flops * args.steps if dom == "update" else dfl
     achieved_tf = useful / dms / 1e9
-    kname = {"update": "k_update_flat"}.get(dom, f"k_{dom}")  # the FP64 update kernel
-    traffic = None
-    if (dom == "update" and args.workload == WORKLOAD and UPDATE_TRAFFIC["bytes_per_launch"] is not None
-            and UPDATE_TRAFFIC["kernel_sha16"] == kernel_source_sha16("k_update_flat")):
-        traffic = UPDATE_TRAFFIC["bytes_per_launch"]
-    roofline = {"bound": "alu", "kernel": kname, "achieved": achieved_tf, "peak": peak_tf, "unit": "TFLOP/s",
-                "frac": achieved_tf / peak_tf, "frac_executed": exec_tf / peak_tf,
+    tensor = dom in ("update", "gemm")
+    bound_tf = FP16_PEAK_TF / DIGIT_PRODUCTS if tensor else peak_tf
+    roofline = {"bound": "tensor" if tensor else "alu", "kernel": "k_oz" if tensor else f"k_{dom}",
+                "achieved": achieved_tf, "peak": bound_tf, "unit": "TFLOP/s",
+                "frac": achieved_tf / bound_tf, "frac_executed": exec_tf / bound_tf,
+                "frac_of_fp64_pipe": achieved_tf / peak_tf,
                 "flops": "useful (exact pattern, no amalgamation zeros); frac_executed counts executed flops",
-                "traffic": traffic, "launches_per_step": dnl / args.steps,
-                "peak_source": "FP64 FMA peak measured live by sym_fma_peak (152 SMs x 2 DFMA/clk)",
+                "traffic": None, "launches_per_step": dnl / args.steps,
+                "peak_source": f"{FP16_PEAK_TF} TFLOP/s dense FP16 / {DIGIT_PRODUCTS} digit products per FP64 product"
+                if tensor else "FP64 FMA peak measured live by sym_fma_peak (152 SMs x 2 DFMA/clk)",
                 "share_of_step": dms / args.steps / ms_step,
                 "timing": "kernel time from CUDA events in a profiled pass of the same K steps"}
 
