@@ -475,9 +475,11 @@ __global__ void __launch_bounds__(Z_THREADS) k_trsm_z(const SNode *__restrict__ 
 //     complete exchange the sums of the even-slice and odd-slice lanes and update C;
 //   * warps 22-23 prepare the entry descriptors and row maps of the following batches of entries
 //     (of this tile or the next), so their chains of dependent loads stay off the other warps.
-// One CTA per SM: the accumulators take all of tensor memory, the ring 180 KB. The MMAs read 140 KB
-// of shared memory per chunk and the staging writes 57 KB, 1.5k cycles at 128 bytes per clock
-// against 1.27k cycles of MMA time (measured without staging); shared memory is the bound.
+// One CTA per SM: the accumulators take all of tensor memory, the ring 180 KB. A stage of 16 values of K
+// has the MMAs read 70 KB of shared memory and the loaders write 28 KB, 0.76k cycles at 128 bytes per
+// clock, and 0.64k cycles of MMA time (measured without staging); 1.3-1.45k cycles are measured on the
+// 48^3 root, the rest being the read-back (F2I runs at 16 per clock and SM) and the handshakes. The
+// root level's update at 64^3: 8.9 ms, 3.5 ms with the MMAs alone.
 // Measured and not kept: digits kept as bytes and converted while they are staged (half the bytes
 // loaded, ~400 instructions per warp and chunk: 4.6k cycles per chunk); staging and read-back in
 // the same sixteen warps with whole-tile accumulators (4.1k cycles: the read-back, limited by the
