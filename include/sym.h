@@ -71,9 +71,9 @@ extern "C" {
                                   (no lookahead overlap; results are identical either way) */
 #define SYM_FLAG_NO_TENSOR_CORES 8u /* SYM_PREC_MIXED: external updates in FP32 on the SIMT
                                        pipes instead of tcgen05 TF32 splits (x = hi + lo, all four
-                                       partial products accumulated in FP32). SYM_PREC_FP64: updates
-                                       on the FP64 pipe instead of exact products of 8-bit digits
-                                       on the FP16 tensor cores (56-bit fixed point, 64-bit sums) */
+                                       partial products accumulated in FP32). SYM_PREC_FP64: FP64
+                                       arithmetic throughout instead of the fixed point described at
+                                       sym_factor */
 #define SYM_FLAG_NO_FUSED_LEVELS 16u /* run the launches of levels of narrow supernodes apart
                                         instead of as one fused launch per level and phase
                                         (SYM_EXPORT_BATCH_PANEL, _FWD_PANEL, _BWD_PANEL), for
@@ -178,6 +178,17 @@ int sym_set_stream(sym_handle h, void *stream);
  * positive (or is NaN); sym_last_error_column then gives the first failing column in the
  * caller's numbering and the factor is not usable. Returns SYM_ERR_TIMEOUT (factor not usable)
  * when a tensor-core update of SYM_PREC_MIXED waited about a second for its MMAs in vain. */
+/* Arithmetic of SYM_PREC_FP64 for one matrix: tiles of more than 32 columns are factored and multiplied
+ * in fixed point (60 and 56 bits, exact sums) with one scale per row, the power of two at or above
+ * sqrt(a_ii). |A - L L^T|_ij then stays within c sqrt(a_ii a_jj) as in FP64, with c no larger, and
+ * so does the normwise backward error of a solve; but an entry of L far below its row's scale holds
+ * fewer significant bits than a double, down to none below 2^-60 of the scale. Where A's own values
+ * make that matter (large penalties on diagonal entries, parts of the matrix joined by weak couplings
+ * only, diagonals of coupled rows more than 2^14 apart, values that are not finite) the device finds out
+ * before the factorization and all of it runs in FP64. What remains: components of x many orders of
+ * magnitude below the others because the matrix is strongly diagonally dominant (the far field of a
+ * point source) are then accurate relative to the others, not to themselves. SYM_FLAG_NO_TENSOR_CORES,
+ * and a batch, take FP64 always. */
 int sym_factor(sym_handle h, const double *Ax);
 
 /* As sym_factor but returns right after enqueueing (no wait, no status check). Call

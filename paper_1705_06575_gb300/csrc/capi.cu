@@ -29,13 +29,19 @@ struct sym_handle_s {
   double *d_Lx = nullptr;
   double *d_Linv = nullptr;  // inverses of the diagonal tiles (FP64 factor)
   float *d_Lfinv = nullptr;  // the same for an FP32 factor
+  // One value per matrix and a last one, the bits of DevPlan::wide (one matrix); pinned: the reset
+  // values, then the statuses read back.
   long long *d_status = nullptr;
-  long long *h_status = nullptr;  // pinned: [0] holds the reset value, [1] receives the status
+  long long *h_status = nullptr;
   double *d_y = nullptr;          // solve work array
   uint4 *d_dg = nullptr;          // digits of the FP64 panels (one matrix, tensor cores)
   int32_t *d_exps = nullptr;      // their row scale exponents
   int2 *d_zu = nullptr;           // fixed-point data of their diagonal tiles
   void *d_zc = nullptr;
+  int2 *d_links = nullptr;        // A's entries as permuted (row, column), and the work arrays of the
+  int2 *d_ozrows = nullptr;       // check whether a matrix's values allow fixed point
+  int32_t *d_parent = nullptr;
+  uint8_t *d_strength = nullptr;
   bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
   double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix or group of right-hand sides)
@@ -184,7 +190,8 @@ void release_device(sym_handle_s *h) {
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   {
     void *mp[] = {h->d_Linv, h->d_Lfinv, h->d_Lf, h->d_Axc, h->d_anorm, h->d_anorm_work, h->d_csr_p, h->d_csr_i,
-                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps, h->d_zu, h->d_zc};
+                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps, h->d_zu, h->d_zc,
+                  h->d_links, h->d_ozrows, h->d_parent, h->d_strength};
     for (void *p : mp)
       if (p) cudaFree(p);
     if (h->h_eta) cudaFreeHost(h->h_eta);
@@ -311,14 +318,14 @@ int ensure_batch(sym_handle_s *h, int32_t nbatch) {
     }
     h->dp.piv = h->d_piv;
   }
-  if (!rc) rc = regrow((void **)&h->d_status, sizeof(long long) * nb, "cudaMalloc(status batch)");
+  if (!rc) rc = regrow((void **)&h->d_status, sizeof(long long) * (nb + 1), "cudaMalloc(status batch)");
   const int64_t tmats = std::max<int64_t>(nb, h->dp.tgroups);
   if (!rc) rc = regrow((void **)&h->d_t, sizeof(double) * sym::SOLVE_MAXRHS * P.tsize * tmats, "cudaMalloc(solve buffer batch)");
   h->dp.t = h->d_t;
   if (!rc) {
     if (h->h_status) cudaFreeHost(h->h_status);
     h->h_status = nullptr;
-    cudaError_t e = cudaMallocHost(&h->h_status, 2 * sizeof(long long) * nb);
+    cudaError_t e = cudaMallocHost(&h->h_status, (2 * nb + 1) * sizeof(long long));
     if (e != cudaSuccess) rc = cuda_fail(e, "cudaMallocHost(status batch)");
   }
   if (rc) {
@@ -386,11 +393,14 @@ void ensure_digits(sym_handle_s *h) {
     return;
   h->dg_tried = true;
   const size_t n = (size_t)h->plan.n;
-  const size_t bytes[4] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
-                           sizeof(int2) * (size_t)h->plan.dinv_storage, sym::oz_column_bytes() * n};
-  void **const ptr[4] = {(void **)&h->d_dg, (void **)&h->d_exps, (void **)&h->d_zu, &h->d_zc};
+  const size_t bytes[7] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
+                           sizeof(int2) * (size_t)h->plan.dinv_storage, sym::oz_column_bytes() * n,
+                           sizeof(int2) * n, sizeof(int32_t) * n, (size_t)h->plan.nnz_a};
+  void **const ptr[7] = {(void **)&h->d_dg, (void **)&h->d_exps, (void **)&h->d_zu, &h->d_zc,
+                         (void **)&h->d_ozrows, (void **)&h->d_parent, (void **)&h->d_strength};
   bool ok = true;
-  for (int i = 0; i < 4 && ok; ++i) ok = cudaMalloc(ptr[i], bytes[i] > 0 ? bytes[i] : 16) == cudaSuccess;
+  for (int i = 0; i < 7 && ok; ++i) ok = cudaMalloc(ptr[i], bytes[i] > 0 ? bytes[i] : 16) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(h->d_ozrows, 0, sizeof(int2) * n, h->stream) == cudaSuccess;
   if (ok) {
     for (size_t b : bytes) h->device_bytes += (int64_t)b;
   } else {
@@ -404,6 +414,9 @@ void ensure_digits(sym_handle_s *h) {
   h->dp.exps = h->d_exps;
   h->dp.zu = h->d_zu;
   h->dp.zc = h->d_zc;
+  h->dp.oz_rows = h->d_ozrows;
+  h->dp.parent = h->d_parent;
+  h->dp.strength = h->d_strength;
 }
 
 int check_device(sym_handle_s *h) {
@@ -422,12 +435,12 @@ int finish_status(sym_handle_s *h) {
   h->err_col = -1;
   int32_t bad = 0;
   for (int32_t b = 0; b < nb; ++b)
-    if (h->h_status[h->bcap + b] == -1) {
+    if (h->h_status[h->bcap + 1 + b] == -1) {
       h->factored = false;
       return fail(SYM_ERR_TIMEOUT, "a bounded device wait of the factorization ran out");
     }
   for (int32_t b = 0; b < nb; ++b) {
-    const long long s = h->h_status[h->bcap + b];
+    const long long s = h->h_status[h->bcap + 1 + b];
     if (s != LLONG_MAX) {
       h->batch_err[b] = (s >= 0 && s < h->plan.n) ? h->plan.perm[s] : -1;
       if (bad++ == 0) h->err_col = h->batch_err[b];
@@ -584,6 +597,14 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
       for (int64_t k = 0; k < P.n; ++k) dpos[k] = Ap[P.perm[k]];  // the diagonal leads each column
       rc = upload(dpos, &h->d_dpos, bytes);
     }
+    if (!rc && h->precision == SYM_PREC_FP64 && !(opt.flags & SYM_FLAG_NO_TENSOR_CORES) &&
+        P.max_ncols > sym::SMALL_TILE) {
+      std::vector<int2> links(P.nnz_a);
+      for (int64_t j = 0; j < P.n; ++j)
+        for (int64_t p = Ap[j]; p < Ap[j + 1]; ++p) links[p] = make_int2(P.iperm[Ai[p]], P.iperm[j]);
+      rc = upload(links, (void **)&h->d_links, bytes);
+      h->dp.links = h->d_links;
+    }
     if (!rc && h->precision == SYM_PREC_MIXED) {
       e = cudaMalloc(&h->d_Lf, sizeof(float) * (P.storage() > 0 ? P.storage() : 1));
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(L)");
@@ -624,11 +645,11 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
       }
     }
     if (!rc) {
-      e = cudaMalloc(&h->d_status, sizeof(long long));
+      e = cudaMalloc(&h->d_status, 2 * sizeof(long long));
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMalloc(status)");
     }
     if (!rc) {
-      e = cudaMallocHost(&h->h_status, 2 * sizeof(long long));  // [reset value, result] for one matrix
+      e = cudaMallocHost(&h->h_status, 3 * sizeof(long long));
       if (e != cudaSuccess) rc = cuda_fail(e, "cudaMallocHost(status)");
     }
     if (rc) {
@@ -694,8 +715,10 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
   h->factored = false;
   h->nbatch = nbatch;
   if (nbatch == 1) ensure_digits(h);
+  h->dp.wide = (int *)(h->d_status + 1);  // (one matrix)
   for (int32_t b = 0; b < nbatch; ++b) h->h_status[b] = LLONG_MAX;
-  CUDA_TRY(cudaMemcpyAsync(h->d_status, h->h_status, sizeof(long long) * nbatch, cudaMemcpyHostToDevice, h->stream),
+  h->h_status[nbatch] = 0;
+  CUDA_TRY(cudaMemcpyAsync(h->d_status, h->h_status, sizeof(long long) * (nbatch + 1), cudaMemcpyHostToDevice, h->stream),
            "status reset");
   if (!h->prepared) {
     CUDA_TRY(h->precision == SYM_PREC_MIXED ? sym::prepare_factor<float>() : sym::prepare_factor<double>(),
@@ -754,7 +777,7 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
     rc = collect_trace(h, tr, (double)nbatch, false);
     if (rc) return rc;
   }
-  CUDA_TRY(cudaMemcpyAsync(h->h_status + h->bcap, h->d_status, sizeof(long long) * nbatch, cudaMemcpyDeviceToHost,
+  CUDA_TRY(cudaMemcpyAsync(h->h_status + h->bcap + 1, h->d_status, sizeof(long long) * nbatch, cudaMemcpyDeviceToHost,
                            h->stream),
            "status read");
   if (h->precision == SYM_PREC_MIXED && h->plan.n > 0)

@@ -3006,7 +3006,7 @@ cudaError_t patch_address(cudaGraphExec_t exec, cudaGraphNode_t node, int nargs,
   cudaKernelNodeParams p = {};
   cudaError_t e = cudaGraphKernelNodeGetParams(node, &p);
   if (e != cudaSuccess) return e;
-  void *args[8];
+  void *args[SCALE_ARGS];
   for (int i = 0; i < nargs; ++i) args[i] = p.kernelParams[i];
   args[arg] = &address;
   p.kernelParams = args;
@@ -3035,6 +3035,7 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
     if (oz) {
       cudaError_t e = launch_oz_scale(st, d, Ax);
       if (e == cudaSuccess && nodes) e = captured_node(st, &nodes->second);
+      if (e == cudaSuccess) e = launch_oz_range(st, d);
       if (e != cudaSuccess) return e;
     }
   trace_mark(trace, K_SCATTER, st);

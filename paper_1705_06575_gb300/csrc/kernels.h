@@ -57,6 +57,13 @@ struct DevPlan {
   int2 *zu = nullptr;
   void *zc = nullptr;
   const int8_t *oz = nullptr;
+  // ... and whether this matrix's values take FP64 instead (launch_oz_range): every entry of A as
+  // (row, column), permuted; per row; the union-find's parents; per entry; the result for the kernels.
+  const int2 *links = nullptr;
+  int2 *oz_rows = nullptr;
+  int32_t *parent = nullptr;
+  uint8_t *strength = nullptr;
+  int *wide = nullptr;
   const double *axc = nullptr;       // FP32 factors: the FP64 copy of A's values (nnz_a per matrix)
   const int64_t *dpos = nullptr;     // index in A's values of C_kk, per column k
 };
@@ -99,7 +106,7 @@ struct CapturedNodes {
 };
 cudaError_t captured_node(cudaStream_t st, cudaGraphNode_t *node);
 cudaError_t patch_address(cudaGraphExec_t exec, cudaGraphNode_t node, int nargs, int arg, const void *address);
-constexpr int SCATTER_ARGS = 5, SCALE_ARGS = 4, PERM_ARGS = 7;
+constexpr int SCATTER_ARGS = 5, SCALE_ARGS = 10, PERM_ARGS = 7;
 
 // Per-device function attributes the factor kernels need (call with the device current, before
 // the first run_factor and outside stream capture).
@@ -118,12 +125,14 @@ cudaError_t launch_update_tc(dim3 grid, cudaStream_t st, int prio, const DevPlan
                              const Batch &bt, long long *status);
 
 // FP64 factors of one matrix on the tensor cores (oz_update.cu). Attributes (once per device,
-// outside capture); the row scales of one set of values; the digits of the row tiles of a TRSM
+// outside capture); the row scales of one set of values and whether they allow fixed point (*wide
+// zero before; two calls); the digits of the row tiles of a TRSM
 // launch; full diagonal tiles and their panel solves in fixed point (the latter with the digits;
 // oz_column_bytes: size of DevPlan::zc per column); one launch of external updates (cluster CTAs per tile share its entries); one launch of
 // trailing updates. A bounded wait that runs out records -1 in status.
 cudaError_t prepare_oz();
 cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax);
+cudaError_t launch_oz_range(cudaStream_t st, const DevPlan &d);
 cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
                             int64_t toff);
 size_t oz_column_bytes();

@@ -4,6 +4,7 @@
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -25,11 +26,108 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
   return (int)(r < NB ? r : NB);
 }
 
-// Row scales of one factorization: exps[k] from C_kk (permuted column k).
-__global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restrict__ dpos, int32_t *__restrict__ exps,
-                           int64_t n) {
+// Row scales of one factorization (exps[k] from C_kk, permuted column k) and whether fixed point with
+// these scales can stand for FP64 on this matrix. An entry of L is held to 2^-56 of its row's scale
+// where FP64 keeps 2^-53 of the entry itself, so what reaches x only through entries far below the
+// scale of their rows loses accuracy: a row whose diagonal is a large penalty passes 1 / sqrt(penalty)
+// of its scale on to its neighbours, and parts of the matrix that only weak couplings join drive each
+// other through those. Measured on a 14^3 7-point conductance matrix, largest relative error of a
+// component of x, FP64 kernels | fixed point: penalties of 1e4 on 5% of the diagonal 3e-15 | 3e-15, 1e5
+// 4e-15 | 9e-15, 1e8 5e-15 | 3e-13, 1e16 4e-15 | 3e-9; a plane of couplings scaled by 0.1 5e-15 | 1e-14,
+// 0.01 4e-15 | 5e-14, 1e-6 2e-14 | 6e-10, 1e-12 4e-15 | 8e-4. So *wide gets bit 0, and every kernel of
+// this file then works in FP64, if
+//   * a value is not finite;
+//   * a row's strongest coupling is below 2^-WEAK of its diagonal (a penalty on it);
+//   * two coupled rows' diagonals are more than 2^SPREAD apart;
+//   * couplings below 2^-WEAK of the smaller diagonal are the only links between two parts of the
+//     matrix: strong couplings are united into components (lock-free union-find on parent), and a weak
+//     coupling between two components decides. Weak couplings inside a component (irregular meshes,
+//     media of varying coefficients have them everywhere) lose nothing that matters: other paths
+//     between the same rows carry far more.
+// (Exponents are compared, so a limit is exact to a factor of two.) A well-coupled matrix pays two more
+// small launches; factor and solve of the 64^2 and 31^3 grids take the same time with and without them
+// (762 us, 5.1 ms).
+constexpr int WEAK = 9, SPREAD = 14;
+constexpr int WIDE = 1, LINKS = 2;  // bits of *wide: FP64; weak couplings present
+constexpr uint8_t LINK_WEAK = 1, LINK_STRONG = 2;
+// rows[k]: exponent + 1 of row k's strongest coupling (0: none; zero before the first kernel) and the
+// exponent of its diagonal.
+__device__ __forceinline__ int exponent_of(double a) { return (__double2hiint(a) >> 20) & 0x7ff; }
+
+__global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restrict__ dpos,
+                           const int2 *__restrict__ links, int32_t *__restrict__ exps, int2 *rows,
+                           int32_t *__restrict__ parent, uint8_t *__restrict__ strength, int *wide, int64_t n,
+                           int64_t nnz) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) exps[k] = oz::scale_exponent(Ax[dpos[k]]);
+  int bits = 0;
+  if (k < n) {
+    const double a = Ax[dpos[k]];
+    exps[k] = oz::scale_exponent(a);
+    parent[k] = (int32_t)k;
+    rows[k].y = exponent_of(a);
+    if (exponent_of(a) == 0x7ff) bits = WIDE;
+  }
+  if (k < nnz) {
+    const int2 l = links[k];
+    const double a = Ax[k];
+    uint8_t s = 0;
+    if (l.x != l.y && a != 0.0) {
+      const int x = exponent_of(a), er = exponent_of(Ax[dpos[l.x]]), ec = exponent_of(Ax[dpos[l.y]]);
+      const bool weak = x + WEAK < min(er, ec);
+      s = weak ? LINK_WEAK : LINK_STRONG;
+      if (weak) bits |= LINKS;
+      if (x == 0x7ff || er - ec > SPREAD || ec - er > SPREAD) bits |= WIDE;
+      for (const int r : {l.x, l.y})  // (only rising values need the atomic)
+        if (*(volatile int *)&rows[r].x < x + 1) atomicMax(&rows[r].x, x + 1);
+    }
+    strength[k] = s;
+  }
+  if (bits & ~*(volatile int *)wide) atomicOr(wide, bits);
+}
+
+// The root of v: chains of parents descend in index, and a step moves v two links up.
+__device__ __forceinline__ int32_t root_of(volatile int32_t *parent, int32_t v) {
+  int32_t p = parent[v];
+  while (p != v) {
+    const int32_t g = parent[p];
+    parent[v] = g;
+    v = g;
+    p = parent[v];
+  }
+  return v;
+}
+
+// Rows against their strongest coupling (cleared for the next matrix); with weak couplings present, the
+// components of the strong ones: the larger of two roots becomes a child of the smaller one.
+__global__ void k_oz_unite(const int2 *__restrict__ links, int2 *__restrict__ rows, int32_t *parent,
+                           const uint8_t *__restrict__ strength, int *wide, int64_t n, int64_t nnz) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < n) {
+    const int2 r = rows[k];
+    rows[k].x = 0;
+    if (r.x > 0 && r.x - 1 + WEAK < r.y) atomicOr(wide, WIDE);
+  }
+  if (k >= nnz || *(volatile int *)wide != LINKS || strength[k] != LINK_STRONG) return;
+  int32_t a = root_of(parent, links[k].x), b = root_of(parent, links[k].y);
+  while (a != b) {
+    if (a < b) {
+      const int32_t c = a;
+      a = b;
+      b = c;
+    }
+    const int32_t old = atomicCAS(&parent[a], a, b);
+    if (old == a) break;
+    a = root_of(parent, old);
+    b = root_of(parent, b);
+  }
+}
+
+__global__ void k_oz_bridges(const int2 *__restrict__ links, int32_t *parent, const uint8_t *__restrict__ strength,
+                             int *wide, int64_t nnz) {
+  if (*(volatile int *)wide != LINKS) return;
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < nnz && strength[k] == LINK_WEAK && root_of(parent, links[k].x) != root_of(parent, links[k].y))
+    atomicOr(wide, WIDE);
 }
 
 // Digits of a factored row tile (task {J, i, s} of a TRSM launch): thread (row, o) takes the eight
@@ -38,10 +136,10 @@ __global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restr
 __global__ void __launch_bounds__(256) k_oz_split(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
                                                   const int32_t *__restrict__ rows, const double *__restrict__ Lx,
                                                   uint4 *__restrict__ dg, const int32_t *__restrict__ exps,
-                                                  int64_t toff) {
+                                                  const int *__restrict__ wide, int64_t toff) {
   const Int4 t = tasks[toff + blockIdx.x];
   const SNode sj = sn[t.a];
-  if (sj.dg < 0) return;
+  if (sj.dg < 0 || (*wide & WIDE)) return;
   const int i = t.b, s = t.c;
   const int ts = min(NB, sj.ncols - s * NB);
   int64_t rb = tile_base(i, sj.ncols, sj.ncb);
@@ -128,6 +226,46 @@ __device__ __forceinline__ double rsqrt_delta(double d) {
 // one barrier for all, 46 us for 64 columns: 800 cycles per column; the FP64 kernel 44 us.)
 constexpr size_t POTRF_SMEM = 2 * NB * NB * sizeof(int2);
 constexpr int POTRF_Z_THREADS = 512;
+
+// The same tile in FP64 (WIDE): the operations of k_potrf in their order. Warp 0 carries the chain, the
+// others the trailing columns, lanes along the rows.
+__device__ __noinline__ void potrf_wide(double (*a)[NB + 1], double *D, int64_t ld, int ts, int64_t g0,
+                                        long long *status) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int idx = tid; idx < ts * NB; idx += POTRF_Z_THREADS) {
+    const int r = idx & (NB - 1), c = idx / NB;
+    a[c][r] = r >= c && r < ts ? D[(int64_t)c * ld + r] : 0.0;
+  }
+  __syncthreads();
+  auto finish_column = [&](int c) {
+    double d = a[c][c];
+    if (!(d > 0.0)) {
+      if (lane == 0) atomicMin(status, (long long)(g0 + c));
+      d = 1.0;
+    }
+    const double x = d > 1e-30 && d < 1e30 ? rsqrt_delta(d) : 1.0 / sqrt(d);
+    __syncwarp();
+    for (int r = c + lane; r < ts; r += 32) a[c][r] = r == c ? d * x : a[c][r] * x;
+  };
+  if (warp == 0 && ts > 0) finish_column(0);
+  __syncthreads();
+  for (int c = 0; c + 1 < ts; ++c) {
+    if (warp == 0) {
+      const double l = a[c][c + 1];
+      for (int r = c + 1 + lane; r < ts; r += 32) a[c + 1][r] = fma(-a[c][r], l, a[c + 1][r]);
+      __syncwarp();
+      finish_column(c + 1);
+    } else {
+      for (int cc = c + 1 + warp; cc < ts; cc += POTRF_Z_THREADS / 32 - 1)
+        for (int r = cc + lane; r < ts; r += 32) a[cc][r] = fma(-a[c][r], a[c][cc], a[cc][r]);
+    }
+    __syncthreads();
+  }
+  for (int idx = tid; idx < ts * NB; idx += POTRF_Z_THREADS) {
+    const int r = idx & (NB - 1), c = idx / NB;
+    if (r < ts) D[(int64_t)c * ld + r] = a[c][r];
+  }
+}
 __device__ __forceinline__ void bar_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -138,7 +276,8 @@ __device__ __forceinline__ void bar_arrive(int id, int threads) {
 __global__ void __launch_bounds__(POTRF_Z_THREADS) k_potrf_z(const SNode *__restrict__ sn,
                                                              const Int4 *__restrict__ tasks, double *__restrict__ Lx,
                                                              const int32_t *__restrict__ exps, int2 *__restrict__ zu,
-                                                             ZCol *__restrict__ zc, long long *status, int64_t toff) {
+                                                             ZCol *__restrict__ zc, long long *status,
+                                                             const int *__restrict__ wide, int64_t toff) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   int2(*ys)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw);                           // [c][row]: -yh
   int2(*us)[NB] = reinterpret_cast<int2(*)[NB]>(smem_raw + NB * NB * sizeof(int2));  // [c][row]: uh
@@ -151,6 +290,10 @@ __global__ void __launch_bounds__(POTRF_Z_THREADS) k_potrf_z(const SNode *__rest
   const int ts = min(NB, sj.ncols - s * NB);
   const int64_t ld = sj.nrows, g0 = sj.first + (int64_t)s * NB;
   double *D = Lx + sj.lx + (int64_t)(s * NB) * ld + s * NB;
+  if (*wide & WIDE) {
+    potrf_wide(reinterpret_cast<double(*)[NB + 1]>(smem_raw), D, ld, ts, g0, status);
+    return;
+  }
   const int32_t *ec = exps + g0;
   const int tid = threadIdx.x, lane = tid & 31, w = (tid >> 5) & 7, low = tid >> 8;  // low: rows 32-63
   const int row = lane + 32 * low;
@@ -437,11 +580,37 @@ __device__ __forceinline__ void trsm_z(unsigned char *smem_raw, const SNode &sj,
   }
 }
 
+// The same tile in FP64 (WIDE): the operations of k_trsm in their order, thread (row, group of columns).
+__device__ __noinline__ void trsm_wide(double (*Ls)[NB], double (*X)[NB], double *dinv, double *B, const double *D,
+                                       int64_t ld, int ts, int tm) {
+  const int tid = threadIdx.x, r = tid & (NB - 1), g = tid / NB;
+  constexpr int G = Z_THREADS / NB;
+  for (int c = g; c < ts; c += G) {
+    Ls[c][r] = r >= c && r < ts ? D[(int64_t)c * ld + r] : 0.0;
+    X[c][r] = r < tm ? B[(int64_t)c * ld + r] : 0.0;
+  }
+  __syncthreads();
+  if (tid < ts) dinv[tid] = 1.0 / Ls[tid][tid];
+  __syncthreads();
+  const bool live = (r & ~31) < tm;  // (warp-uniform)
+  for (int c = 0; c < ts; ++c) {
+    double xc = 0.0;
+    if (live) {
+      xc = X[c][r] * dinv[c];
+      for (int cc = c + 1 + g; cc < ts; cc += G) X[cc][r] = fma(-xc, Ls[c][cc], X[cc][r]);
+    }
+    __syncthreads();  // (X[c] is not read again)
+    if (live && g == 0 && r < tm) B[(int64_t)c * ld + r] = xc;
+  }
+}
+static_assert(sizeof(double) * (2 * NB * NB + NB) <= TRSM_SMEM, "shared memory of the FP64 form");
+static_assert(sizeof(double) * NB * (NB + 1) <= POTRF_SMEM, "shared memory of the FP64 form");
+
 __global__ void __launch_bounds__(Z_THREADS) k_trsm_z(const SNode *__restrict__ sn, const Int4 *__restrict__ tasks,
                                                       const int32_t *__restrict__ rows, double *__restrict__ Lx,
                                                       uint4 *__restrict__ dg, const int32_t *__restrict__ exps,
                                                       const int2 *__restrict__ zu, const ZCol *__restrict__ zc,
-                                                      int64_t toff) {
+                                                      const int *__restrict__ wide, int64_t toff) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const Int4 t = tasks[toff + blockIdx.x];
   const SNode sj = sn[t.a];
@@ -451,6 +620,13 @@ __global__ void __launch_bounds__(Z_THREADS) k_trsm_z(const SNode *__restrict__ 
   if (half) {
     rb += (half - 1) * (NB / 2);
     tm = max(0, min(NB / 2, tm - (half - 1) * (NB / 2)));
+  }
+  if (*wide & WIDE) {
+    const int64_t ld = sj.nrows, c0 = (int64_t)t.c * NB;
+    double *s = reinterpret_cast<double *>(smem_raw), *P = Lx + sj.lx + c0 * ld;
+    trsm_wide(reinterpret_cast<double(*)[NB]>(s), reinterpret_cast<double(*)[NB]>(s + NB * NB), s + 2 * NB * NB, P + rb,
+              P + c0, ld, min(NB, sj.ncols - (int)c0), tm);
+    return;
   }
   if (tm > NB / 2) trsm_z<4>(smem_raw, sj, t.c, rb, tm, rows, Lx, dg, exps, zu, zc);
   else trsm_z<8>(smem_raw, sj, t.c, rb, tm, rows, Lx, dg, exps, zu, zc);
@@ -541,15 +717,192 @@ struct Segments {
   }
 };
 
+// The same tiles in FP64 (WIDE), as the SIMT kernels: an entry's elements are mapped flat onto the
+// threads (a warp's multiply-add takes 64 cycles of the FP64 pipe however many lanes work, so every lane
+// should), the operands of eight columns are copied while the eight before are used, the tile's sums stay
+// in shared memory. Three groups of 256 threads (the SIMT kernels' three CTAs per SM) take every third
+// entry of an external update, their sums and then those of a cluster's CTAs added up in order, or a
+// tile each of a trailing update, so that one group's loads hide behind the others' arithmetic. Updates
+// and trailing updates of 7-point grids, milliseconds here | SIMT kernels: 31^3 4.5, 3.9 | 5.4, 3.6; 64^3
+// 240, 143 | 222, 132.
+constexpr int WIDE_SLOTS = 8, WIDE_K = 8;
+struct WideOperands {  // two chunks of columns: one in use, one on its way
+  double A[2][WIDE_K][NB], B[2][WIDE_K][NB];
+};
+constexpr int WIDE_GROUPS = 3;
+struct WideShared {
+  double sum[WIDE_GROUPS][NB][NB + 1];
+  WideOperands op[WIDE_GROUPS];
+};
+static_assert(sizeof(WideShared) <= NSTAGE * oz::STAGE, "the FP64 form uses the ring's memory");
+
+template <int J>
+__device__ __forceinline__ void wide_chunk(double (&v)[WIDE_SLOTS], const int (&ab)[WIDE_SLOTS],
+                                           const double (*A)[NB], const double (*B)[NB], int nk) {
+#pragma unroll J == 1 ? 4 : 2
+  for (int k = 0; k < nk; ++k)
+#pragma unroll
+    for (int q = 0; q < J; ++q) v[q] = fma(-A[k][ab[q] & 0xff], B[k][ab[q] >> 8], v[q]);
+}
+
+template <bool UPD>
+__device__ __noinline__ void update_wide(WideShared &W, const SNode *sn, const UpdTask *utasks,
+                                         const UpdEntry *ents, const int32_t *rel, const Int4 *tasks, double *Lx,
+                                         int64_t toff, int ntiles) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int cs = UPD ? (int)cluster.num_blocks() : 1, rank = UPD ? (int)cluster.block_rank() : 0;
+  constexpr int NG = WIDE_GROUPS, TG = OZ_THREADS / NG;
+  const int grp = threadIdx.x / TG, tid = threadIdx.x % TG, w = tid >> 5;
+  double(*sum)[NB + 1] = W.sum[grp];
+  WideOperands &O = W.op[grp];
+  const int tile0 = UPD ? blockIdx.x / cs : blockIdx.x + grp * gridDim.x;
+  const int tstep = UPD ? gridDim.x / cs : gridDim.x * NG;
+  for (int round = 0; round * tstep < ntiles; ++round) {
+    // (an update's tiles are sorted by work: every other round runs backwards over the CTAs)
+    const int tile = round * tstep + (UPD && (round & 1) ? tstep - 1 - tile0 : tile0);
+    if (tile >= ntiles) continue;
+    int J, i, j, s = 0, hoff = 0, tm = NB;
+    int64_t ea = 0, ez = 1;
+    if (UPD) {
+      const UpdTask t = utasks[toff + tile];
+      J = t.J;
+      i = t.bi;
+      j = t.bj;
+      ea = t.e0 + (t.e1 - t.e0) * rank / cs;
+      ez = t.e0 + (t.e1 - t.e0) * (rank + 1) / cs;
+    } else {
+      const Int4 t = tasks[toff + tile];
+      J = t.a;
+      i = t.b;
+      j = t.c;
+      s = t.d & 0xffff;
+      if (t.d >> 16) {
+        hoff = ((t.d >> 16) - 1) * (NB / 2);
+        tm = NB / 2;
+      }
+    }
+    const SNode sj = sn[J];
+    const int64_t ld = sj.nrows, rb = tile_base(i, sj.ncols, sj.ncb) + hoff;
+    const int cb = j * NB, tn = min(NB, sj.ncols - cb);
+    tm = max(0, min(tm, tile_rows(i, sj.ncols, sj.nrows, sj.ncb) - hoff));
+    double *C = Lx + sj.lx + (int64_t)cb * ld + rb;
+    for (int idx = tid; idx < NB * NB; idx += TG) {
+      const int r = idx & (NB - 1), c = idx / NB;
+      sum[c][r] = rank == 0 && (grp == 0 || !UPD) && r < tm && c < tn ? C[(int64_t)c * ld + r] : 0.0;
+    }
+    for (int64_t e = UPD ? ea + grp : ea; e < ez; e += NG) {
+      bar_sync(1 + grp, TG);  // the tile's sums as the entry before left them
+      const UpdEntry E = UPD ? ents[e] : UpdEntry();
+      const SNode sk = UPD ? sn[E.K] : sj;
+      const int m = UPD ? E.m : tm, nc = UPD ? E.n : tn, kc = UPD ? sk.ncols : min(NB, sj.ncols - s * NB);
+      const bool tri = UPD && i == j;  // a diagonal tile's entry: its rows are its columns
+      const int cnt = tri ? m * (m + 1) / 2 : m * nc;
+      const int64_t lk = sk.nrows;
+      const double *K = Lx + sk.lx + (UPD ? 0 : (int64_t)s * NB * ld);
+      const double *A = K + (UPD ? E.r_lo : rb), *B = K + (UPD ? E.c_lo : cb);
+      for (int e0 = 0; e0 < cnt; e0 += WIDE_SLOTS * TG) {
+        int ab[WIDE_SLOTS], at[WIDE_SLOTS];
+        double v[WIDE_SLOTS];
+#pragma unroll
+        for (int q = 0; q < WIDE_SLOTS; ++q) {
+          const int el = e0 + tid + TG * q;
+          int a = 0, b = 0;
+          at[q] = -1;
+          v[q] = 0.0;
+          if (el < cnt) {
+            if (tri) {
+              a = (int)((sqrtf(8.0f * el + 1.0f) - 1.0f) * 0.5f);
+              while ((a + 1) * (a + 2) / 2 <= el) ++a;
+              while (a * (a + 1) / 2 > el) --a;
+              b = el - a * (a + 1) / 2;
+            } else {
+              a = el % m;
+              b = el / m;
+            }
+            const int r = UPD ? rel[E.relr + a] - (int)rb : a, c = UPD ? rel[E.relc + b] - cb : b;
+            if (UPD || i != j || c <= r + hoff) {  // (not above the diagonal)
+              at[q] = c * (NB + 1) + r;
+              v[q] = sum[0][at[q]];
+            }
+          }
+          ab[q] = a | (b << 8);
+        }
+        const int left = cnt - e0 - 32 * w;  // elements from this warp's first one on
+        auto fetch = [&](int k0) {
+          const int nk = min(WIDE_K, kc - k0), u = (k0 / WIDE_K) & 1;
+          for (int idx = tid; idx < nk * NB; idx += TG) {
+            const int r = idx & (NB - 1), k = idx / NB;
+            if (r < m) oz::copy8(&O.A[u][k][r], A + (k0 + k) * lk + r);
+            if (r < nc) oz::copy8(&O.B[u][k][r], B + (k0 + k) * lk + r);
+          }
+          oz::copies_commit();
+        };
+        fetch(0);
+        for (int k0 = 0; k0 < kc; k0 += WIDE_K) {
+          const int nk = min(WIDE_K, kc - k0), u = (k0 / WIDE_K) & 1;
+          if (k0 + WIDE_K < kc) {
+            fetch(k0 + WIDE_K);
+            oz::copies_wait<1>();
+          } else {
+            oz::copies_wait<0>();
+          }
+          bar_sync(1 + grp, TG);
+          switch (left > 0 ? (left + TG - 1) / TG : 0) {  // this warp's slots with elements
+            case 0: break;
+            case 1: wide_chunk<1>(v, ab, O.A[u], O.B[u], nk); break;
+            case 2: wide_chunk<2>(v, ab, O.A[u], O.B[u], nk); break;
+            case 3: wide_chunk<3>(v, ab, O.A[u], O.B[u], nk); break;
+            case 4: wide_chunk<4>(v, ab, O.A[u], O.B[u], nk); break;
+            case 5: wide_chunk<5>(v, ab, O.A[u], O.B[u], nk); break;
+            case 6: wide_chunk<6>(v, ab, O.A[u], O.B[u], nk); break;
+            case 7: wide_chunk<7>(v, ab, O.A[u], O.B[u], nk); break;
+            default: wide_chunk<8>(v, ab, O.A[u], O.B[u], nk); break;
+          }
+          bar_sync(1 + grp, TG);  // (the chunk has been read)
+        }
+#pragma unroll
+        for (int q = 0; q < WIDE_SLOTS; ++q)
+          if (at[q] >= 0) sum[0][at[q]] = v[q];
+      }
+    }
+    if (!UPD) {
+      bar_sync(1 + grp, TG);
+      for (int idx = tid; idx < NB * tn; idx += TG) {
+        const int r = idx & (NB - 1), c = idx / NB;
+        if (r < tm) C[(int64_t)c * ld + r] = sum[c][r];
+      }
+      continue;  // (a thread's elements of the next tile's sums are those that it has written here)
+    }
+    __syncthreads();
+    if (cs > 1) cluster.sync();  // every rank's sums are complete
+    for (int idx = threadIdx.x; idx < NB * tn; idx += OZ_THREADS) {
+      const int r = idx & (NB - 1), c = idx / NB;
+      if (r >= tm || c % cs != rank) continue;
+      double v = 0.0;
+      for (int o = 0; o < cs; ++o) {
+        const double *p = cs > 1 ? cluster.map_shared_rank(&W.sum[0][0][0], o) : &W.sum[0][0][0];
+        for (int q = 0; q < NG; ++q) v += p[(q * NB + c) * (NB + 1) + r];
+      }
+      C[(int64_t)c * ld + r] = v;
+    }
+    if (cs > 1) cluster.sync();  // keep the other ranks' shared memory alive until it has been read
+    else __syncthreads();
+  }
+}
+
 template <bool UPD>
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     k_oz(const SNode *__restrict__ sn, const UpdTask *__restrict__ utasks, const UpdEntry *__restrict__ ents,
          const int32_t *__restrict__ rel, const Int4 *__restrict__ tasks, const int32_t *__restrict__ rows,
          double *__restrict__ Lx, const uint4 *__restrict__ dg, const int32_t *__restrict__ exps, int64_t toff,
-         int ntiles, long long *status, uint64_t wait_ns, int withhold) {
+         int ntiles, long long *status, const int *__restrict__ wide, uint64_t wait_ns, int withhold) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *stage0 = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
   OzShared &sh = *reinterpret_cast<OzShared *>(stage0 + NSTAGE * oz::STAGE);
+  if (*wide & WIDE) {
+    update_wide<UPD>(*reinterpret_cast<WideShared *>(stage0), sn, utasks, ents, rel, tasks, Lx, toff, ntiles);
+    return;
+  }
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = UPD ? (int)cluster.num_blocks() : 1, rank = UPD ? (int)cluster.block_rank() : 0;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -1005,36 +1358,44 @@ cudaError_t prepare_oz() {
   return cudaFuncSetAttribute(k_oz<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OZ_SMEM);
 }
 cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax) {
-  k_oz_scale<<<(unsigned)((d.n + 255) / 256), 256, 0, st>>>(Ax, d.dpos, d.exps, d.n);
+  const unsigned grid = (unsigned)((std::max(d.n, d.nnz_a) + 255) / 256);
+  k_oz_scale<<<grid, 256, 0, st>>>(Ax, d.dpos, d.links, d.exps, d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
+  return cudaGetLastError();
+}
+cudaError_t launch_oz_range(cudaStream_t st, const DevPlan &d) {
+  const unsigned grid = (unsigned)((std::max(d.n, d.nnz_a) + 255) / 256);
+  k_oz_unite<<<grid, 256, 0, st>>>(d.links, d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
+  k_oz_bridges<<<grid, 256, 0, st>>>(d.links, d.parent, d.strength, d.wide, d.nnz_a);
   return cudaGetLastError();
 }
 cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
                             int64_t toff) {
   return launch_oz(k_oz_split, tasks, 256, 0, 1, st, prio, d.sn, d.tasks, d.rows, Lx, d.dg, (const int32_t *)d.exps,
-                   toff);
+                   (const int *)d.wide, toff);
 }
 size_t oz_column_bytes() { return sizeof(ZCol); }
 cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
                            long long *status) {
   return launch_oz(k_potrf_z, tasks, POTRF_Z_THREADS, POTRF_SMEM, 1, st, prio, d.sn, d.tasks, Lx, (const int32_t *)d.exps,
-                   d.zu, (ZCol *)d.zc, status, toff);
+                   d.zu, (ZCol *)d.zc, status, (const int *)d.wide, toff);
 }
 cudaError_t launch_trsm_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff) {
   return launch_oz(k_trsm_z, tasks, Z_THREADS, TRSM_SMEM, 1, st, prio, d.sn, d.tasks, d.rows, Lx, d.dg,
-                   (const int32_t *)d.exps, (const int2 *)d.zu, (const ZCol *)d.zc, toff);
+                   (const int32_t *)d.exps, (const int2 *)d.zu, (const ZCol *)d.zc, (const int *)d.wide, toff);
 }
 cudaError_t launch_update_oz(unsigned tasks, int cluster, cudaStream_t st, int prio, const DevPlan &d, double *Lx,
                              int64_t toff, long long *status) {
   const unsigned grid = cluster > 1 ? tasks : tasks < OZ_CTAS ? tasks : OZ_CTAS;
   return launch_oz(k_oz<true>, grid, OZ_THREADS, OZ_SMEM, cluster, st, prio, d.sn, d.upd_tasks, d.upd_entries, d.rel,
                    d.tasks, d.rows, Lx, (const uint4 *)d.dg, (const int32_t *)d.exps, toff, (int)tasks, status,
-                   d.tc_wait_ns, (int)d.tc_withhold);
+                   (const int *)d.wide, d.tc_wait_ns, (int)d.tc_withhold);
 }
 cudaError_t launch_gemm_oz(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
                            long long *status) {
   return launch_oz(k_oz<false>, tasks < OZ_CTAS ? tasks : OZ_CTAS, OZ_THREADS, OZ_SMEM, 1, st, prio, d.sn,
                    d.upd_tasks, d.upd_entries, d.rel, d.tasks, d.rows, Lx, (const uint4 *)d.dg,
-                   (const int32_t *)d.exps, toff, (int)tasks, status, d.tc_wait_ns, (int)d.tc_withhold);
+                   (const int32_t *)d.exps, toff, (int)tasks, status, (const int *)d.wide,
+                   d.tc_wait_ns, (int)d.tc_withhold);
 }
 
 }  // namespace sym
