@@ -937,10 +937,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   tc::fence_after_sync();
   const uint32_t tmem = sh.tmem;
   volatile int *bad = &sh.bad;
-  // a bounded wait that also records its failure; false when this CTA gives up
+  // A bounded wait of a whole warp that also records its failure; false when this CTA gives up. One
+  // answer for the warp: lanes time out, and see another warp's failure, at different moments, and
+  // those that went on alone would wait for the others at the next warp-wide operation for ever.
   auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
-    if (!tc::mbar_wait(bar, parity, wait_ns)) *bad = 1;
-    return *bad == 0;
+    const bool done = tc::mbar_wait(bar, parity, wait_ns);
+    const bool ok = __all_sync(0xffffffffu, done && *bad == 0);
+    if (!ok) *bad = 1;
+    return ok;
   };
 
   if (warp >= META_WARP) {
@@ -981,7 +985,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (b % NMETA != me) continue;
         if (uses > 0) ok = wait(&sh.mempty[me], (uint32_t)(uses - 1) & 1u);
         ++uses;
-        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         int total = -1;
         if (!end) {
@@ -1071,7 +1074,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     bool ok = true;
     for (int b = 0; ok; ++b) {
       const int mb = b % NMETA;
-      if (!(ok = __all_sync(0xffffffffu, wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u)))) break;
+      if (!(ok = wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) break;
       const int total = __shfl_sync(0xffffffffu, *(volatile int *)&sh.eb[mb].total, 0);
       const int last = __shfl_sync(0xffffffffu, *(volatile int *)&sh.eb[mb].last, 0);
       if (total < 0) break;
@@ -1082,7 +1085,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t first = (info >> h) & 1u;
         // the accumulators are free once the half's previous segment has been read
         ok = (!first || segs == 0 || wait(&sh.drained[h], (segs - 1) & 1u)) && wait(&sh.full[st], ph);
-        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+        if (!ok) break;
         segs += first;
         const uint64_t a = adesc + st * (oz::STAGE >> 4), bd = bdesc + st * (oz::STAGE >> 4);
         if (!withhold && lane == 0) {
