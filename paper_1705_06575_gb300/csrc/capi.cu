@@ -39,9 +39,9 @@ struct sym_handle_s {
   int2 *d_zu = nullptr;           // fixed-point data of their diagonal tiles
   void *d_zc = nullptr;
   int2 *d_links = nullptr;        // A's entries as permuted (row, column), and the work arrays of the
-  int2 *d_ozrows = nullptr;       // check whether a matrix's values allow fixed point
+  void *d_ozrows = nullptr;       // check whether a matrix's values allow fixed point
   int32_t *d_parent = nullptr;
-  uint8_t *d_strength = nullptr;
+  int16_t *d_strength = nullptr;
   bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
   double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix or group of right-hand sides)
@@ -395,12 +395,12 @@ void ensure_digits(sym_handle_s *h) {
   const size_t n = (size_t)h->plan.n;
   const size_t bytes[7] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
                            sizeof(int2) * (size_t)h->plan.dinv_storage, sym::oz_column_bytes() * n,
-                           sizeof(int2) * n, sizeof(int32_t) * n, (size_t)h->plan.nnz_a};
+                           sym::oz_row_bytes() * n, sizeof(int32_t) * n, sizeof(int16_t) * (size_t)h->plan.nnz_a};
   void **const ptr[7] = {(void **)&h->d_dg, (void **)&h->d_exps, (void **)&h->d_zu, &h->d_zc,
-                         (void **)&h->d_ozrows, (void **)&h->d_parent, (void **)&h->d_strength};
+                         &h->d_ozrows, (void **)&h->d_parent, (void **)&h->d_strength};
   bool ok = true;
   for (int i = 0; i < 7 && ok; ++i) ok = cudaMalloc(ptr[i], bytes[i] > 0 ? bytes[i] : 16) == cudaSuccess;
-  ok = ok && cudaMemsetAsync(h->d_ozrows, 0, sizeof(int2) * n, h->stream) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(h->d_ozrows, 0, sym::oz_row_bytes() * n, h->stream) == cudaSuccess;
   if (ok) {
     for (size_t b : bytes) h->device_bytes += (int64_t)b;
   } else {

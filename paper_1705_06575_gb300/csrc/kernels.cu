@@ -3022,6 +3022,23 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
   // when tracing) every launch goes to st in list order, which satisfies every wait.
   const bool dual = two && two->aux && two->events && !trace;
   trace_mark(trace, -1, st);
+  // one FP64 matrix on the tensor cores: its row scales and range, where there are two streams beside
+  // the scatter and the launches that need neither (of the 64^2 grid's 762 us the range check takes 2,
+  // 9 with one launch after the other)
+  const bool oz = std::is_same<T, double>::value && nb == 1 && d.exps && d.tensor_cores;
+  if constexpr (std::is_same<T, double>::value)
+    if (oz) {
+      cudaStream_t s = dual ? two->aux : st;
+      if (dual) {
+        cudaEventRecord(two->fork, st);
+        cudaStreamWaitEvent(s, two->fork, 0);
+      }
+      cudaError_t e = launch_oz_scale(s, d, Ax);
+      if (e == cudaSuccess && nodes) e = captured_node(s, &nodes->second);
+      if (e == cudaSuccess) e = launch_oz_range(s, d);
+      if (e != cudaSuccess) return e;
+      if (dual) cudaEventRecord(two->join, s);
+    }
   k_zero<T><<<dim3(grid_for(d.storage, THREADS * 4), nb), THREADS, 0, st>>>(Lx, d.storage, bt);
   if (d.nnz_a > 0)
     k_scatter<T><<<dim3(grid_for(d.nnz_a, THREADS * 4), nb), THREADS, 0, st>>>(Ax, d.amap, Lx, d.nnz_a, bt);
@@ -3029,26 +3046,22 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
     cudaError_t e = captured_node(st, &nodes->first);
     if (e != cudaSuccess) return e;
   }
-  // one FP64 matrix on the tensor cores
-  const bool oz = std::is_same<T, double>::value && nb == 1 && d.exps && d.tensor_cores;
-  if constexpr (std::is_same<T, double>::value)
-    if (oz) {
-      cudaError_t e = launch_oz_scale(st, d, Ax);
-      if (e == cudaSuccess && nodes) e = captured_node(st, &nodes->second);
-      if (e == cudaSuccess) e = launch_oz_range(st, d);
-      if (e != cudaSuccess) return e;
-    }
   trace_mark(trace, K_SCATTER, st);
   if (dual) {  // the auxiliary stream starts after the panels hold A
     cudaEventRecord(two->fork, st);
     cudaStreamWaitEvent(two->aux, two->fork, 0);
   }
+  bool range = oz && dual;  // the main stream has not waited for the scales yet (the other one made them)
   for (size_t li = 0; li < launches.size(); ++li) {
     const Launch &L = launches[li];
     const unsigned g = (unsigned)L.count;
     cudaStream_t s = (dual && L.stream == 1) ? two->aux : st;
     const int prio = (dual && L.stream == 1) ? two->prio_low : two ? two->prio_high : 0;
     if (dual && L.wait >= 0) cudaStreamWaitEvent(s, (*two->events)[L.wait], 0);
+    if (range && s == st && (d.oz[li] || (L.tb != SMALL_TB && (L.kind == K_POTRF || L.kind == K_TRSM)))) {
+      cudaStreamWaitEvent(st, two->join, 0);
+      range = false;
+    }
     // a fused narrow level: its POTRF launch factors and inverts the whole panels, its TRSM and
     // TRTRI launches have nothing left to do
     int32_t panel = d.batch_panel ? d.batch_panel[li].role : PANEL_NONE;

@@ -60,9 +60,9 @@ struct DevPlan {
   // ... and whether this matrix's values take FP64 instead (launch_oz_range): every entry of A as
   // (row, column), permuted; per row; the union-find's parents; per entry; the result for the kernels.
   const int2 *links = nullptr;
-  int2 *oz_rows = nullptr;
+  void *oz_rows = nullptr;
   int32_t *parent = nullptr;
-  uint8_t *strength = nullptr;
+  int16_t *strength = nullptr;
   int *wide = nullptr;
   const double *axc = nullptr;       // FP32 factors: the FP64 copy of A's values (nnz_a per matrix)
   const int64_t *dpos = nullptr;     // index in A's values of C_kk, per column k
@@ -128,7 +128,7 @@ cudaError_t launch_update_tc(dim3 grid, cudaStream_t st, int prio, const DevPlan
 // outside capture); the row scales of one set of values and whether they allow fixed point (*wide
 // zero before; two calls); the digits of the row tiles of a TRSM
 // launch; full diagonal tiles and their panel solves in fixed point (the latter with the digits;
-// oz_column_bytes: size of DevPlan::zc per column); one launch of external updates (cluster CTAs per tile share its entries); one launch of
+// oz_column_bytes: size of DevPlan::zc per column, oz_row_bytes: of oz_rows per row); one launch of external updates (cluster CTAs per tile share its entries); one launch of
 // trailing updates. A bounded wait that runs out records -1 in status.
 cudaError_t prepare_oz();
 cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax);
@@ -136,6 +136,7 @@ cudaError_t launch_oz_range(cudaStream_t st, const DevPlan &d);
 cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
                             int64_t toff);
 size_t oz_column_bytes();
+size_t oz_row_bytes();
 cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
                            long long *status);
 cudaError_t launch_trsm_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff);

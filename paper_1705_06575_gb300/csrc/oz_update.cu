@@ -37,26 +37,41 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
 // 0.01 4e-15 | 5e-14, 1e-6 2e-14 | 6e-10, 1e-12 4e-15 | 8e-4. So *wide gets bit 0, and every kernel of
 // this file then works in FP64, if
 //   * a value is not finite;
-//   * a row's strongest coupling is below 2^-WEAK of its diagonal (a penalty on it);
+//   * a row's couplings add up to less than 2^-WEAK of its diagonal (a penalty on it);
 //   * two coupled rows' diagonals are more than 2^SPREAD apart;
-//   * couplings below 2^-WEAK of the smaller diagonal are the only links between two parts of the
-//     matrix: strong couplings are united into components (lock-free union-find on parent), and a weak
-//     coupling between two components decides. Weak couplings inside a component (irregular meshes,
-//     media of varying coefficients have them everywhere) lose nothing that matters: other paths
-//     between the same rows carry far more.
+//   * weak couplings are the only links between two parts of the matrix: couplings below 2^-WEAK of the
+//     smaller of the two diagonals and below 2^-FAINT of the strongest couplings of both rows (a long
+//     row's are all far below its diagonal). The others are united into components (lock-free
+//     union-find on parent), and a weak one between two components decides. Weak couplings inside a
+//     component (irregular meshes, media of varying coefficients have them everywhere) lose nothing
+//     that matters: other paths between the same rows carry far more.
 // (Exponents are compared, so a limit is exact to a factor of two.) A well-coupled matrix pays two more
-// small launches; factor and solve of the 64^2 and 31^3 grids take the same time with and without them
-// (762 us, 5.1 ms).
-constexpr int WEAK = 9, SPREAD = 14;
-constexpr int WIDE = 1, LINKS = 2;  // bits of *wide: FP64; weak couplings present
-constexpr uint8_t LINK_WEAK = 1, LINK_STRONG = 2;
-// rows[k]: exponent + 1 of row k's strongest coupling (0: none; zero before the first kernel) and the
-// exponent of its diagonal.
+// small launches, beside the scatter (run_factor): 2 of the 64^2 grid's 762 us for factor and solve,
+// nothing that shows on larger ones.
+constexpr int WEAK = 9, FAINT = 6, SPREAD = 14;
+constexpr int WIDE = 1, LINKS = 2;  // bits of *wide: FP64; couplings below 2^-WEAK of the diagonals present
+struct OzRow {  // (sum and strongest are zero before the first kernel)
+  unsigned long long sum;  // of the row's couplings, units of 2^-SUM_UNIT of the diagonal's power of two
+  int strongest;           // exponent + 1 of its strongest coupling, 0: none
+  int diagonal;            // exponent
+};
+constexpr int SUM_UNIT = 40;
+constexpr unsigned long long COUPLED = 1ull << (SUM_UNIT - WEAK);  // (no more is added to a sum beyond)
 __device__ __forceinline__ int exponent_of(double a) { return (__double2hiint(a) >> 20) & 0x7ff; }
 
+// x: exponent of a coupling of row r.
+__device__ __forceinline__ void add_coupling(OzRow *r, int x, int diagonal) {
+  if (*(volatile int *)&r->strongest < x + 1) atomicMax(&r->strongest, x + 1);
+  if (*(volatile unsigned long long *)&r->sum < COUPLED) {
+    const int sh = x - diagonal + SUM_UNIT;
+    if (sh >= 0) atomicAdd(&r->sum, sh < SUM_UNIT - WEAK ? 1ull << sh : COUPLED);
+  }
+}
+
+// strength[k]: exponent + 1 of entry k below the diagonal, 0: no coupling.
 __global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restrict__ dpos,
-                           const int2 *__restrict__ links, int32_t *__restrict__ exps, int2 *rows,
-                           int32_t *__restrict__ parent, uint8_t *__restrict__ strength, int *wide, int64_t n,
+                           const int2 *__restrict__ links, int32_t *__restrict__ exps, OzRow *rows,
+                           int32_t *__restrict__ parent, int16_t *__restrict__ strength, int *wide, int64_t n,
                            int64_t nnz) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int bits = 0;
@@ -64,25 +79,29 @@ __global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restr
     const double a = Ax[dpos[k]];
     exps[k] = oz::scale_exponent(a);
     parent[k] = (int32_t)k;
-    rows[k].y = exponent_of(a);
+    rows[k].diagonal = exponent_of(a);
     if (exponent_of(a) == 0x7ff) bits = WIDE;
   }
   if (k < nnz) {
     const int2 l = links[k];
     const double a = Ax[k];
-    uint8_t s = 0;
+    int x = -1;
     if (l.x != l.y && a != 0.0) {
-      const int x = exponent_of(a), er = exponent_of(Ax[dpos[l.x]]), ec = exponent_of(Ax[dpos[l.y]]);
-      const bool weak = x + WEAK < min(er, ec);
-      s = weak ? LINK_WEAK : LINK_STRONG;
-      if (weak) bits |= LINKS;
+      x = exponent_of(a);
+      const int er = exponent_of(Ax[dpos[l.x]]), ec = exponent_of(Ax[dpos[l.y]]);
+      if (x + WEAK < min(er, ec)) bits |= LINKS;
       if (x == 0x7ff || er - ec > SPREAD || ec - er > SPREAD) bits |= WIDE;
-      for (const int r : {l.x, l.y})  // (only rising values need the atomic)
-        if (*(volatile int *)&rows[r].x < x + 1) atomicMax(&rows[r].x, x + 1);
+      add_coupling(&rows[l.x], x, er);
+      add_coupling(&rows[l.y], x, ec);
     }
-    strength[k] = s;
+    strength[k] = (int16_t)(x + 1);
   }
   if (bits & ~*(volatile int *)wide) atomicOr(wide, bits);
+}
+// Whether entry k is a weak coupling.
+__device__ __forceinline__ bool weak_link(const OzRow *rows, int2 l, int strength) {
+  const OzRow &r = rows[l.x], &c = rows[l.y];
+  return strength - 1 + WEAK < min(r.diagonal, c.diagonal) && strength + FAINT < min(r.strongest, c.strongest);
 }
 
 // The root of v: chains of parents descend in index, and a step moves v two links up.
@@ -97,17 +116,18 @@ __device__ __forceinline__ int32_t root_of(volatile int32_t *parent, int32_t v) 
   return v;
 }
 
-// Rows against their strongest coupling (cleared for the next matrix); with weak couplings present, the
-// components of the strong ones: the larger of two roots becomes a child of the smaller one.
-__global__ void k_oz_unite(const int2 *__restrict__ links, int2 *__restrict__ rows, int32_t *parent,
-                           const uint8_t *__restrict__ strength, int *wide, int64_t n, int64_t nnz) {
+// Rows against the sum of their couplings; with couplings below 2^-WEAK of the diagonals present, the
+// components of the strong ones (the larger of two roots becomes a child of the smaller one); weak ones get
+// strength -1.
+__global__ void k_oz_unite(const int2 *__restrict__ links, const OzRow *__restrict__ rows, int32_t *parent,
+                           int16_t *__restrict__ strength, int *wide, int64_t n, int64_t nnz) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < n) {
-    const int2 r = rows[k];
-    rows[k].x = 0;
-    if (r.x > 0 && r.x - 1 + WEAK < r.y) atomicOr(wide, WIDE);
+  if (k < n && rows[k].strongest > 0 && rows[k].sum < COUPLED) atomicOr(wide, WIDE);
+  if (k >= nnz || *(volatile int *)wide != LINKS || strength[k] == 0) return;
+  if (weak_link(rows, links[k], strength[k])) {
+    strength[k] = -1;
+    return;
   }
-  if (k >= nnz || *(volatile int *)wide != LINKS || strength[k] != LINK_STRONG) return;
   int32_t a = root_of(parent, links[k].x), b = root_of(parent, links[k].y);
   while (a != b) {
     if (a < b) {
@@ -122,11 +142,16 @@ __global__ void k_oz_unite(const int2 *__restrict__ links, int2 *__restrict__ ro
   }
 }
 
-__global__ void k_oz_bridges(const int2 *__restrict__ links, int32_t *parent, const uint8_t *__restrict__ strength,
-                             int *wide, int64_t nnz) {
-  if (*(volatile int *)wide != LINKS) return;
+// Weak couplings between two components. The rows are cleared for the next matrix.
+__global__ void k_oz_bridges(const int2 *__restrict__ links, OzRow *__restrict__ rows, int32_t *parent,
+                             const int16_t *__restrict__ strength, int *wide, int64_t n, int64_t nnz) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < nnz && strength[k] == LINK_WEAK && root_of(parent, links[k].x) != root_of(parent, links[k].y))
+  if (k < n) {
+    rows[k].sum = 0;
+    rows[k].strongest = 0;
+  }
+  if (k < nnz && *(volatile int *)wide == LINKS && strength[k] < 0 &&
+      root_of(parent, links[k].x) != root_of(parent, links[k].y))
     atomicOr(wide, WIDE);
 }
 
@@ -1362,13 +1387,14 @@ cudaError_t prepare_oz() {
 }
 cudaError_t launch_oz_scale(cudaStream_t st, const DevPlan &d, const double *Ax) {
   const unsigned grid = (unsigned)((std::max(d.n, d.nnz_a) + 255) / 256);
-  k_oz_scale<<<grid, 256, 0, st>>>(Ax, d.dpos, d.links, d.exps, d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
+  k_oz_scale<<<grid, 256, 0, st>>>(Ax, d.dpos, d.links, d.exps, (OzRow *)d.oz_rows, d.parent, d.strength, d.wide, d.n,
+                                   d.nnz_a);
   return cudaGetLastError();
 }
 cudaError_t launch_oz_range(cudaStream_t st, const DevPlan &d) {
   const unsigned grid = (unsigned)((std::max(d.n, d.nnz_a) + 255) / 256);
-  k_oz_unite<<<grid, 256, 0, st>>>(d.links, d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
-  k_oz_bridges<<<grid, 256, 0, st>>>(d.links, d.parent, d.strength, d.wide, d.nnz_a);
+  k_oz_unite<<<grid, 256, 0, st>>>(d.links, (const OzRow *)d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
+  k_oz_bridges<<<grid, 256, 0, st>>>(d.links, (OzRow *)d.oz_rows, d.parent, d.strength, d.wide, d.n, d.nnz_a);
   return cudaGetLastError();
 }
 cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, const double *Lx,
@@ -1377,6 +1403,7 @@ cudaError_t launch_oz_split(unsigned tasks, cudaStream_t st, int prio, const Dev
                    (const int *)d.wide, toff);
 }
 size_t oz_column_bytes() { return sizeof(ZCol); }
+size_t oz_row_bytes() { return sizeof(OzRow); }
 cudaError_t launch_potrf_z(unsigned tasks, cudaStream_t st, int prio, const DevPlan &d, double *Lx, int64_t toff,
                            long long *status) {
   return launch_oz(k_potrf_z, tasks, POTRF_Z_THREADS, POTRF_SMEM, 1, st, prio, d.sn, d.tasks, Lx, (const int32_t *)d.exps,

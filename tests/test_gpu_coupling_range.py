@@ -105,6 +105,24 @@ def test_scattered_weak_couplings(torch_cuda):
     compare(torch_cuda, M, dominant(M, Ax), rng.uniform(0.5, 1.5, M.n))
 
 
+@pytest.mark.parametrize("n", [700, 1200])
+def test_long_rows_keep_the_tensor_cores(torch_cuda, n):
+    """A dense matrix's couplings are all far below its diagonals and still join it strongly: with the
+    MMAs withheld the factorization times out, so it takes the tensor cores; a penalty row does not."""
+    torch = torch_cuda
+    import paper_1705_06575_gb300 as S
+    M = w.random_spd_pattern(n, 1.0, np.random.default_rng(9))
+    s = S.Solver(M.n, M.Ap, M.Ai, M.perm)
+    S.sym_set_tc_wait(s.h, 20000, 1)
+    with pytest.raises(S.SymError) as e:
+        s.factor(torch.from_numpy(M.Ax).cuda())
+    assert e.value.code == S.SYM_ERR_TIMEOUT
+    Ax = M.Ax.copy()
+    Ax[M.Ap[5]] *= 1e6
+    s.factor(torch.from_numpy(Ax).cuda())
+    s.close()
+
+
 @pytest.mark.parametrize("maker", ["dense150", "star14"])
 @pytest.mark.parametrize("kind", ["inf_diagonal", "huge_diagonal", "inf_coupling", "nan_coupling"])
 def test_not_finite(torch_cuda, maker, kind):
