@@ -4,17 +4,30 @@
 // Fixed point. In a Cholesky factor every entry obeys |l_ik| <= sqrt(a_ii). Row i of the factor
 // gets the scale 2^e_i with sqrt(a_ii) < 0.986 * 2^e_i (e_i from the diagonal of A alone, known
 // before the factorization), and v = l_ik / 2^e_i is held as a 56-bit fixed-point number
-// v = sum_{s<7} d_s 2^(-7 - 8 s), the digits d_s integers in [-128, 127] (rounding error at most
+// v = sum_{s<7} d_s 2^(-7 - 8 s), the digits d_s integers in [-128, 128] (rounding error at most
 // 2^-56). A digit is exact in FP16, a product of digits is an integer of magnitude <= 2^14, and
 // an FP32 accumulator is exact while its sum stays below 2^24.
 //
-// Products. sum_k v_ik v_jk = sum_p 2^(-14 - 8 p) sum_{s+t=p} sum_k d_s(i,k) d_t(j,k). All pairs
-// s + t <= 7 are formed (34 products of digit matrices); the dropped ones are below 2^-62 of the
-// scale per term, as is the rounding of the digits, so the sum carries an error of the order of
-// 2^-62 sqrt(K) in units of sqrt(a_ii a_jj), less than FP64 multiply-adds leave (one rounding of
-// 2^-54 of the running value per step). The accumulators are combined in 64-bit integers (unit
-// 2^-62: the sum is below 2^62 by Cauchy-Schwarz, intermediate wrap-around cancels), whole tiles
-// are summed without any rounding, and the tile is updated with one FP64 rounding per entry.
+// Products (Ozaki's error-free splitting, with one exponent per row as in its integer variants: Ozaki,
+// Ogita, Oishi, Rump, Numer. Algorithms 59, 2012; Ootomo, Ozaki, Yokota 2024).
+// sum_k v_ik v_jk = sum_p 2^(-14 - 8 p) sum_{s+t=p} sum_k d_s(i,k) d_t(j,k). All pairs s + t <= 7 are
+// formed (34 products of digit matrices). Errors per term, in units of sqrt(a_ii a_jj): the rounding of
+// one operand's digits is at most 2^-56 times the other operand (to even, so without a preferred sign),
+// the dropped pairs are 2^-64.4 (root mean square; at most 2^-61.7). Off the diagonal the dropped pairs
+// have no preferred sign either once the columns' offsets alternate (OFFSET_ODD), so a sum's error grows
+// like sqrt(K), as FP64's does with one rounding of 2^-54 of the running value per step. On the diagonal
+// the pair s = t = 4 is a square, 2^-65.6 on average: these are added up apart (dropped_squares). A
+// bias would be invisible in residual norms and for random solutions; in a smooth solution of a nearly
+// singular matrix it adds up over a row. Row sums of L L^T - A of 40^3 7-point grids, mean over the
+// supernodes wider than 512 | standard deviation / sqrt(rows): here -5e-17 | 1e-16; one offset for all
+// columns 2.0e-15 | 1e-16; the FP64 kernels 5e-16 | 4e-16. Errors of x = 1, geometric means over seeds,
+// FP64 kernels | here | no squares, one offset, halves rounded up: 20^3 2.4e-14 | 1.2e-14 | 3.1e-14, 31^3
+// 3.4e-14 | 1.2e-14 | 4.5e-14, 48^3 1.4e-14 | 3.9e-14 | 5.6e-13 (here the solve's own 4e-14, which the FP64
+// kernels' factor happens to cancel), 27-point 28^3 7.4e-14 | 3.6e-14 | 6.8e-13. Random x: 1.3e-14 | 5.0e-15,
+// 9.5e-15 | 7.0e-15, 2.1e-14 | 9.4e-15, 1.2e-13 | 2.5e-14. The accumulators are combined in 64-bit integers
+// (unit 2^-62: the sum is below 2^62 by Cauchy-Schwarz, intermediate wrap-around cancels), whole tiles are
+// summed without any rounding but the last digits' (2^-63 per segment), and the tile is updated with one
+// FP64 rounding per entry.
 //
 // Layout. The digits of a factored panel are kept in FP16 as the tensor core reads them: octets of
 // eight columns, per octet the seven slices, per slice the rows, sixteen bytes each. A stage holds
@@ -30,6 +43,7 @@
 // then read back.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -52,8 +66,13 @@ constexpr uint32_t B_BYTES = 2 * B_LBO;
 constexpr uint32_t STAGE = A_BYTES + B_BYTES;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr int SEG_STEPS = 16;               // K = 16 steps per segment (256 values of k)
-constexpr uint64_t OFFSET = 0x0080808080808080ull;  // digit 0 is stored as byte 128
+// Digit 0 is stored as byte 128 in even columns (digits -128 .. 127), as byte 127 in odd ones (-127 ..
+// 128). A column's lower digits average -1/2 or 1/2; where they meet leading digits of one sign (the
+// entries of an M-matrix's factor) in pairs that are dropped, a single offset leaves a bias that grows
+// with K.
+constexpr uint64_t OFFSET = 0x0080808080808080ull, OFFSET_ODD = 0x007F7F7F7F7F7F7Full;
 constexpr uint64_t QMAX = 0x00FFFFFFFFFFFFFFull - OFFSET;
+__device__ __forceinline__ constexpr uint64_t offset_of(int column) { return column & 1 ? OFFSET_ODD : OFFSET; }
 
 // Scale exponent of a row from its diagonal entry a of A: sqrt(a) <= 0.986 * 2^e. Rows whose
 // diagonal is not a positive finite number fail as pivots whatever their scale.
@@ -67,8 +86,9 @@ __device__ __forceinline__ int scale_exponent(double a) {
   return (x + 1) >> 1;
 }
 
-// |v| / 2^e as a fixed-point number with unit 2^-U, rounded to nearest, at most `most` (a saturated
-// row fails as a pivot: its sum of squares exceeds its diagonal; so does a NaN's row).
+// |v| / 2^e as a fixed-point number with unit 2^-U, rounded to nearest even (few bits are dropped where
+// |v| is large, so halves are frequent; rounded up they would lengthen every row), at most `most` (a
+// saturated row fails as a pivot: its sum of squares exceeds its diagonal; so does a NaN's row).
 template <int U>
 __device__ __forceinline__ uint64_t fixed_magnitude(double v, int e, uint64_t most) {
   const uint64_t bits = (uint64_t)__double_as_longlong(v);
@@ -78,14 +98,14 @@ __device__ __forceinline__ uint64_t fixed_magnitude(double v, int e, uint64_t mo
   uint64_t q;
   if (E == 0x7ff || sh > U - 53) q = most;
   else if (sh >= 0) q = m << sh;
-  else if (sh >= -54) q = (m + (1ull << (-sh - 1))) >> (-sh);
+  else if (sh >= -54) q = (m + (1ull << (-sh - 1)) - 1 + (m >> (-sh) & 1)) >> (-sh);
   else q = 0;
   return q < most ? q : most;
 }
-// v / 2^e with unit 2^-55 plus OFFSET: the digits' bytes.
-__device__ __forceinline__ uint64_t to_fixed(double v, int e) {
+// v / 2^e with unit 2^-55 plus a column's offset: the digits' bytes.
+__device__ __forceinline__ uint64_t to_fixed(double v, int e, uint64_t offset) {
   const uint64_t q = fixed_magnitude<55>(v, e, QMAX);
-  return v < 0.0 ? OFFSET - q : OFFSET + q;
+  return v < 0.0 ? offset - q : offset + q;
 }
 // v / 2^e with unit 2^-60 (the panel solve's arithmetic).
 constexpr int64_t Q60MAX = (int64_t)(QMAX << 5);
@@ -139,14 +159,15 @@ __device__ __forceinline__ void transpose4(uint32_t w0, uint32_t w1, uint32_t w2
   out[2] = prmt(t2, t3, 0x5410);
   out[3] = prmt(t2, t3, 0x7632);
 }
-// Two digits (bytes 128 + d) to FP16: the byte under the exponent byte 0x64 is 1024 + 128 + d,
-// exact; minus 1152.
+// Two digits (bytes 128 + d, 127 + d) to FP16: the byte under the exponent byte 0x64 is 1024 + 128 + d,
+// exact; minus 1152 (1151).
 __device__ __forceinline__ uint32_t half2_of(uint32_t w, uint32_t sel) {
   uint32_t h = prmt(w, 0x64646464u, sel), r;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x647F6480u));
   return r;
 }
-// The FP16 digits of eight values (fixed-point numbers with OFFSET), one slice per element of w.
+// The FP16 digits of eight values (fixed-point numbers with their columns' offsets), one slice per
+// element of w.
 __device__ __forceinline__ void to_digits(const uint64_t (&q)[8], uint4 (&w)[SL]) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -250,6 +271,22 @@ __device__ __forceinline__ void drain(uint32_t addr, bool up, unsigned long long
       else acc[q] += (unsigned long long)(long long)(x + ((y + 128) >> 8));
     }
   }
+}
+
+// The sum of the squares of eight digits.
+__device__ __forceinline__ float square_sum(uint4 w) {
+  const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+  float s[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&u[k]));
+    s[k] = fmaf(f.x, f.x, f.y * f.y);
+  }
+  return (s[0] + s[1]) + (s[2] + s[3]);
+}
+// Squares of digit 4 (unit 2^-78) in the unit of the 64-bit sums.
+__device__ __forceinline__ unsigned long long dropped_squares(float sq) {
+  return (unsigned long long)__float2ll_rn(sq * (1.0f / 65536.0f));
 }
 
 // c - q 2^(-62) 2^ei 2^ej with one rounding of the product's conversion and one of the sum.

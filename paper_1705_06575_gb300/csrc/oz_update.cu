@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(256) k_oz_split(const SNode *__restrict__ sn, 
     for (int c = 0; c < 8; ++c) v[c] = 8 * o + c < ts ? src[c * ld] : 0.0;
     uint64_t q[8];
 #pragma unroll
-    for (int c = 0; c < 8; ++c) q[c] = oz::to_fixed(v[c], e);
+    for (int c = 0; c < 8; ++c) q[c] = oz::to_fixed(v[c], e, oz::offset_of(c));
     uint4 w[oz::SL];
     oz::to_digits(q, w);
     uint4 *dst = dg + sj.dg + (int64_t)(s * (NB / 8) + o) * oz::SL * ld + r;
@@ -590,9 +590,9 @@ __device__ __forceinline__ void trsm_z(unsigned char *smem_raw, const SNode &sj,
           x = oz::mul60(make_int2(-ny.x, -ny.y), col[c].lam);
           B[(int64_t)c * ld + r] = oz::from_fixed60(x, er);
         }
-        x = (x + 16) >> 5;
+        x = (x + 15 + (x >> 5 & 1)) >> 5;  // (to even)
         x = max(min(x, (int64_t)oz::QMAX), -(int64_t)oz::QMAX);
-        q[k] = (uint64_t)(x + (int64_t)oz::OFFSET);
+        q[k] = (uint64_t)(x + (int64_t)oz::offset_of(k));
       }
       if (sj.dg >= 0) {
         uint4 w[oz::SL];
@@ -703,6 +703,7 @@ struct OzBatch {
   int32_t cld, tm, tn;
   int16_t erow[NB], ecol[NB];  // scale exponents of the tile's rows and columns
   int8_t inv[2][EB][NB];   // [0] rows, [1] columns: tile position -> entry row, or -1
+  float sq[2][NB];         // (last batch of a diagonal tile) squares of digit 4: rows, even octets; columns, odd
 };
 struct OzShared {
   OzBatch eb[NMETA];
@@ -1137,18 +1138,36 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     // cycles each on the barrier, 1k cycles per chunk) LAG chunks after its copies were issued, or
     // when the sequence pauses.
     int it = 0, told = 0;  // chunks issued, chunks announced
-    auto tell = [&]() {
+    // On a diagonal tile each thread also adds up the squares of digit 4 of its row (operand A: the first
+    // octet of every chunk, B: the second one), read back once its copies have landed. kinds: four bits per
+    // chunk that is not announced yet (1: of a diagonal tile, 2: the tile's last one, 4: its batch's place).
+    // The sum is written before the tile's last chunk is announced, so before its MMAs are issued and
+    // before the read-back learns that they are done.
+    const uint8_t *digit4 = stage0 + (op ? oz::A_BYTES + (p >> 5) * oz::B_HALF + 16 * (p & 31) + 4 * oz::B_SLICE + oz::B_LBO
+                                         : 16 * p + 4 * oz::A_SLICE);
+    float sq = 0.f;
+    uint32_t kinds = 0;
+    auto announce = [&]() {
+      const uint32_t kind = kinds & 15u;
+      kinds >>= 4;
+      if (kind & 1u) {
+        sq += oz::square_sum(*reinterpret_cast<const uint4 *>(digit4 + (told % NSTAGE) * oz::STAGE));
+        if ((kind & 2u) && cs == 1) {
+          sh.eb[kind >> 2].sq[op][p] = sq;
+          sq = 0.f;
+        }
+      }
       tc::fence_smem_to_async();
       __syncwarp();
-      for (; told < it; ++told)
-        if (lane == 0) tc::mbar_arrive(&sh.full[told % NSTAGE]);
+      if (lane == 0) tc::mbar_arrive(&sh.full[told % NSTAGE]);
+      ++told;
     };
     bool ok = true;
     for (int b = 0; ok; ++b) {
       const int mb = b % NMETA;
       if (told < it && !__all_sync(0xffffffffu, tc::mbar_test(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) {
         oz::copies_wait<0>();
-        tell();
+        while (told < it) announce();
       }
       if (!(ok = wait(&sh.mfull[mb], (uint32_t)(b / NMETA) & 1u))) break;
       const OzBatch &eb = sh.eb[mb];
@@ -1180,12 +1199,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             src += ld;
           }
         oz::copies_commit();
+        kinds |= ((eb.diag ? 1u : 0u) | (eb.last && c + 1 == total ? 2u : 0u) | (uint32_t)mb << 2) << (4 * (it - told));
         if (it - told >= LAG) {
           oz::copies_wait<LAG>();
-          tc::fence_smem_to_async();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&sh.full[told % NSTAGE]);
-          ++told;
+          announce();
         }
         if (++cgp == eb.ng[ci]) {
           cgp = 0;
@@ -1198,7 +1215,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       if (lane == 0) tc::mbar_arrive(&sh.mempty[mb]);
     }
     oz::copies_wait<0>();
-    tell();
+    while (told < it) announce();
+    if (UPD && cs > 1) sh.eb[0].sq[op][p] = sq;  // (for the end)
   } else {
     // ---- read-back: lanes 32 (warp & 3) .. of tensor memory, columns 8 (warp >> 2) .. of each
     // half of the tile
@@ -1259,7 +1277,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         for (int q = 0; q < 4; ++q) {
           const int c = k0 + q;
           if (c < tn && !(dtop >= 0 && c > drow)) {
-            const unsigned long long v = acc[q] + buf[(up ? q + 4 : q) * 32];
+            unsigned long long v = acc[q] + buf[(up ? q + 4 : q) * 32];
+            if (dtop >= 0 && c == drow) v += oz::dropped_squares(eb.sq[0][row] + eb.sq[1][c]);
             C[(int64_t)q * eb.cld] =
                 dtop >= 0 && c == drow && sh.dred[h][pair][0][lane] + sh.dred[h][pair][1][lane] > 1.5f
                     ? -1.0
@@ -1340,14 +1359,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       double *x = C + (int64_t)c * sj.nrows + r;
       const double old = *x;
       unsigned long long v = 0;
-      float d = 0.f;
+      float d = 0.f, sq = 0.f;
       for (int o = 0; o < cs; ++o) {
         v += cluster.map_shared_rank(sh.red, o)[c * NB + r];
         if (diag && c == r) {
           const float *dr = cluster.map_shared_rank(&sh.dred[c >> 5][(r >> 5) | ((c >> 3 & 3) << 1)][0][0], o);
           d += dr[r & 31] + dr[32 + (r & 31)];
+          const float *q = cluster.map_shared_rank(&sh.eb[0].sq[0][0], o);
+          sq += q[r] + q[NB + c];
         }
       }
+      v += oz::dropped_squares(sq);
       *x = d > 1.5f ? -1.0 : oz::apply(old, (long long)v, exps[rows[sj.rowp + rb + r]], exps[sj.first + cb + c]);
     }
     cluster.sync();  // keep the other ranks' shared memory alive until it has been read
