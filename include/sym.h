@@ -219,19 +219,22 @@ int sym_solve_batch(sym_handle h, int32_t nbatch, int32_t nrhs, const double *B,
  * sym_factor), every factor launch that has two kernel forms is timed in both with CUDA events
  * over reps kernel-by-kernel factorizations of the given values, and the faster form is stored
  * in the plan for every later factorization of the handle (the captured graphs are rebuilt).
- * Forms: in a batch, FP64 updates run with the lanes of a warp on several matrices or one warp
- * per (tile, matrix) (small tiles, and full tiles with small entries) or one CTA per tile and
- * matrix (full tiles with large entries); small-tile POTRF, TRSM and TRTRI one warp per (tile,
- * matrix), four matrices per CTA, or one CTA per tile and matrix; for one
- * matrix, FP64 updates of tiles with many entries run on a thread-block cluster per tile or one
+ * Without it the forms of a batch's launches follow their number of (tile, matrix) pairs; a stored
+ * form holds for batches of any size at which that rule gives the same answer as at the size
+ * that was timed, the rule elsewhere.
+ * Forms: in a batch, FP64 updates of small tiles run with the lanes of a warp on several matrices or one
+ * warp per (tile, matrix), of full tiles with small entries one warp or one CTA per (tile, matrix), with
+ * large entries lanes on several matrices or one CTA; small-tile POTRF, TRSM and TRTRI one warp per
+ * (tile, matrix) or one CTA; for one matrix, FP64 updates of tiles with many entries run on the
+ * tensor cores (or, with SYM_FLAG_NO_TENSOR_CORES, on a thread-block cluster per tile) or one
  * CTA per tile, FP32 updates of full tiles on the tensor cores or the SIMT pipes, and small-tile
  * POTRF and TRTRI one CTA or one warp per tile. A batch's levels of narrow supernodes
  * (SYM_EXPORT_BATCH_PANEL) are first timed as one fused launch against their separate POTRF,
  * TRSM and TRTRI launches (the sums of the level's launch times), the faster kept; the launches
  * of a level kept separate then have their forms tuned like the others. The
  * per-kernel profile totals are left as they were. *tuned: fused levels plus launches with two
- * forms; *changed: levels returned to separate launches plus launches now on their second form
- * (either pointer may be NULL). Errors as sym_factor_batch,
+ * forms; *changed: levels returned to separate launches plus launches now on another form than the
+ * rule's (either pointer may be NULL). Errors as sym_factor_batch,
  * and SYM_ERR_INVALID for reps outside 1..100; the factor afterwards is that of the last run. */
 int sym_autotune(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride, int32_t reps, int32_t *tuned,
                  int32_t *changed);

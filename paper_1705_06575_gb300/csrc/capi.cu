@@ -677,6 +677,7 @@ static int analyze_impl(int64_t n, const int64_t *Ap, const int32_t *Ai, const i
     h->dp.piv = h->d_piv;
     h->dp.oz = h->plan.oz.data();
     for (int c = 0; c < 2; ++c) h->dp.variant[c] = h->plan.variant[c].data();
+    h->dp.tuned_nb = &h->plan.tuned_nb;
     h->dp.batch_warp = h->plan.batch_warp.data();
     h->dp.batch_lanes = h->plan.batch_lanes.data();
     h->dp.batch_panel = (opt.flags & SYM_FLAG_NO_FUSED_LEVELS) ? nullptr : h->plan.batch_panel.data();
@@ -1201,6 +1202,8 @@ int sym_autotune(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride,
   // where its panels fit the fused kernel)
   std::vector<int8_t> &apart = P.panel_apart[nbatch > 1 ? 1 : 0];
   const bool f32 = h->precision != SYM_PREC_FP64;
+  if (nbatch > 1) P.tuned_nb = nbatch;
+  const int8_t untimed = nbatch > 1 ? -1 : 0;
   std::vector<size_t> heads;
   if (h->dp.batch_panel)
     for (size_t li = 0; li < nl; ++li)
@@ -1233,7 +1236,7 @@ int sym_autotune(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride,
   int32_t ntun = 0, nchg = 0;
   std::vector<double> t[2];
   if (!heads.empty()) {
-    std::fill(var.begin(), var.end(), 0);
+    std::fill(var.begin(), var.end(), untimed);
     time_forms([&](int v) { for (size_t hd : heads) apart[hd] = (int8_t)v; }, t);
     for (size_t hd : heads) {  // the level's launches in either form (covered ones take ~0 fused)
       double sum[2] = {0.0, 0.0};
@@ -1256,10 +1259,12 @@ int sym_autotune(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride,
                                                                         h->precision == SYM_PREC_FP64);
   }
   if (nform > 0 && !rc) {
-    time_forms([&](int v) { for (size_t li = 0; li < nl; ++li) var[li] = tunable[li] ? (int8_t)v : 0; }, t);
+    time_forms([&](int v) { for (size_t li = 0; li < nl; ++li) var[li] = tunable[li] ? (int8_t)v : untimed; }, t);
     for (size_t li = 0; li < nl; ++li) {
-      var[li] = tunable[li] && !rc && t[1][li] < t[0][li] ? 1 : 0;
-      nchg += var[li];
+      var[li] = tunable[li] && !rc ? (t[1][li] < t[0][li] ? 1 : 0) : untimed;
+      const bool rule = nbatch > 1 && sym::batch_default_form(P.factor_launches[li], P.batch_lanes[li],
+                                                              P.batch_warp[li] != 0, nbatch, !f32);
+      nchg += var[li] >= 0 && (var[li] != 0) != rule;
     }
   }
   ntun += nform;

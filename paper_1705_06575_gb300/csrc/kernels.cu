@@ -3069,9 +3069,10 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
       const int32_t head = d.batch_panel[li].head;
       const int8_t *apart = d.panel_apart[nb > 1 ? 1 : 0];
       constexpr bool f32 = std::is_same<T, float>::value;
-      const bool sep = !apart             ? false
-                       : apart[head] >= 0 ? apart[head] != 0
-                                          : batch_level_apart(d.batch_panel[head], launches[head].count, nb, f32);
+      const bool sep = !apart    ? false
+                       : nb == 1 ? apart[head] != 0
+                                 : batch_apart(d.batch_panel[head], launches[head].count, nb, f32, apart[head],
+                                               (unsigned)*d.tuned_nb);
       if (sep || panel_lanes_for(d.batch_panel[head], nb, f32) == 0) panel = PANEL_NONE;
     }
     if (panel == PANEL_COVERED) {
@@ -3086,10 +3087,13 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
     }
     cudaError_t e = cudaSuccess;
     const bool small = L.tb == SMALL_TB;  // every tile of the launch fits the small variant
-    // the autotuner's choice for this launch: false keeps the default form of a batch
+    // the launch's form where it has two: one matrix, the autotuner's choice (false: the default); a
+    // batch, by its number of pairs or as timed at that size (batch_form)
+    constexpr bool fp64 = std::is_same<T, double>::value;
     const int8_t *var = d.variant[nb > 1 ? 1 : 0];
-    const bool alt = var && var[li] != 0 &&
-                     factor_launch_has_alternative(L, (int32_t)nb, std::is_same<T, double>::value);
+    const bool alt = var && factor_launch_has_alternative(L, (int32_t)nb, fp64) &&
+                     (nb > 1 ? batch_form(L, d.batch_lanes[li], d.batch_warp[li] != 0, nb, fp64, var[li], *d.tuned_nb)
+                             : var[li] != 0);
     constexpr int TS = TileCfg<SMALL_TB>::threads;
     switch (L.kind) {
       case K_UPDATE:
@@ -3108,23 +3112,20 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         else if (oz && d.oz[li] && !alt)
           e = launch_update_oz(g, d.oz[li], s, prio, d, Lx, L.off, status);
         // a batch's small tiles: lanes = matrices, or a warp per (tile, matrix) where there are few
-        // (the alternative the other way round)
-        else if (small && nb > 1 && d.batch_lanes && d.batch_lanes[li] > 0 &&
-                 ((int64_t)g * nb > BATCH_WARP_UPDATE) != alt)
+        else if (small && nb > 1 && d.batch_lanes[li] > 0 && alt)
           e = launch_update_mb<T>(d.batch_lanes[li], g, nb, s, prio, d, Lx, L.off, bt);
         else if (small && nb > 1)
           e = launch_prio(k_update_wb<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, 0, s, prio,
                           d.sn, d.upd_tasks, d.upd_entries, d.rel, Lx, L.off, (int32_t)nb, bt);
         // a batch's full tiles with small entries: a warp per (tile, matrix) in global memory, or one
-        // CTA per pair where there are few (the alternative the other way round: 64 x 100^2 and 128 x
-        // 64^2 grids at 256 - 7000 pairs; against lanes = matrices the warps are 1.1 - 5 times faster
-        // on every such level of these and of 512 x 128^2)
-        else if (!small && nb > 1 && d.batch_warp && d.batch_warp[li] &&
-                 ((int64_t)g * nb > BATCH_CTA_UPDATE) != alt)
+        // CTA per pair where there are few (64 x 100^2 and 128 x 64^2 grids at 256 - 7000 pairs; against
+        // lanes = matrices the warps are 1.1 - 5 times faster on every such level of these and of
+        // 512 x 128^2)
+        else if (!small && nb > 1 && d.batch_warp[li] && alt)
           e = launch_prio(k_update_wg<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, 0, s, prio,
                           d.sn, d.upd_tasks, d.upd_entries, d.rel, Lx, L.off, (int32_t)nb, bt);
         // (full tiles with large entries: one CTA per pair, alternative lanes = matrices)
-        else if (!small && nb > 1 && d.batch_warp && !d.batch_warp[li] && d.batch_lanes && d.batch_lanes[li] > 0 && alt)
+        else if (!small && nb > 1 && !d.batch_warp[li] && d.batch_lanes[li] > 0 && alt)
           e = launch_update_mb<T>(d.batch_lanes[li], g, nb, s, prio, d, Lx, L.off, bt);
         else if (small)
           e = launch_prio(k_update_flat<T, SMALL_TB, false>, dim3(g, nb), TS, 0, s, prio, d.sn, d.upd_tasks,
@@ -3138,11 +3139,10 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
         break;
       case K_POTRF:
         // small tiles of a large batch: a warp per tile (throughput); otherwise a CTA per tile, whose
-        // four warps shorten each column step of the tile (latency; 64^2 factor 0.96 -> 0.83 ms);
-        // the autotuner's choice (alt) swaps the two
+        // four warps shorten each column step of the tile (latency; 64^2 factor 0.96 -> 0.83 ms)
         if (panel == PANEL_FUSED)
           e = launch_panel_b<T>(d, d.batch_panel[li], g, nb, s, prio, Lx, Linv, status, L.off, bt);
-        else if (small && (nb > 1 && (int64_t)g * nb > BATCH_CTA_POTRF) != alt)
+        else if (small && alt)
           e = launch_prio(k_potrf_w<T>, dim3((g + WT_WARPS - 1) / WT_WARPS, nb), 32 * WT_WARPS, 0, s, prio, d.sn,
                           d.tasks, (int64_t)g, Lx, status, d.piv, d.axc, d.dpos, L.off, bt);
         else if (small)
@@ -3158,8 +3158,8 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
                           d.dpos, L.off, bt);
         break;
       case K_TRSM:
-        // small tiles of a large batch: a warp per (tile, matrix) (the alternative the other way round)
-        if (small && nb > 1 && ((int64_t)g * nb > BATCH_CTA_TRSM) != alt)
+        // small tiles of a large batch: a warp per (tile, matrix)
+        if (small && nb > 1 && alt)
           e = launch_prio(k_trsm_w<T>, dim3(g, (nb + WT_WARPS - 1) / WT_WARPS), 32 * WT_WARPS, trsm_w_smem<T>(), s,
                           prio, d.sn, d.tasks, Lx, L.off, (int32_t)nb, bt);
         else if (small)
@@ -3189,7 +3189,7 @@ cudaError_t run_factor(const DevPlan &d, const std::vector<Launch> &launches, co
           e = launch_prio(k_gemm_f32, dim3(g, nb), F32_THREADS, 0, s, prio, d.sn, d.tasks, Lx, L.off, bt);
         break;
       case K_TRTRI:
-        if (small && (nb > 1 && (int64_t)g * nb > BATCH_CTA_TRTRI) != alt)  // (as for POTRF)
+        if (small && alt)  // (as for POTRF)
           e = launch_prio(k_trtri_w<T>, dim3((g + WT_WARPS - 1) / WT_WARPS, nb), 32 * WT_WARPS, 0, s, prio, d.sn,
                           d.tasks, (int64_t)g, (const T *)Lx, Linv, L.off, bt);
         else

@@ -44,10 +44,11 @@ struct DevPlan {
   const PanelForm *fwd_panel = nullptr;    // HOST arrays (Plan::fwd_panel, bwd_panel): the fused
   const PanelForm *bwd_panel = nullptr;    // narrow solve levels; null: none
   int64_t nfwd_panel = 0, nbwd_panel = 0;  // their lengths (the solve lists' launch counts)
+  const int32_t *tuned_nb = nullptr;  // HOST: Plan::tuned_nb
   const int8_t *variant[2] = {nullptr, nullptr};  // HOST arrays, one entry per factor launch,
-                                     // [0] for one matrix, [1] for batches: 1 runs the launch's
-                                     // alternative kernel form (see factor_launch_has_alternative),
-                                     // as the autotuner chose; null or 0: the default form
+                                     // [0] for one matrix: 1 runs the launch's alternative kernel
+                                     // form (see factor_launch_has_alternative), as the autotuner
+                                     // chose; [1] for batches: see batch_form
   // FP64 factors of one matrix on the tensor cores (oz_update.cu): digits of the factored panels,
   // row scale exponents and fixed-point data of the diagonal tiles (exps, zc: per permuted column;
   // zu: laid out as the diagonal-tile inverses) and the HOST array of launches (Plan::oz). exps is

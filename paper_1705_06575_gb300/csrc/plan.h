@@ -207,6 +207,35 @@ struct Int4 {
   int32_t a, b, c, d;
 };
 
+// The kernel form of a factor launch in a batch of nb matrices: false a CTA per (tile, matrix) pair (small
+// updates: a warp), true a warp per pair (updates: or lanes mapped to matrices, see run_factor). lanes,
+// warp: the launch's Plan::batch_lanes and batch_warp.
+inline bool batch_default_form(const Launch &L, int lanes, bool warp, int64_t nb, bool fp64) {
+  const bool small = L.tb == SMALL_TILE;
+  const int64_t pairs = L.count * nb;
+  switch (L.kind) {
+    case K_UPDATE:
+      if (!fp64) return false;
+      return small ? lanes > 0 && pairs > BATCH_WARP_UPDATE : warp && pairs > BATCH_CTA_UPDATE;
+    case K_POTRF: return small && pairs > BATCH_CTA_POTRF;
+    case K_TRSM: return small && pairs > BATCH_CTA_TRSM;
+    case K_TRTRI: return small && pairs > BATCH_CTA_TRTRI;
+    default: return false;
+  }
+}
+// The same with the form that the autotuner found faster in a batch of tuned_nb matrices (-1: not timed).
+// Which form is faster depends on the number of pairs, so where the rule above changes its answer between
+// the two sizes what was timed says nothing, and the rule holds.
+inline bool batch_form(const Launch &L, int lanes, bool warp, int64_t nb, bool fp64, int stored, int64_t tuned_nb) {
+  const bool rule = batch_default_form(L, lanes, warp, nb, fp64);
+  return stored < 0 || batch_default_form(L, lanes, warp, tuned_nb, fp64) != rule ? rule : stored != 0;
+}
+// Whether a batch runs a narrow level as separate launches, likewise.
+inline bool batch_apart(const PanelForm &pf, int64_t count, unsigned nb, bool f32, int stored, unsigned tuned_nb) {
+  const bool rule = batch_level_apart(pf, count, nb, f32);
+  return stored < 0 || batch_level_apart(pf, count, tuned_nb, f32) != rule ? rule : stored != 0;
+}
+
 struct Plan {
   int64_t n = 0;
   int64_t nnz_a = 0;
@@ -240,8 +269,10 @@ struct Plan {
   std::vector<UpdTask> upd_tasks;
   std::vector<Int4> tasks;            // every other kind of task
   std::vector<Launch> factor_launches;
-  std::vector<int8_t> variant[2];     // per factor launch: the autotuner's kernel form (0 default),
-                                      // [0] for one matrix, [1] for batches
+  std::vector<int8_t> variant[2];     // per factor launch: the autotuner's kernel form, [0] for one
+                                      // matrix (0 default), [1] for batches (see batch_form; -1 not
+                                      // timed)
+  int32_t tuned_nb = 0;               // matrices in the batch that the autotuner timed last
   std::vector<int8_t> batch_warp;     // per factor launch: 1 if a batch's default form of this
                                       // full-tile update is one warp per (tile, matrix)
   std::vector<int8_t> batch_lanes;     // per factor launch: for a small-tile update, a batch's
@@ -250,7 +281,7 @@ struct Plan {
   std::vector<PanelForm> batch_panel;  // per factor launch: fused narrow levels (batches and,
                                        // where panel_apart[0] allows, single matrices)
   std::vector<int8_t> panel_apart[2];  // per factor launch, on PANEL_FUSED ones (-1 for batches:
-                                       // not timed, batch_level_apart decides): 1 if the
+                                       // not timed, see batch_apart): 1 if the
                                        // autotuner found the level faster as separate launches;
                                        // [0] one matrix, [1] batches
   // Per factor launch of one FP64 matrix: nonzero if the launch runs on the tensor cores (K_UPDATE:

@@ -887,7 +887,7 @@ int analyze(int64_t n, const int64_t *Ap, const int32_t *Ai, const int32_t *perm
     mark(P.fwd_launches, P.fwd_panel, S_FSTEP);
     mark(P.bwd_launches, P.bwd_panel, S_BSTEP);
   }
-  for (auto &v : P.variant) v.assign(P.factor_launches.size(), 0);
+  for (int c = 0; c < 2; ++c) P.variant[c].assign(P.factor_launches.size(), (int8_t)-c);
   // Default form of a batch's full-tile FP64 update launches: one warp per (tile, matrix) when
   // the launch's entries are small (at most BATCH_WARP_ELEMS output elements on average: the
   // one-CTA form then spends its time staging and waiting at barriers), else one CTA per tile.
