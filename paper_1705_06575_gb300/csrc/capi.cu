@@ -740,7 +740,20 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
   }
   if (!trp && h->use_graphs) {
     // Replay the captured launch sequence; capture it again when the batch changes. A moved Ax is
-    // patched into the nodes that read it (a capture of the 64^2 grid's 87 launches takes 0.3 ms).
+    // patched into the nodes that read it (a capture of the 64^2 grid's 87 launches takes 0.3 ms); a
+    // graph that does not take it is captured again.
+    if (h->fgraph && h->fgraph_nb == nbatch && h->fgraph_stride == stride && h->fgraph_ax != Ax) {
+      cudaError_t e = cudaSuccess;
+      if (h->fnodes.first) e = sym::patch_address(h->fgraph, h->fnodes.first, sym::SCATTER_ARGS, 0, Ax);
+      if (e == cudaSuccess && h->fnodes.second)
+        e = sym::patch_address(h->fgraph, h->fnodes.second, sym::SCALE_ARGS, 0, Ax);
+      if (e == cudaSuccess) {
+        h->fgraph_ax = Ax;
+      } else {
+        drop_factor_graph(h);
+        cudaGetLastError();
+      }
+    }
     if (!h->fgraph || h->fgraph_nb != nbatch || h->fgraph_stride != stride) {
       rc = ensure_capture_stream(h);
       if (rc) return rc;
@@ -759,16 +772,6 @@ int factor_impl(sym_handle h, int32_t nbatch, const double *Ax, int64_t stride) 
       h->fgraph_ax = Ax;
       h->fgraph_nb = nbatch;
       h->fgraph_stride = stride;
-    } else if (h->fgraph_ax != Ax) {
-      cudaError_t e = cudaSuccess;
-      if (h->fnodes.first) e = sym::patch_address(h->fgraph, h->fnodes.first, sym::SCATTER_ARGS, 0, Ax);
-      if (e == cudaSuccess && h->fnodes.second)
-        e = sym::patch_address(h->fgraph, h->fnodes.second, sym::SCALE_ARGS, 0, Ax);
-      if (e != cudaSuccess) {
-        drop_factor_graph(h);
-        return cuda_fail(e, "factor graph");
-      }
-      h->fgraph_ax = Ax;
     }
     CUDA_TRY(cudaGraphLaunch(h->fgraph, h->stream), "factor graph");
   } else {
@@ -857,9 +860,22 @@ int solve_impl(sym_handle h, int32_t nbatch, int32_t nrhs, const double *B, int6
     trp = &tr;
   }
   if (!trp && h->use_graphs && n > 0 && nrhs > 0) {
-    const bool same = h->sgraph && h->sgraph_key[2] == h->d_y && h->sgraph_ikey[0] == nrhs && h->sgraph_ikey[1] == ldb &&
+    bool same = h->sgraph && h->sgraph_key[2] == h->d_y && h->sgraph_ikey[0] == nrhs && h->sgraph_ikey[1] == ldb &&
                       h->sgraph_ikey[2] == ldx && h->sgraph_nb == nbatch && h->sgraph_bx[0] == bstride &&
                       h->sgraph_bx[1] == xstride;
+    if (same) {  // moved right-hand sides or solutions: patched into the permutations
+      cudaError_t e = cudaSuccess;
+      if (h->sgraph_key[0] != B) e = sym::patch_address(h->sgraph, h->snodes.first, sym::PERM_ARGS, 1, B);
+      if (e == cudaSuccess && h->sgraph_key[1] != X)
+        e = sym::patch_address(h->sgraph, h->snodes.second, sym::PERM_ARGS, 2, X);
+      if (e == cudaSuccess) {
+        h->sgraph_key[0] = B;
+        h->sgraph_key[1] = X;
+      } else {  // captured again
+        same = false;
+        cudaGetLastError();
+      }
+    }
     if (!same) {
       rc = ensure_capture_stream(h);
       if (rc) return rc;
@@ -884,17 +900,6 @@ int solve_impl(sym_handle h, int32_t nbatch, int32_t nrhs, const double *B, int6
       h->sgraph_nb = nbatch;
       h->sgraph_bx[0] = bstride;
       h->sgraph_bx[1] = xstride;
-    } else {  // moved right-hand sides or solutions: patched into the permutations
-      cudaError_t e = cudaSuccess;
-      if (h->sgraph_key[0] != B) e = sym::patch_address(h->sgraph, h->snodes.first, sym::PERM_ARGS, 1, B);
-      if (e == cudaSuccess && h->sgraph_key[1] != X)
-        e = sym::patch_address(h->sgraph, h->snodes.second, sym::PERM_ARGS, 2, X);
-      if (e != cudaSuccess) {
-        drop_solve_graph(h);
-        return cuda_fail(e, "solve graph");
-      }
-      h->sgraph_key[0] = B;
-      h->sgraph_key[1] = X;
     }
     CUDA_TRY(cudaGraphLaunch(h->sgraph, h->stream), "solve graph");
     return SYM_OK;
