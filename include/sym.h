@@ -113,9 +113,10 @@ typedef struct {
   int64_t npairs;           /* (descendant, ancestor) update pairs */
   int64_t nlaunch_factor;   /* kernel launches per sym_factor (one matrix, current forms) */
   int64_t nlaunch_solve;    /* kernel launches per sym_solve (FP64 factors: also per pass of up to
-                               8 right-hand sides of sym_solve_multi; FP32: passes of one or two) */
+                               32 right-hand sides of sym_solve_multi; FP32: passes of one or two) */
   double analyze_seconds;   /* host time of the inspector */
-  int64_t device_bytes;     /* device memory held by the handle */
+  int64_t device_bytes;     /* device memory held by the handle (the first factorization of one FP64
+                               matrix adds to it, see sym_factor) */
   int64_t upd_tasks;        /* tiles receiving descendant updates */
   int64_t upd_entries;      /* (tile, descendant) update entries */
   int64_t dense_tasks;      /* POTRF + TRSM + GEMM + inverse tile tasks */
@@ -188,7 +189,10 @@ int sym_set_stream(sym_handle h, void *stream);
  * before the factorization and all of it runs in FP64. What remains: components of x many orders of
  * magnitude below the others because the matrix is strongly diagonally dominant (the far field of a
  * point source) are then accurate relative to the others, not to themselves. SYM_FLAG_NO_TENSOR_CORES,
- * and a batch, take FP64 always. */
+ * and a batch, take FP64 always. The fixed-point copies take 14 bytes per entry of the supernodes that
+ * update others or have more than 64 columns (1.75 times their panels), allocated by the first
+ * factorization of one matrix; where they cannot be allocated, or that call's stream is being
+ * captured, it runs in FP64. */
 int sym_factor(sym_handle h, const double *Ax);
 
 /* As sym_factor but returns right after enqueueing (no wait, no status check). Call
@@ -424,8 +428,9 @@ int sym_get_factor_host(sym_handle h, double *Lx_host);
  * diagonal block) in this one launch, with pmax the level's largest panel (rows x columns) and
  * ncmax its widest supernode; role 2: that level's TRSM and TRTRI launches, then skipped; role
  * 0: other launches. head: for roles 1 and 2 the index of the level's role-1 launch, else -1.
- * Batches run such a level fused where its panels fit the kernel's shared memory; a single
- * matrix where the level has at least 1216 supernodes; sym_autotune times both ways. */
+ * Batches run such a level fused where its panels fit the kernel's shared memory and the batch
+ * gives the level enough warps; a single matrix where the level has at least 1216 supernodes;
+ * sym_autotune times both ways. */
 #define SYM_EXPORT_BATCH_PANEL 27
 /* The same for the forward and backward solve lists (SYM_EXPORT_FWD_LAUNCHES, _BWD_LAUNCHES):
  * role 1 on the step launch of a level whose supernodes all have at most 32 columns, on which

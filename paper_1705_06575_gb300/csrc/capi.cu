@@ -319,8 +319,15 @@ int ensure_batch(sym_handle_s *h, int32_t nbatch) {
     h->dp.piv = h->d_piv;
   }
   if (!rc) rc = regrow((void **)&h->d_status, sizeof(long long) * (nb + 1), "cudaMalloc(status batch)");
-  const int64_t tmats = std::max<int64_t>(nb, h->dp.tgroups);
-  if (!rc) rc = regrow((void **)&h->d_t, sizeof(double) * sym::SOLVE_MAXRHS * P.tsize * tmats, "cudaMalloc(solve buffer batch)");
+  if (!rc) {  // for the batch, or the groups of right-hand sides that one matrix's solve takes along
+    const size_t tb = sizeof(double) * sym::SOLVE_MAXRHS * P.tsize, groups = (size_t)h->dp.tgroups;
+    rc = regrow((void **)&h->d_t, tb * std::max(nb, groups), "cudaMalloc(solve buffer batch)");
+    if (rc && groups > nb) {  // as many groups as the batch has matrices
+      cudaGetLastError();
+      h->dp.tgroups = (int32_t)nb;
+      rc = regrow((void **)&h->d_t, tb * nb, "cudaMalloc(solve buffer batch)");
+    }
+  }
   h->dp.t = h->d_t;
   if (!rc) {
     if (h->h_status) cudaFreeHost(h->h_status);
@@ -387,10 +394,16 @@ int ensure_stage(sym_handle_s *h, int64_t count) {
 
 // Digits and fixed-point data of one FP64 matrix's factor on the tensor cores, at the first
 // factorization of a single matrix that has tiles of more than SMALL_TILE columns. Without the
-// memory the SIMT kernels run.
+// memory, and while the caller captures the stream (nothing may be allocated then), the SIMT kernels
+// run.
 void ensure_digits(sym_handle_s *h) {
   if (h->dg_tried || h->precision != SYM_PREC_FP64 || !h->dp.tensor_cores || h->plan.max_ncols <= sym::SMALL_TILE)
     return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return;
+  }
   h->dg_tried = true;
   const size_t n = (size_t)h->plan.n;
   const size_t bytes[7] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
