@@ -1065,6 +1065,13 @@ int sym_info(sym_handle h, sym_stats *s) {
       for (const sym::PanelForm &pf : *forms)
         if (pf.role == sym::PANEL_COVERED && sym::solve_lanes_for((*forms)[pf.head], 1, !f32) > 0) --s->nlaunch_solve;
   }
+  // on the tensor cores the scales and the range check (three), and the digits of small tiles
+  if (!h->host_only && h->precision == SYM_PREC_FP64 && h->d_links && (h->d_exps || !h->dg_tried)) {
+    s->nlaunch_factor += 3;
+    for (size_t li = 0; li < P.factor_launches.size(); ++li)
+      s->nlaunch_factor += P.factor_launches[li].kind == sym::K_TRSM && P.factor_launches[li].tb == sym::SMALL_TILE &&
+                           P.oz[li];
+  }
   s->analyze_seconds = P.analyze_seconds;
   s->device_bytes = h->device_bytes;
   s->upd_tasks = (int64_t)P.upd_tasks.size();

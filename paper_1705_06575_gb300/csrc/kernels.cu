@@ -3263,7 +3263,11 @@ cudaError_t launch_solve_b(bool forward, const DevPlan &d, const PanelForm &pf, 
 // 1.89 / 2.42; 48^3, 8 columns (500 M) 3.95 / 4.27 / 5.02 and 32 (2 G) 11.0 / 9.95 / 10.9; 64^3, 4
 // columns (790 M) 6.42 / 6.32, 16 columns 17.9 / 15.4 / 16.9; FP32 with refinement: 31^3, 16 columns
 // (150 M) 2.9 / 3.1 / 3.8 and 32 4.5 / 4.0 / 4.6. (One group of 8 after another: 48^3, 16 columns
-// 10.1 ms against 6.3 now.) A width that does not divide the columns leaves the rest to another pass.
+// 10.1 ms against 6.3 now.) All groups of a pass have one width, so beyond SHARE a count without a
+// divisor near four runs as columns (up to 16, 64^3: 11 columns 13.1 ms, 13 columns 15.0, between 12
+// columns' 12.5 and 16 columns' 15.4) or pairs, or leaves the rest to another pass (29 and 31 columns 27.8
+// and 29.8 ms, 32 columns 27.4). No count of 1 - 37 is slower than in passes of eight (64^3: 11 columns
+// 23.0 ms, 22 44.8, 31 62.1).
 template <typename T>
 int group_width(int64_t storage, int columns) {
   constexpr int64_t SHARE = std::is_same<T, double>::value ? 600000000 : 250000000;

@@ -962,7 +962,7 @@ int analyze(int64_t n, const int64_t *Ap, const int32_t *Ai, const int32_t *perm
       P.oz[li] = (int8_t)cs;
       for (int64_t t = L.off; t < L.off + L.count; ++t)
         for (int64_t e = P.upd_tasks[t].e0; e < P.upd_tasks[t].e1; ++e) keep[P.upd_entries[e].K] = 1;
-    } else if (L.kind == K_GEMM) {
+    } else if (L.kind == K_GEMM) {  // (always: launches of 2 - 72 tasks take 12 - 16 us, SIMT 12 - 45)
       P.oz[li] = 1;
       for (int64_t q = L.off; q < L.off + L.count; ++q) keep[P.tasks[q].a] = 1;
     }
