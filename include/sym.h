@@ -185,10 +185,11 @@ int sym_set_stream(sym_handle h, void *stream);
  * so does the normwise backward error of a solve; but an entry of L far below its row's scale holds
  * fewer significant bits than a double, down to none below 2^-60 of the scale. Where A's own values
  * make that matter (large penalties on diagonal entries, parts of the matrix joined by weak couplings
- * only, diagonals of coupled rows more than 2^14 apart, values that are not finite) the device finds out
- * before the factorization and all of it runs in FP64. What remains: components of x many orders of
- * magnitude below the others because the matrix is strongly diagonally dominant (the far field of a
- * point source) are then accurate relative to the others, not to themselves. SYM_FLAG_NO_TENSOR_CORES,
+ * only, jumps of more than 2^14 between weakly coupled rows, values that are not finite) the device finds
+ * out before the factorization and all of it runs in FP64; a scaling of rows and columns by D A D alone
+ * does not matter. What remains: components of sqrt(a_ii) x_i many orders of magnitude below the others
+ * although nothing weak joins them (the far field of a point source in a strongly diagonally dominant
+ * matrix) are accurate relative to the others, not to themselves. SYM_FLAG_NO_TENSOR_CORES,
  * and a batch, take FP64 always. The fixed-point copies take 14 bytes per entry of the supernodes that
  * update others or have more than 64 columns (1.75 times their panels), allocated by the first
  * factorization of one matrix; where they cannot be allocated, or that call's stream is being

@@ -34,11 +34,13 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
 // other through those. Measured on a 14^3 7-point conductance matrix, largest relative error of a
 // component of x, FP64 kernels | fixed point: penalties of 1e4 on 5% of the diagonal 3e-15 | 3e-15, 1e5
 // 4e-15 | 9e-15, 1e8 5e-15 | 3e-13, 1e16 4e-15 | 3e-9; a plane of couplings scaled by 0.1 5e-15 | 1e-14,
-// 0.01 4e-15 | 5e-14, 1e-6 2e-14 | 6e-10, 1e-12 4e-15 | 8e-4. So *wide gets bit 0, and every kernel of
-// this file then works in FP64, if
+// 0.01 4e-15 | 5e-14, 1e-6 2e-14 | 6e-10, 1e-12 4e-15 | 8e-4; one half's coefficients 1e2 times the other
+// half's, which it drives alone, 5e-15 | 2e-14, 1e4 5e-15 | 2e-13 (in norm 9e-16 | 5e-15). Rows and columns
+// scaled by powers of two up to 2^100 instead: 4e-15 | 2e-15, the row scales absorb them. So *wide gets
+// bit 0, and every kernel of this file then works in FP64, if
 //   * a value is not finite;
-//   * a row's couplings add up to less than 2^-WEAK of its diagonal (a penalty on it);
-//   * two coupled rows' diagonals are more than 2^SPREAD apart;
+//   * a row's couplings |a_ij| / sqrt(a_ii a_jj) add up to less than 2^-LOOSE (a penalty on it);
+//   * a coupling below 2^-WEAK in that measure joins rows whose diagonals are more than 2^SPREAD apart;
 //   * weak couplings are the only links between two parts of the matrix: couplings below 2^-WEAK of the
 //     smaller of the two diagonals and below 2^-FAINT of the strongest couplings of both rows (a long
 //     row's are all far below its diagonal). The others are united into components (lock-free
@@ -48,23 +50,23 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
 // (Exponents are compared, so a limit is exact to a factor of two.) A well-coupled matrix pays two more
 // small launches, beside the scatter (run_factor): 2 of the 64^2 grid's 762 us for factor and solve,
 // nothing that shows on larger ones.
-constexpr int WEAK = 9, FAINT = 6, SPREAD = 14;
+constexpr int WEAK = 9, FAINT = 6, SPREAD = 14, LOOSE = 6;
 constexpr int WIDE = 1, LINKS = 2;  // bits of *wide: FP64; couplings below 2^-WEAK of the diagonals present
 struct OzRow {  // (sum and strongest are zero before the first kernel)
-  unsigned long long sum;  // of the row's couplings, units of 2^-SUM_UNIT of the diagonal's power of two
+  unsigned long long sum;  // of the row's couplings |a_ij| / sqrt(a_ii a_jj), unit 2^-SUM_UNIT
   int strongest;           // exponent + 1 of its strongest coupling, 0: none
   int diagonal;            // exponent
 };
 constexpr int SUM_UNIT = 40;
-constexpr unsigned long long COUPLED = 1ull << (SUM_UNIT - WEAK);  // (no more is added to a sum beyond)
+constexpr unsigned long long COUPLED = 1ull << (SUM_UNIT - LOOSE);  // (no more is added to a sum beyond)
 __device__ __forceinline__ int exponent_of(double a) { return (__double2hiint(a) >> 20) & 0x7ff; }
 
-// x: exponent of a coupling of row r.
-__device__ __forceinline__ void add_coupling(OzRow *r, int x, int diagonal) {
+// x: exponent of a coupling of row r, scaled: of its measure.
+__device__ __forceinline__ void add_coupling(OzRow *r, int x, int scaled) {
   if (*(volatile int *)&r->strongest < x + 1) atomicMax(&r->strongest, x + 1);
   if (*(volatile unsigned long long *)&r->sum < COUPLED) {
-    const int sh = x - diagonal + SUM_UNIT;
-    if (sh >= 0) atomicAdd(&r->sum, sh < SUM_UNIT - WEAK ? 1ull << sh : COUPLED);
+    const int sh = scaled + SUM_UNIT;
+    if (sh >= 0) atomicAdd(&r->sum, sh < SUM_UNIT - LOOSE ? 1ull << sh : COUPLED);
   }
 }
 
@@ -90,9 +92,10 @@ __global__ void k_oz_scale(const double *__restrict__ Ax, const int64_t *__restr
       x = exponent_of(a);
       const int er = exponent_of(Ax[dpos[l.x]]), ec = exponent_of(Ax[dpos[l.y]]);
       if (x + WEAK < min(er, ec)) bits |= LINKS;
-      if (x == 0x7ff || er - ec > SPREAD || ec - er > SPREAD) bits |= WIDE;
-      add_coupling(&rows[l.x], x, er);
-      add_coupling(&rows[l.y], x, ec);
+      const int scaled = x - ((er + ec) >> 1);
+      if (x == 0x7ff || (scaled + WEAK < 0 && (er - ec > SPREAD || ec - er > SPREAD))) bits |= WIDE;
+      add_coupling(&rows[l.x], x, scaled);
+      add_coupling(&rows[l.y], x, scaled);
     }
     strength[k] = (int16_t)(x + 1);
   }

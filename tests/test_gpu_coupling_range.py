@@ -93,6 +93,33 @@ def test_weakly_joined_parts(torch_cuda, maker, power):
     compare(torch_cuda, M, dominant(M, Ax), np.where(side, rng.uniform(0.5, 1.5, M.n), 0.0))
 
 
+@pytest.mark.parametrize("power", [2, 4, 6, 12])
+@pytest.mark.parametrize("maker", sorted(MAKERS))
+def test_coefficient_jumps(torch_cuda, maker, power):
+    """Two halves with coefficients 1 and 10^power, the soft one driven by the stiff one alone."""
+    rng = np.random.default_rng(6)
+    M = MAKERS[maker](rng)
+    side = (np.arange(M.n) % 14 >= 7) if maker == "star14" else rng.integers(0, 2, M.n).astype(bool)
+    c = np.where(side, 10.0 ** power, 1.0)
+    Ax = -np.abs(M.Ax) * np.minimum(c[M.Ai], c[columns(M)])
+    compare(torch_cuda, M, dominant(M, Ax), np.where(side, rng.uniform(0.5, 1.5, M.n) * c, 0.0))
+
+
+def test_scaled_rows_keep_the_tensor_cores(torch_cuda):
+    """D A D of a well-coupled A: with the MMAs withheld the factorization times out (it takes the tensor
+    cores), whatever powers of two D holds."""
+    torch = torch_cuda
+    import paper_1705_06575_gb300 as S
+    M = w.conduct3d(14, np.random.default_rng(3), "star")
+    d = 2.0 ** np.random.default_rng(4).integers(-100, 101, M.n).astype(np.float64)
+    s = S.Solver(M.n, M.Ap, M.Ai, M.perm)
+    S.sym_set_tc_wait(s.h, 20000, 1)
+    with pytest.raises(S.SymError) as e:
+        s.factor(torch.from_numpy(M.Ax * d[M.Ai] * d[columns(M)]).cuda())
+    assert e.value.code == S.SYM_ERR_TIMEOUT
+    s.close()
+
+
 def test_scattered_weak_couplings(torch_cuda):
     """Weak couplings between rows that strong ones join as well, next to explicit zeros: either form
     of the factor is as good, and the check of the couplings ends."""
