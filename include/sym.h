@@ -185,7 +185,7 @@ int sym_set_stream(sym_handle h, void *stream);
  * so does the normwise backward error of a solve; but an entry of L far below its row's scale holds
  * fewer significant bits than a double, down to none below 2^-60 of the scale. Where A's own values
  * make that matter (large penalties on diagonal entries, parts of the matrix joined by weak couplings
- * only, jumps of more than 2^14 between weakly coupled rows, values that are not finite) the device finds
+ * only, jumps of more than 2^16 between weakly coupled rows, values that are not finite) the device finds
  * out before the factorization and all of it runs in FP64; a scaling of rows and columns by D A D alone
  * does not matter. What remains: components of sqrt(a_ii) x_i many orders of magnitude below the others
  * although nothing weak joins them (the far field of a point source in a strongly diagonally dominant

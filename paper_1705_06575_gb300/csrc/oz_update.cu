@@ -40,7 +40,9 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
 // bit 0, and every kernel of this file then works in FP64, if
 //   * a value is not finite;
 //   * a row's couplings |a_ij| / sqrt(a_ii a_jj) add up to less than 2^-LOOSE (a penalty on it);
-//   * a coupling below 2^-WEAK in that measure joins rows whose diagonals are more than 2^SPREAD apart;
+//   * a coupling below 2^-WEAK in that measure joins rows whose diagonals are more than 2^SPREAD apart (the
+//     27-point vector problem's jumps of 1e4 stay: 2^15.2 between an inner row and one at the border,
+//     errors of 3.0e-13 | 2.1e-13);
 //   * weak couplings are the only links between two parts of the matrix: couplings below 2^-WEAK of the
 //     smaller of the two diagonals and below 2^-FAINT of the strongest couplings of both rows (a long
 //     row's are all far below its diagonal). The others are united into components (lock-free
@@ -50,7 +52,7 @@ __device__ __forceinline__ int tile_rows(int32_t i, int32_t ncols, int32_t nrows
 // (Exponents are compared, so a limit is exact to a factor of two.) A well-coupled matrix pays two more
 // small launches, beside the scatter (run_factor): 2 of the 64^2 grid's 762 us for factor and solve,
 // nothing that shows on larger ones.
-constexpr int WEAK = 9, FAINT = 6, SPREAD = 14, LOOSE = 6;
+constexpr int WEAK = 9, FAINT = 6, SPREAD = 16, LOOSE = 6;
 constexpr int WIDE = 1, LINKS = 2;  // bits of *wide: FP64; couplings below 2^-WEAK of the diagonals present
 struct OzRow {  // (sum and strongest are zero before the first kernel)
   unsigned long long sum;  // of the row's couplings |a_ij| / sqrt(a_ii a_jj), unit 2^-SUM_UNIT
@@ -107,11 +109,20 @@ __device__ __forceinline__ bool weak_link(const OzRow *rows, int2 l, int strengt
   return strength - 1 + WEAK < min(r.diagonal, c.diagonal) && strength + FAINT < min(r.strongest, c.strongest);
 }
 
-// The root of v: chains of parents descend in index, and a step moves v two links up.
+// Roots are linked in the order of a scrambled index (a bijection): linked by index, the neighbours k and
+// k + 1 of a grid form chains of n links (14^3 vector problem, scatter and range check: 1.5 ms, 0.2 so).
+__device__ __forceinline__ uint32_t link_order(int32_t v) {
+  uint32_t h = (uint32_t)v * 0x9E3779B1u;
+  h ^= h >> 15;
+  h *= 0x85EBCA77u;
+  return h ^ (h >> 13);
+}
+// The root of v: chains of parents descend in link_order, and a step moves v two links up.
 __device__ __forceinline__ int32_t root_of(volatile int32_t *parent, int32_t v) {
   int32_t p = parent[v];
   while (p != v) {
     const int32_t g = parent[p];
+    if (g == p) return p;
     parent[v] = g;
     v = g;
     p = parent[v];
@@ -120,7 +131,7 @@ __device__ __forceinline__ int32_t root_of(volatile int32_t *parent, int32_t v) 
 }
 
 // Rows against the sum of their couplings; with couplings below 2^-WEAK of the diagonals present, the
-// components of the strong ones (the larger of two roots becomes a child of the smaller one); weak ones get
+// components of the strong ones (the later of two roots becomes a child of the earlier one); weak ones get
 // strength -1.
 __global__ void k_oz_unite(const int2 *__restrict__ links, const OzRow *__restrict__ rows, int32_t *parent,
                            int16_t *__restrict__ strength, int *wide, int64_t n, int64_t nnz) {
@@ -133,7 +144,7 @@ __global__ void k_oz_unite(const int2 *__restrict__ links, const OzRow *__restri
   }
   int32_t a = root_of(parent, links[k].x), b = root_of(parent, links[k].y);
   while (a != b) {
-    if (a < b) {
+    if (link_order(a) < link_order(b)) {
       const int32_t c = a;
       a = b;
       b = c;
