@@ -18,13 +18,13 @@
 // like sqrt(K), as FP64's does with one rounding of 2^-54 of the running value per step. On the diagonal
 // the pair s = t = 4 is a square, 2^-65.6 on average: these are added up apart (dropped_squares). A
 // bias would be invisible in residual norms and for random solutions; in a smooth solution of a nearly
-// singular matrix it adds up over a row. Row sums of L L^T - A of 40^3 7-point grids, mean over the
-// supernodes wider than 512 | standard deviation / sqrt(rows): here -5e-17 | 1e-16; one offset for all
-// columns 2.0e-15 | 1e-16; the FP64 kernels 5e-16 | 4e-16. Errors of x = 1, geometric means over seeds,
-// FP64 kernels | here | no squares, one offset, halves rounded up: 20^3 2.4e-14 | 1.2e-14 | 3.1e-14, 31^3
-// 3.4e-14 | 1.2e-14 | 4.5e-14, 48^3 1.4e-14 | 3.9e-14 | 5.6e-13 (here the solve's own 4e-14, which the FP64
-// kernels' factor happens to cancel), 27-point 28^3 7.4e-14 | 3.6e-14 | 6.8e-13. Random x: 1.3e-14 | 5.0e-15,
-// 9.5e-15 | 7.0e-15, 2.1e-14 | 9.4e-15, 1.2e-13 | 2.5e-14. The accumulators are combined in 64-bit integers
+// singular matrix it adds up over a row. Row sums of L L^T - A of 7-point grids, mean over the supernodes
+// wider than 512 | standard deviation / sqrt(rows): here, 48^3, 1.3e-16 | 7e-17 (the FP64 kernels 0 |
+// 1.8e-16); with one offset for all columns, 40^3, 2.0e-15 | 1e-16. Errors of x = 1, geometric means over
+// seeds, FP64 kernels | here | without the squares, one offset, halves rounded up: 31^3 3.4e-14 | 1.2e-14
+// | 4.5e-14, 40^3 1.0e-14 | 8.3e-15 | 2.3e-13, 48^3 1.4e-14 | 1.6e-14 | 5.6e-13, 27-point 28^3 7.4e-14 |
+// 2.8e-14 | 6.8e-13. Random x: 31^3 9.5e-15 | 7.2e-15, 48^3 2.1e-14 | 1.0e-14, 27-point 28^3 1.2e-13 |
+// 2.7e-14. The accumulators are combined in 64-bit integers
 // (unit 2^-62: the sum is below 2^62 by Cauchy-Schwarz, intermediate wrap-around cancels), whole tiles are
 // summed without any rounding but the last digits' (2^-63 per segment), and the tile is updated with one
 // FP64 rounding per entry.
@@ -69,9 +69,10 @@ constexpr int SEG_STEPS = 16;               // K = 16 steps per segment (256 val
 // Digit 0 is stored as byte 128 in even columns (digits -128 .. 127), as byte 127 in odd ones (-127 ..
 // 128). A column's lower digits average -1/2 or 1/2; where they meet leading digits of one sign (the
 // entries of an M-matrix's factor) in pairs that are dropped, a single offset leaves a bias that grows
-// with K.
-constexpr uint64_t OFFSET = 0x0080808080808080ull, OFFSET_ODD = 0x007F7F7F7F7F7F7Full;
-constexpr uint64_t QMAX = 0x00FFFFFFFFFFFFFFull - OFFSET;
+// with K. Digit 6 has the other offset of its column: of the five dropped pairs of weight 8, each worth 1/4
+// on average if both digits have the same offset, the two with digit 6 then cancel two others.
+constexpr uint64_t OFFSET = 0x008080808080807Full, OFFSET_ODD = 0x007F7F7F7F7F7F80ull;
+constexpr uint64_t QMAX = 0x007F7F7F7F7F7F7Full;
 __device__ __forceinline__ constexpr uint64_t offset_of(int column) { return column & 1 ? OFFSET_ODD : OFFSET; }
 
 // Scale exponent of a row from its diagonal entry a of A: sqrt(a) <= 0.986 * 2^e. Rows whose
@@ -161,9 +162,9 @@ __device__ __forceinline__ void transpose4(uint32_t w0, uint32_t w1, uint32_t w2
 }
 // Two digits (bytes 128 + d, 127 + d) to FP16: the byte under the exponent byte 0x64 is 1024 + 128 + d,
 // exact; minus 1152 (1151).
-__device__ __forceinline__ uint32_t half2_of(uint32_t w, uint32_t sel) {
+__device__ __forceinline__ uint32_t half2_of(uint32_t w, uint32_t sel, uint32_t offsets) {
   uint32_t h = prmt(w, 0x64646464u, sel), r;
-  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x647F6480u));
+  asm("sub.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(offsets));
   return r;
 }
 // The FP16 digits of eight values (fixed-point numbers with their columns' offsets), one slice per
@@ -181,7 +182,8 @@ __device__ __forceinline__ void to_digits(const uint64_t (&q)[8], uint4 (&w)[SL]
     for (int k = 0; k < 3; ++k) b[2 - k] = hi[k];
 #pragma unroll
     for (int s = 0; s < SL; ++s) {
-      const uint32_t x = half2_of(b[s], 0x4140), y = half2_of(b[s], 0x4342);
+      const uint32_t offsets = s == 6 ? 0x6480647Fu : 0x647F6480u;
+      const uint32_t x = half2_of(b[s], 0x4140, offsets), y = half2_of(b[s], 0x4342, offsets);
       if (h == 0) {
         w[s].x = x;
         w[s].y = y;
@@ -268,7 +270,7 @@ __device__ __forceinline__ void drain(uint32_t addr, bool up, unsigned long long
       else if (p == 4) acc[q] += SHORT ? (unsigned long long)((long long)(x * 256 + y) * 256)
                                        : (unsigned long long)((long long)x * (1 << 16)) +
                                              (unsigned long long)((long long)y * 256);
-      else acc[q] += (unsigned long long)(long long)(x + ((y + 128) >> 8));
+      else acc[q] += (unsigned long long)(long long)(x + ((y + 127 + (y >> 8 & 1)) >> 8));  // (halves to even)
     }
   }
 }
