@@ -34,14 +34,10 @@ struct sym_handle_s {
   long long *d_status = nullptr;
   long long *h_status = nullptr;
   double *d_y = nullptr;          // solve work array
-  uint4 *d_dg = nullptr;          // digits of the FP64 panels (one matrix, tensor cores)
-  int32_t *d_exps = nullptr;      // their row scale exponents
-  int2 *d_zu = nullptr;           // fixed-point data of their diagonal tiles
-  void *d_zc = nullptr;
-  int2 *d_links = nullptr;        // A's entries as permuted (row, column), and the work arrays of the
-  void *d_ozrows = nullptr;       // check whether a matrix's values allow fixed point
-  int32_t *d_parent = nullptr;
-  int16_t *d_strength = nullptr;
+  // FP64 on the tensor cores (one matrix): digits, scales, fixed-point tiles and the arrays of the range
+  // check (see ensure_digits); A's entries as permuted (row, column).
+  unsigned char *d_oz = nullptr;
+  int2 *d_links = nullptr;
   bool dg_tried = false;
   void *d_cptr = nullptr, *d_contrib = nullptr;  // contribution lists of the forward solve
   double *d_t = nullptr;          // forward-solve buffer (SOLVE_MAXRHS x tsize per matrix or group of right-hand sides)
@@ -190,8 +186,7 @@ void release_device(sym_handle_s *h) {
   if (h->aux_stream) cudaStreamDestroy(h->aux_stream);
   {
     void *mp[] = {h->d_Linv, h->d_Lfinv, h->d_Lf, h->d_Axc, h->d_anorm, h->d_anorm_work, h->d_csr_p, h->d_csr_i,
-                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_dg, h->d_exps, h->d_zu, h->d_zc,
-                  h->d_links, h->d_ozrows, h->d_parent, h->d_strength};
+                  h->d_csr_map, h->d_rwork, h->d_piv, h->d_dpos, h->d_pivinfo, h->d_oz, h->d_links};
     for (void *p : mp)
       if (p) cudaFree(p);
     if (h->h_eta) cudaFreeHost(h->h_eta);
@@ -406,30 +401,30 @@ void ensure_digits(sym_handle_s *h) {
   }
   h->dg_tried = true;
   const size_t n = (size_t)h->plan.n;
+  // (one allocation: each takes tens of microseconds of the first call)
   const size_t bytes[7] = {sizeof(uint4) * (size_t)h->plan.dg_size, sizeof(int32_t) * n,
                            sizeof(int2) * (size_t)h->plan.dinv_storage, sym::oz_column_bytes() * n,
                            sym::oz_row_bytes() * n, sizeof(int32_t) * n, sizeof(int16_t) * (size_t)h->plan.nnz_a};
-  void **const ptr[7] = {(void **)&h->d_dg, (void **)&h->d_exps, (void **)&h->d_zu, &h->d_zc,
-                         &h->d_ozrows, (void **)&h->d_parent, (void **)&h->d_strength};
-  bool ok = true;
-  for (int i = 0; i < 7 && ok; ++i) ok = cudaMalloc(ptr[i], bytes[i] > 0 ? bytes[i] : 16) == cudaSuccess;
-  ok = ok && cudaMemsetAsync(h->d_ozrows, 0, sym::oz_row_bytes() * n, h->stream) == cudaSuccess;
-  if (ok) {
-    for (size_t b : bytes) h->device_bytes += (int64_t)b;
-  } else {
-    cudaGetLastError();
-    for (void **p : ptr) {
-      if (*p) cudaFree(*p);
-      *p = nullptr;
-    }
+  size_t at[7], total = 0;
+  for (int i = 0; i < 7; ++i) {
+    at[i] = total;
+    total += (bytes[i] + 255) / 256 * 256;
   }
-  h->dp.dg = h->d_dg;
-  h->dp.exps = h->d_exps;
-  h->dp.zu = h->d_zu;
-  h->dp.zc = h->d_zc;
-  h->dp.oz_rows = h->d_ozrows;
-  h->dp.parent = h->d_parent;
-  h->dp.strength = h->d_strength;
+  if (cudaMalloc(&h->d_oz, total) != cudaSuccess ||
+      cudaMemsetAsync(h->d_oz + at[4], 0, bytes[4], h->stream) != cudaSuccess) {
+    cudaGetLastError();
+    if (h->d_oz) cudaFree(h->d_oz);
+    h->d_oz = nullptr;
+    return;
+  }
+  h->device_bytes += (int64_t)total;
+  h->dp.dg = (uint4 *)(h->d_oz + at[0]);
+  h->dp.exps = (int32_t *)(h->d_oz + at[1]);
+  h->dp.zu = (int2 *)(h->d_oz + at[2]);
+  h->dp.zc = h->d_oz + at[3];
+  h->dp.oz_rows = h->d_oz + at[4];
+  h->dp.parent = (int32_t *)(h->d_oz + at[5]);
+  h->dp.strength = (int16_t *)(h->d_oz + at[6]);
 }
 
 int check_device(sym_handle_s *h) {
@@ -1066,7 +1061,7 @@ int sym_info(sym_handle h, sym_stats *s) {
         if (pf.role == sym::PANEL_COVERED && sym::solve_lanes_for((*forms)[pf.head], 1, !f32) > 0) --s->nlaunch_solve;
   }
   // on the tensor cores the scales and the range check (three), and the digits of small tiles
-  if (!h->host_only && h->precision == SYM_PREC_FP64 && h->d_links && (h->d_exps || !h->dg_tried)) {
+  if (!h->host_only && h->precision == SYM_PREC_FP64 && h->d_links && (h->d_oz || !h->dg_tried)) {
     s->nlaunch_factor += 3;
     for (size_t li = 0; li < P.factor_launches.size(); ++li)
       s->nlaunch_factor += P.factor_launches[li].kind == sym::K_TRSM && P.factor_launches[li].tb == sym::SMALL_TILE &&

@@ -663,7 +663,8 @@ __global__ void __launch_bounds__(TileCfg<TB>::threads) k_trsm(const SNode *__re
 // it takes 64 cycles, conversions too, whatever the number of active lanes (30 us per 64-column tile,
 // 34 us with one barrier per column, 25 us with integers). So the diagonals are held as 64-bit integers (FIX): unit 2^(E-60)
 // for a diagonal in [2^E, 2^(E+1)), where the square of an FP32 number is exact before one shift and
-// the error per column, 2^-60 of the diagonal, is below that of an FP64 subtraction. A tile with a
+// the error per column, at most 2^-60 of the diagonal (the shift drops bits, so a pivot errs upwards, by
+// at most 2^-54 over 64 columns), is below that of an FP64 subtraction. A tile with a
 // diagonal that is not positive and finite, or whose E is outside [-60, 100], takes FP64 throughout.
 constexpr int PR_THREADS = 256, PR_LD = NB + 4;
 
