@@ -166,9 +166,9 @@ int sym_analyze_rules(int64_t n, const int64_t *Ap, const int32_t *Ai, const int
 int sym_set_stream(sym_handle h, void *stream);
 
 /* Launching. sym_factor* and sym_solve_multi capture their launch sequence in a CUDA graph on
- * first use (on a private stream) and replay it on the handle's stream while the device
- * pointers and sizes stay the same (a change re-captures). SYM_FLAG_NO_GRAPHS, or profiling,
- * launches kernel by kernel. */
+ * first use (on a private stream) and replay it on the handle's stream while the sizes stay the
+ * same (a change re-captures; moved device pointers are put into the captured graph).
+ * SYM_FLAG_NO_GRAPHS, or profiling, launches kernel by kernel. */
 
 /* Numeric factorization (Sec. 3.2: supernodal left-looking Cholesky; VS-Block turns each
  * supernode into a dense POTRF of its diagonal block and TRSMs of the rows below, and VI-Prune
@@ -178,8 +178,9 @@ int sym_set_stream(sym_handle h, void *stream);
  * then waits for them and reads the pivot status. Returns SYM_ERR_NOT_SPD when a pivot is not
  * positive (or is NaN); sym_last_error_column then gives the first failing column in the
  * caller's numbering and the factor is not usable. Returns SYM_ERR_TIMEOUT (factor not usable)
- * when a tensor-core update of SYM_PREC_MIXED waited about a second for its MMAs in vain. */
-/* Arithmetic of SYM_PREC_FP64 for one matrix: tiles of more than 32 columns are factored and multiplied
+ * when a tensor-core kernel waited about a second for its MMAs in vain.
+ *
+ * Arithmetic of SYM_PREC_FP64 for one matrix: tiles of more than 32 columns are factored and multiplied
  * in fixed point (60 and 56 bits, exact sums) with one scale per row, the power of two at or above
  * sqrt(a_ii). |A - L L^T|_ij then stays within c sqrt(a_ii a_jj) as in FP64, with c no larger, and
  * so does the normwise backward error of a solve; but an entry of L far below its row's scale holds
@@ -314,7 +315,7 @@ int sym_pivot_info(sym_handle h, int32_t index, double *min_ratio, int64_t *colu
 /* The breakdown threshold of sym_pivot_info (0 <= threshold <= 1). */
 int sym_set_pivot_threshold(sym_handle h, double threshold);
 
-/* Bounded waits of the tensor-core update (SYM_PREC_MIXED; no counterpart in the paper). Each
+/* Bounded waits of the tensor-core kernels (both precisions; no counterpart in the paper). Each
  * wait of a CTA on its MMAs gives up after limit_ns nanoseconds (1e3 .. 1e10; default 1e9); the
  * kernel then waits (with the same limit) for anything it still has in flight, frees its tensor
  * memory and records the failure, and the factorization returns SYM_ERR_TIMEOUT with the handle
